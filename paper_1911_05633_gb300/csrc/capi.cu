@@ -21,6 +21,7 @@
 #include "oz.h"
 #include "ktimer.h"
 #include "dyson.h"
+#include "gj.h"
 
 struct gw_plan_s {
   gw::HostPlan h;
@@ -59,8 +60,7 @@ struct gw_plan_s {
   size_t ws_cap = 0;            // cap on the W-solve scratch
   // scratch left for the first call that needs it (gw_options.defer_scratch)
   bool w_pending = false, oz_pending = false, ozp_pending = false;
-  size_t smem_P = 0, smem_S = 0, smem_T = 0, smem_GJ = 0;
-  bool gj_blocked = false;
+  size_t smem_P = 0, smem_S = 0, smem_T = 0;
   // tensor-core inverse (FP32 Gauss-Jordan + sliced FP64-accurate residual)
   bool w_tensor = false;
   size_t smem_GJ32 = 0;
@@ -275,13 +275,7 @@ gw_status launch_scatter(gw_plan_s* p, gw_block kind, int n_slices, const double
 
 // Batched in-place inverse of `batch` dense N x N matrices (perm and status from the plan).
 gw_status launch_gj(gw_plan_s* p, double2* mats, int batch, long long N, cudaStream_t st) {
-  if (p->gj_blocked) {
-    gw::TimedLaunch tl_("k_gj_inverse_blocked", st);
-    gw::k_gj_inverse_blocked<<<batch, 512, p->smem_GJ, st>>>(mats, p->d_perm, (int)N, N * N, p->d_status);
-  } else {
-    gw::TimedLaunch tl_("k_gj_inverse", st);
-    gw::k_gj_inverse<<<batch, 512, p->smem_GJ, st>>>(mats, p->d_perm, (int)N, N * N, p->d_status);
-  }
+  gw::gj_batch(mats, p->d_perm, batch, (int)N, N * N, p->d_status, st);
   return check_launch("k_gj_inverse");
 }
 
@@ -571,17 +565,14 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
   p->smem_P = smem_polar(h);
   p->smem_S = smem_sigma(h);
   p->smem_T = (size_t)std::max(std::max(h.n_tau, h.n_omega), h.n_nu) * 32 * sizeof(double2);
-  // Gauss-Jordan form: blocked (panel in shared memory) when the panel fits, else unblocked
-  p->gj_blocked = npb >= 64 && (2 * npb * gw::kGJB + npb) * sizeof(double2) <= 220 * 1024;
-  p->smem_GJ = p->gj_blocked ? (2 * npb * gw::kGJB + npb) * sizeof(double2) : 2 * npb * sizeof(double2);
-  if (p->smem_GJ > 227 * 1024) {
+  if (2 * npb * sizeof(double2) > 227 * 1024) {
     set_last_error("product basis too large for the single-block Gauss-Jordan solve");
     return fail(GW_ERR_UNSUPPORTED);
   }
   if (gw::raise_smem_limit(gw::k_polarizability_fp64, (int)p->smem_P) != cudaSuccess ||
       gw::raise_smem_limit(gw::k_self_energy_fp64, (int)p->smem_S) != cudaSuccess ||
       gw::raise_smem_limit(gw::k_transform, (int)p->smem_T) != cudaSuccess ||
-      gw::raise_smem_limit(p->gj_blocked ? gw::k_gj_inverse_blocked : gw::k_gj_inverse, (int)p->smem_GJ) != cudaSuccess) {
+      gw::gj_setup((int)npb) != cudaSuccess) {
     cudaError_t e = cudaGetLastError();
     set_last_error(std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
     return fail(GW_ERR_UNSUPPORTED);
@@ -1126,8 +1117,8 @@ gw_status gw_chemical_potential(gw_plan_t p, const void* H_k, const void* Sigx_k
   const double2* Sx = (const double2*)Sigx_k;
   const double2* Tlast = p->d_Tf_inv + (size_t)(h.n_tau - 1) * h.n_omega;  // the row of tau = beta-
   std::vector<double> part(h.n_k);
-  // N(mu) = s (1/N_k) sum_k Re Tr[-G(k, beta-)], one Dyson solve per evaluation
-  auto count = [&](double mu, double* n) -> gw_status {
+  // N(mu) = s (1/N_k) sum_k Re Tr[-G(k, beta-)] from a whole Dyson solve
+  auto solve_count = [&](double mu, double* n) -> gw_status {
     gw_status e = gw::dyson_solve(p->dyson, h, H, Sx, (const double2*)Sig_k_iw, mu, p->d_status, s);
     if (e == GW_OK) e = gw::dyson_density(p->dyson, h, H, Sx, mu, Tlast, s);
     if (e != GW_OK) return e;
@@ -1146,6 +1137,21 @@ gw_status gw_chemical_potential(gw_plan_t p, const void* H_k, const void* Sigx_k
     for (double v : part) t += v;
     *n = h.spin * t / h.n_k;
     return GW_OK;
+  };
+  // The same from the Hessenberg forms, reduced once; a mu at which one of the matrices is
+  // singular to rounding goes to the solve, whose pivots decide, and the forms (in the same
+  // buffer) are made again.
+  bool reduced = false;
+  auto count = [&](double mu, double* n) -> gw_status {
+    if (h.n_orb_total() > gw::kHessMaxN) return solve_count(mu, n);
+    gw_status e = GW_OK;
+    if (!reduced) e = gw::dyson_search_begin(p->dyson, h, H, Sx, (const double2*)Sig_k_iw, s);
+    if (e != GW_OK) return e;
+    reduced = true;
+    bool weak = false;
+    if ((e = gw::dyson_search_count(p->dyson, h, mu, Tlast, n, &weak, s)) != GW_OK || !weak) return e;
+    reduced = false;
+    return solve_count(mu, n);
   };
   double lo = mu_lo, hi = mu_hi, n = 0.0;
   for (int it = 0; it < 200 && hi - lo > tol; ++it) {
@@ -1333,8 +1339,7 @@ extern "C" gw_status gw_screened_W_iw_noalloc(gw_plan_t p, const void* P_R_iw, c
     dim3 gc((unsigned)std::min<long long>((NN + 255) / 256, 1024), 1);
     gw::k_copy_mats<<<gc, 256, 0, s>>>(v, p->d_qh + qi, vinv, NN);
     if ((st = check_launch("k_copy_mats")) != GW_OK) return st;
-    if (p->gj_blocked) gw::k_gj_inverse_blocked<<<1, 512, p->smem_GJ, s>>>(vinv, perm, (int)N, NN, p->d_status);
-    else gw::k_gj_inverse<<<1, 512, p->smem_GJ, s>>>(vinv, perm, (int)N, NN, p->d_status);
+    gw::gj_batch(vinv, perm, 1, (int)N, NN, p->d_status, s);
     if ((st = check_launch("k_gj_inverse")) != GW_OK) return st;
     for (int c0 = 0; c0 < n_work; c0 += n_slots) {
       const int nc = std::min(n_slots, n_work - c0);
@@ -1342,8 +1347,7 @@ extern "C" gw_status gw_screened_W_iw_noalloc(gw_plan_t p, const void* P_R_iw, c
       if ((st = launch_scatter(p, GW_BLOCK_PB, nc, (const double2*)P_R_iw, h.n_nu, slot0, slots, NN, NN, s,
                                p->d_qh + qi, 1, vinv, -1.0)) != GW_OK)
         return st;
-      if (p->gj_blocked) gw::k_gj_inverse_blocked<<<nc, 512, p->smem_GJ, s>>>(slots, perm, (int)N, NN, p->d_status);
-      else gw::k_gj_inverse<<<nc, 512, p->smem_GJ, s>>>(slots, perm, (int)N, NN, p->d_status);
+      gw::gj_batch(slots, perm, nc, (int)N, NN, p->d_status, s);
       if ((st = check_launch("k_gj_inverse")) != GW_OK) return st;
       dim3 gg((unsigned)p->n_active, (unsigned)nc, (unsigned)((maxblk + 127) / 128));
       k_gather_one_q<<<gg, 128, 0, s>>>(p->d_ent, p->d_pair_first, p->d_pb_off, p->d_phase, h.n_k, qh[qi], qw[qi], slots, NN, v,

@@ -19,6 +19,12 @@ struct DysonPlan {
   double* tau = nullptr;   // [n_tau]
   double* part = nullptr;  // [n_k] per-k traces for the particle number
   double2* ainv = nullptr;  // [n_k][N][N] scratch of the quasiparticle energies
+  // the particle-number search: traces of G(k, i w_n), matrix scales, tr (H + Sigma_x) per k,
+  // and {N(mu), flag, device flag}
+  double2* tr = nullptr;
+  double* scale = nullptr;
+  double2* m1 = nullptr;
+  double* count = nullptr;
   void* cont = nullptr;      // small tables of the continued fraction
   size_t cont_bytes = 0;
   void* spec = nullptr;      // matrices, pivots and frequencies of the spectral function
@@ -37,6 +43,17 @@ gw_status dyson_to_tau(DysonPlan& d, const HostPlan& h, const double2* H, const 
 // d.part[k] = Re Tr[-G(k, beta-)] from d.M; Tlast: the last row of the inverse transform.
 gw_status dyson_density(DysonPlan& d, const HostPlan& h, const double2* H, const double2* Sigx, double mu,
                         const double2* Tlast, cudaStream_t st);
+
+// The search for mu evaluates N(mu) many times on the same H and Sigma: dyson_search_begin
+// leaves the Hessenberg forms of M(k, n) = i w_n - H - Sigma_x - Sigma_c in d.M, and each
+// dyson_search_count takes N(mu) from tr (mu + M)^{-1}, O(N^2) per matrix (synchronous on
+// st).  *weak: some mu + M is singular to the trace's rounding.  N <= kHessMaxN.
+// 64 k x 48 frequencies of order 72, 43 evaluations: before, one inverse per evaluation,
+// 17 ms each.
+gw_status dyson_search_begin(DysonPlan& d, const HostPlan& h, const double2* H, const double2* Sigx,
+                             const double2* Sigc, cudaStream_t st);
+gw_status dyson_search_count(DysonPlan& d, const HostPlan& h, double mu, const double2* Tlast, double* n, bool* weak,
+                             cudaStream_t st);
 
 // Linearised quasiparticle energies E [n_k][N] ascending (kernels_qp.cu): Sigma_c from
 // the sampled frequencies n = 0 and n = 1; ainv_scratch: [n_k][N][N] complex.  N <= kQpMaxN.

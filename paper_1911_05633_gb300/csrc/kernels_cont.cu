@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "dyson.h"
+#include "gj.h"
 #include "kernels.h"
 #include "ktimer.h"
 
@@ -130,10 +131,7 @@ gw_status spectral_function(DysonPlan& d, const HostPlan& h, const double2* H, c
     TimedLaunch tl_("k_retarded_build", st);
     k_retarded_build<<<(unsigned)nb, 256, 0, st>>>(H, Sigx, Sigc_w, d_wr, delta, mu, N, n_real, M);
   }
-  {
-    TimedLaunch tl_("k_gj_inverse", st);
-    k_gj_inverse<<<(unsigned)nb, 512, 2 * (size_t)N * sizeof(double2), st>>>(M, perm, N, NN, d_status);
-  }
+  gj_batch(M, perm, (int)nb, N, NN, d_status, st);
   {
     TimedLaunch tl_("k_trace_spectral", st);
     k_trace_spectral<<<(unsigned)((nb + 7) / 8), 256, 0, st>>>(M, N, nb, A);

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "dyson.h"
+#include "gj.h"
 #include "kernels.h"
 #include "ktimer.h"
 #include "smem_limit.h"
@@ -122,6 +123,55 @@ __global__ void __launch_bounds__(256) k_density_trace(const double2* __restrict
   }
 }
 
+// m1[k] = tr (H(k) + Sigma_x(k)).  One warp per k.
+__global__ void __launch_bounds__(32) k_trace_m1(const double2* __restrict__ H, const double2* __restrict__ Sx, int N,
+                                                 double2* __restrict__ m1) {
+  const long long k = blockIdx.x, NN = (long long)N * N;
+  double2 a = make_double2(0.0, 0.0);
+  for (int i = threadIdx.x; i < N; i += 32) {
+    const double2 m = tail_m1(H, Sx, k, NN, (long long)i * (N + 1), true, 0.0);
+    a.x += m.x;
+    a.y += m.y;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+    a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+  }
+  if (threadIdx.x == 0) m1[k] = a;
+}
+
+// out[0] = (s / N_k) sum_k Re Tr[-G(k, beta-)] from the traces tr[k n_w + n] of G(k, i w_n)
+// (the sum that k_density_trace takes element by element), out[1] = *flag, which is
+// cleared.  One block: n_k n_w terms of a few FP64 operations.
+__global__ void __launch_bounds__(512) k_density_of_traces(const double2* __restrict__ tr,
+                                                           const double2* __restrict__ m1,
+                                                           const double* __restrict__ w,
+                                                           const double2* __restrict__ Tlast, double beta, double mu,
+                                                           int N, int n_w, int n_k, double spin, int* flag,
+                                                           double* __restrict__ out) {
+  __shared__ double red[16];
+  double acc = 0.0;
+  for (int b = threadIdx.x; b < n_k * n_w; b += blockDim.x) {
+    const int k = b / n_w, n = b - k * n_w;
+    const double iw = 1.0 / w[n], iw2 = iw * iw;
+    const double2 g = tr[b], m = m1[k], t = Tlast[n];
+    const double rx = fma(fma(-mu, (double)N, m.x), iw2, g.x), ry = fma(m.y, iw2, g.y) + N * iw;
+    acc += t.x * rx - t.y * ry;
+  }
+  for (int k = threadIdx.x; k < n_k; k += blockDim.x)
+    acc += fma(fma(-mu, (double)N, m1[k].x), 0.25 * beta, -0.5 * N);
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int i = 0; i < 16; ++i) s += red[i];
+    out[0] = -spin * s / n_k;
+    out[1] = (double)*flag;
+    *flag = 0;
+  }
+}
+
 gw_status launch_ok(const char* what) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -152,7 +202,11 @@ gw_status dyson_init(DysonPlan& d, const HostPlan& h) {
                     up((void**)&d.w, w.data(), w.size() * sizeof(double)) &&
                     up((void**)&d.tau, h.tau.data(), h.tau.size() * sizeof(double)) &&
                     up((void**)&d.part, nullptr, (size_t)d.n_k * sizeof(double)) &&
-                    up((void**)&d.ainv, nullptr, (size_t)d.n_k * d.N * d.N * sizeof(double2));
+                    up((void**)&d.ainv, nullptr, (size_t)d.n_k * d.N * d.N * sizeof(double2)) &&
+                    up((void**)&d.tr, nullptr, nb * sizeof(double2)) &&
+                    up((void**)&d.scale, nullptr, nb * sizeof(double)) &&
+                    up((void**)&d.m1, nullptr, (size_t)d.n_k * sizeof(double2)) &&
+                    up((void**)&d.count, nullptr, 4 * sizeof(double));
   if (!good) {
     dyson_free(d);
     set_last_error("Dyson scratch allocation failed");
@@ -162,6 +216,12 @@ gw_status dyson_init(DysonPlan& d, const HostPlan& h) {
       raise_smem_limit(k_green_tau, (int)((size_t)d.n_w * 64 * sizeof(double2))) != cudaSuccess) {
     dyson_free(d);
     set_last_error("Dyson transform: too many fermionic frequencies for shared memory");
+    return GW_ERR_UNSUPPORTED;
+  }
+  if (gj_setup(d.N) != cudaSuccess || (d.N <= kHessMaxN && hess_setup(d.N) != cudaSuccess) ||
+      cudaMemset(d.count, 0, 4 * sizeof(double)) != cudaSuccess) {
+    dyson_free(d);
+    set_last_error("Dyson solve: shared-memory opt-in");
     return GW_ERR_UNSUPPORTED;
   }
   if (uploads_landed() != cudaSuccess) {
@@ -174,7 +234,7 @@ gw_status dyson_init(DysonPlan& d, const HostPlan& h) {
 }
 
 void dyson_free(DysonPlan& d) {
-  void* ptrs[] = {d.M, d.perm, d.w, d.tau, d.part, d.ainv, d.cont, d.spec};
+  void* ptrs[] = {d.M, d.perm, d.w, d.tau, d.part, d.ainv, d.tr, d.scale, d.m1, d.count, d.cont, d.spec};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   d = DysonPlan{};
@@ -190,11 +250,7 @@ gw_status dyson_solve(DysonPlan& d, const HostPlan& h, const double2* H, const d
   }
   gw_status s = launch_ok("k_dyson_build");
   if (s != GW_OK) return s;
-  {
-    TimedLaunch tl_("k_gj_inverse", st);
-    k_gj_inverse<<<nb, 512, 2 * (size_t)d.N * sizeof(double2), st>>>(d.M, d.perm, d.N, (long long)d.N * d.N,
-                                                                       d_status);
-  }
+  gj_batch(d.M, d.perm, nb, d.N, (long long)d.N * d.N, d_status, st);
   return launch_ok("k_gj_inverse");
 }
 
@@ -217,6 +273,39 @@ gw_status dyson_density(DysonPlan& d, const HostPlan& h, const double2* H, const
     k_density_trace<<<d.n_k, 256, 0, st>>>(d.M, H, Sigx, d.w, Tlast, h.beta, mu, d.N, d.n_w, d.part);
   }
   return launch_ok("k_density_trace");
+}
+
+gw_status dyson_search_begin(DysonPlan& d, const HostPlan& h, const double2* H, const double2* Sigx,
+                             const double2* Sigc, cudaStream_t st) {
+  const long long nb = (long long)h.n_k * d.n_w;
+  hess_reduce(H, Sigx, Sigc, d.w, d.N, d.n_w, nb, d.M, d.scale, st);
+  {
+    TimedLaunch tl_("k_trace_m1", st);
+    k_trace_m1<<<d.n_k, 32, 0, st>>>(H, Sigx, d.N, d.m1);
+  }
+  return launch_ok("k_hessenberg");
+}
+
+gw_status dyson_search_count(DysonPlan& d, const HostPlan& h, double mu, const double2* Tlast, double* n, bool* weak,
+                             cudaStream_t st) {
+  hess_trace(d.M, d.scale, mu, d.N, (long long)h.n_k * d.n_w, d.tr, reinterpret_cast<int*>(d.count + 2), st);
+  {
+    TimedLaunch tl_("k_density_of_traces", st);
+    k_density_of_traces<<<1, 512, 0, st>>>(d.tr, d.m1, d.w, Tlast, h.beta, mu, d.N, d.n_w, d.n_k, h.spin,
+                                           reinterpret_cast<int*>(d.count + 2), d.count);
+  }
+  gw_status s = launch_ok("k_hess_trace");
+  if (s != GW_OK) return s;
+  double got[2];
+  cudaError_t e = cudaMemcpyAsync(got, d.count, sizeof(got), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    set_last_error(std::string("particle number: ") + cudaGetErrorString(e));
+    return GW_ERR_CUDA;
+  }
+  *n = got[0];
+  *weak = got[1] != 0.0;
+  return GW_OK;
 }
 
 }  // namespace gw
