@@ -396,8 +396,9 @@ gw_status gw_chemical_potential(gw_plan_t plan, const void* H_k, const void* Sig
  * Hermitian parts (h) and A = (I - S1^h)^{1/2}, E(k) are the eigenvalues of
  * A^{-1} (H(k) + Sigma_x^h(k) + S0^h - mu) A^{-1}, plus mu, in ascending order.
  * H_k, Sigx_k, Sig_k_iw as for gw_dyson_green_tau (Sigx_k, Sig_k_iw may be NULL);
- * E_k: device double [N_k][N].  FP64 throughout (Hermitian eigenproblems by cyclic
- * Jacobi, one block per momentum).  GW_ERR_ARG if the sampled set lacks n = 0 or 1,
+ * E_k: device double [N_k][N].  FP64 throughout (as the generalised
+ * Hermitian problem with the metric I - S1^h, one block per momentum; NaN where that
+ * metric is not positive definite).  GW_ERR_ARG if the sampled set lacks n = 0 or 1,
  * GW_ERR_UNSUPPORTED for more than 80 orbitals in total. */
 gw_status gw_qp_energies(gw_plan_t plan, const void* H_k, const void* Sigx_k, const void* Sig_k_iw, double mu,
                          void* E_k, void* stream);

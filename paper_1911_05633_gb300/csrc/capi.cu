@@ -1176,7 +1176,7 @@ gw_status gw_qp_energies(gw_plan_t p, const void* H_k, const void* Sigx_k, const
   gw::ActiveTimer at_(&p->timer);
   if ((st = gw::dyson_init(p->dyson, p->h)) != GW_OK) return st;
   return gw::qp_energies(p->h, (const double2*)H_k, (const double2*)Sigx_k, (const double2*)Sig_k_iw, mu,
-                         p->dyson.ainv, (double*)E_k, S(stream));
+                         (double*)E_k, S(stream));
 }
 
 gw_status gw_continue_sigma(gw_plan_t p, const void* Sig_k_iw, int n_real, const double* w_real, double delta,

@@ -18,7 +18,6 @@ struct DysonPlan {
   double* w = nullptr;     // [n_w] w_n = (2n + 1) pi / beta
   double* tau = nullptr;   // [n_tau]
   double* part = nullptr;  // [n_k] per-k traces for the particle number
-  double2* ainv = nullptr;  // [n_k][N][N] scratch of the quasiparticle energies
   // the particle-number search: traces of G(k, i w_n), matrix scales, tr (H + Sigma_x) per k,
   // and {N(mu), flag, device flag}
   double2* tr = nullptr;
@@ -56,10 +55,10 @@ gw_status dyson_search_count(DysonPlan& d, const HostPlan& h, double mu, const d
                              cudaStream_t st);
 
 // Linearised quasiparticle energies E [n_k][N] ascending (kernels_qp.cu): Sigma_c from
-// the sampled frequencies n = 0 and n = 1; ainv_scratch: [n_k][N][N] complex.  N <= kQpMaxN.
+// the sampled frequencies n = 0 and n = 1.  N <= kQpMaxN.
 constexpr int kQpMaxN = 80;
 gw_status qp_energies(const HostPlan& h, const double2* H, const double2* Sigx, const double2* Sigc, double mu,
-                      double2* ainv_scratch, double* E, cudaStream_t st);
+                      double* E, cudaStream_t st);
 
 // Eq. sf_9: Sigma(k, w_r + i delta) [n_k][n_real][N][N] from Sigma(k, i w_n) [n_k][n_w][N][N]
 // through the non-negative sampled frequencies (kernels_cont.cu); w_real on the host.

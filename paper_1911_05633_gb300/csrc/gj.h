@@ -8,8 +8,8 @@ namespace gw {
 
 // The largest order held in shared memory: N (N | 1) complex values and the vectors.
 constexpr int kGJSmemMax = 112;
-// The largest order of the trace kernel: a block holds two rows of each of 8 matrices.
-constexpr int kHessMaxN = 896;
+// The largest order of the trace kernel: a block holds four rows of each of 4 matrices.
+constexpr int kHessMaxN = 880;
 
 // Dynamic shared-memory opt-in of the inverse for order N (call with the device current).
 cudaError_t gj_setup(int N);

@@ -202,7 +202,6 @@ gw_status dyson_init(DysonPlan& d, const HostPlan& h) {
                     up((void**)&d.w, w.data(), w.size() * sizeof(double)) &&
                     up((void**)&d.tau, h.tau.data(), h.tau.size() * sizeof(double)) &&
                     up((void**)&d.part, nullptr, (size_t)d.n_k * sizeof(double)) &&
-                    up((void**)&d.ainv, nullptr, (size_t)d.n_k * d.N * d.N * sizeof(double2)) &&
                     up((void**)&d.tr, nullptr, nb * sizeof(double2)) &&
                     up((void**)&d.scale, nullptr, nb * sizeof(double)) &&
                     up((void**)&d.m1, nullptr, (size_t)d.n_k * sizeof(double2)) &&
@@ -234,7 +233,7 @@ gw_status dyson_init(DysonPlan& d, const HostPlan& h) {
 }
 
 void dyson_free(DysonPlan& d) {
-  void* ptrs[] = {d.M, d.perm, d.w, d.tau, d.part, d.ainv, d.tr, d.scale, d.m1, d.count, d.cont, d.spec};
+  void* ptrs[] = {d.M, d.perm, d.w, d.tau, d.part, d.tr, d.scale, d.m1, d.count, d.cont, d.spec};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   d = DysonPlan{};

@@ -37,18 +37,33 @@ __device__ __forceinline__ double wsum(double v) {
   return v;
 }
 
+// |re| + |im| as a key that orders like it: comparisons of doubles run on the FP64 pipe,
+// comparisons of the bits do not.  NaN: -1.
+__device__ __forceinline__ long long size_key(double2 z) {
+  const long long b = __double_as_longlong(fabs(z.x) + fabs(z.y));
+  return b > 0x7ff0000000000000ll ? -1ll : b;
+}
+
 // Leading dimension of a matrix in shared memory: odd, so that the 16-byte words of a
 // column fall on different banks.
 __host__ __device__ inline int ld_odd(int N) { return N | 1; }
+// Words of one matrix of the trace kernel: the row in hand, its derivative, two fresh rows.
+__host__ __device__ inline int trace_stride(int N) { return 4 * N; }
+__device__ __forceinline__ void copy16_async(double2* dst_smem, const double2* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst_smem)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
 // In-place Gauss-Jordan inverse, partial pivoting by |re| + |im| among the rows not yet
 // used (the first of equal ones, rows counted in the order the exchanges of the textbook
 // form would give them).  No rows move: column k is eliminated with pivot row p_k where it
 // lies, and the exchanges are undone as the result is written, inv[k][p_l] = A[p_k][l].
-// Two blocks per SM at N = 72.  3072 inverses of N = 72: 9.24 ms (1.0 TFLOP/s of the 1.25
+// Two blocks per SM at N = 72.  3072 inverses of N = 72: 8.58 ms (1.07 TFLOP/s of the 1.25
 // that FMA chains reach), 17.0 ms for the form that kept the matrix in global memory with
-// one warp per row; 112 of N = 16: 51 us against 134 us.
+// one warp per row; 112 of N = 16: 30 us against 134 us.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kT, 2) k_gj_inverse_smem(double2* __restrict__ A, int N, long long mat_stride,
                                                            int* status) {
@@ -79,15 +94,14 @@ __global__ void __launch_bounds__(kT, 2) k_gj_inverse_smem(double2* __restrict__
   __syncthreads();
   for (int k = 0; k < N; ++k) {
     if (wid == 0) {
-      double best = -1.0;
+      long long best = -1;
       int bi = k;  // place in the exchanged order
       for (int i = k + lane; i < N; i += 32) {
-        const double2 z = M[at[i] * ld + k];
-        const double m = fabs(z.x) + fabs(z.y);
+        const long long m = size_key(M[at[i] * ld + k]);
         if (m > best) { best = m; bi = i; }
       }
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
       }
@@ -97,10 +111,10 @@ __global__ void __launch_bounds__(kT, 2) k_gj_inverse_smem(double2* __restrict__
         at[k] = p;
         piv[k] = p;
         s_p = p;
-        if (!(best > 0.0)) atomicExch(status, 1);
+        if (best <= 0) atomicExch(status, 1);
         const double2 d = M[p * ld + k];
-        const double den = d.x * d.x + d.y * d.y;
-        s_inv = (den > 0.0) ? make_double2(d.x / den, -d.y / den) : make_double2(0.0, 0.0);
+        const double den = fma(d.x, d.x, d.y * d.y), id = 1.0 / den;
+        s_inv = den > 0.0 ? make_double2(d.x * id, -d.y * id) : make_double2(0.0, 0.0);
       }
     }
     __syncthreads();
@@ -298,12 +312,12 @@ __global__ void __launch_bounds__(kT) k_hessenberg(const double2* __restrict__ H
 // neighbouring rows, carried with its derivative in mu.  G lanes per matrix (a warp holds
 // 32 / G), because a row shrinks to one element and the scalar work per column (a
 // reciprocal and two multipliers) is done by every lane of the matrix alike.  The row in
-// hand and its derivative are in shared memory.  A pivot below `tiny` of the matrix's
-// largest element, or a trace that is not finite, sets *flag.  3072 of N = 72: 0.48 ms per
-// mu, 17 ms for the inverses it replaces.
+// hand and its derivative are in shared memory, the fresh rows arrive there one step ahead.  A pivot below `tiny` of the matrix's
+// largest element, or a trace that is not finite, sets *flag.  3072 of N = 72: 0.34 ms per
+// mu (0.48 with the rows fetched as they are needed, 0.66 with four lanes per matrix), 17 ms for the inverses it replaces.
 // ---------------------------------------------------------------------------
 template <int G>
-__global__ void __launch_bounds__(64) k_hess_trace(const double2* __restrict__ Hs, const double* __restrict__ scale,
+__global__ void __launch_bounds__(32) k_hess_trace(const double2* __restrict__ Hs, const double* __restrict__ scale,
                                                    double mu, int N, long long n_b, double tiny,
                                                    double2* __restrict__ tr, int* __restrict__ flag) {
   extern __shared__ double2 smt[];
@@ -312,28 +326,39 @@ __global__ void __launch_bounds__(64) k_hess_trace(const double2* __restrict__ H
   const int q = threadIdx.x % G;
   const bool on = b < n_b;
   const double2* A = Hs + (on ? b : 0) * (long long)N * N;
-  double2* r = smt + (size_t)(threadIdx.x / G) * 2 * N;  // [N] the row in hand
+  double2* r = smt + (size_t)(threadIdx.x / G) * trace_stride(N);  // [N] the row in hand
   double2* dr = r + N;                                    // [N] its derivative
+  double2* fr = dr + N;                                   // [2][N] rows k + 1 and k + 2
   for (int j = q; j < N; j += G) {
     double2 a = A[j];
     if (j == 0) a.x += mu;
     r[j] = a;
     dr[j] = make_double2(j == 0 ? 1.0 : 0.0, 0.0);
+    if (N > 1) copy16_async(fr + j, A + N + j);
   }
-  __syncwarp();
-  const double low = tiny * (scale[on ? b : 0] + fabs(mu));
+  copies_commit();
+  const long long low = __double_as_longlong(tiny * (scale[on ? b : 0] + fabs(mu)));
   double2 sum = make_double2(0.0, 0.0);
   bool bad = false;
   for (int k = 0; k < N; ++k) {
+    copies_wait();  // row k + 1 has landed; the copy of row k + 2 runs beside this step
+    __syncwarp();
     const double2 rk = r[k], dk = dr[k];
     const bool last = k + 1 == N;
-    const double2* nx = A + (long long)(last ? k : k + 1) * N;  // row k + 1
+    const double2* nx = fr + (k & 1) * N;  // row k + 1
+    if (k + 2 < N) {
+      const double2* src = A + (long long)(k + 2) * N;
+      double2* dst = fr + ((k + 1) & 1) * N;
+      for (int j = k + 1 + q; j < N; j += G) copy16_async(dst + j, src + j);
+    }
+    copies_commit();
     const double2 hk = last ? make_double2(0.0, 0.0) : nx[k];
     // the fresh row's derivative is one at its diagonal, column k + 1: zero in column k
-    const bool fresh = fabs(hk.x) + fabs(hk.y) > fabs(rk.x) + fabs(rk.y);
+    const long long kh = size_key(hk), kr = size_key(rk);
+    const bool fresh = kh > kr;
     const double2 p = fresh ? hk : rk, o = fresh ? rk : hk;
     const double2 dp = fresh ? make_double2(0.0, 0.0) : dk, dof = fresh ? dk : make_double2(0.0, 0.0);
-    bad = bad || !(fabs(p.x) + fabs(p.y) > low);
+    bad = bad || (fresh ? kh : kr) <= low;
     const double id = 1.0 / fma(p.x, p.x, p.y * p.y);
     const double2 inv = make_double2(p.x * id, -p.y * id);
     sum = cfma_(dp, inv, sum);
@@ -341,7 +366,7 @@ __global__ void __launch_bounds__(64) k_hess_trace(const double2* __restrict__ H
     // o -= f p with f = o_k / p_k, f' = (o'_k - f p'_k) / p_k
     const double2 f = cmul_(o, inv), mf = make_double2(-f.x, -f.y);
     const double2 df = cmul_(cfma_(mf, dp, dof), inv), mdf = make_double2(-df.x, -df.y);
-    __syncwarp();
+    __syncwarp();  // every lane has read column k of the row in hand
     for (int j = k + 1 + q; j < N; j += G) {
       double2 a = nx[j];
       if (j == k + 1) a.x += mu;
@@ -352,7 +377,6 @@ __global__ void __launch_bounds__(64) k_hess_trace(const double2* __restrict__ H
       r[j] = cfma_(mf, pj, oj);
       dr[j] = cfma_(mdf, pj, cfma_(mf, dpj, doj));
     }
-    __syncwarp();
   }
   if (on && q == 0) {
     tr[b] = sum;
@@ -396,10 +420,10 @@ void gj_batch(double2* mats, int* perm, int batch, int N, long long stride, int*
   }
 }
 
-constexpr int kTraceG = 8, kTraceThreads = 64, kTracePer = kTraceThreads / kTraceG;
+constexpr int kTraceG = 8, kTraceThreads = 32, kTracePer = kTraceThreads / kTraceG;
 
 cudaError_t hess_setup(int N) {
-  const cudaError_t e = raise_smem_limit(k_hess_trace<kTraceG>, (size_t)kTracePer * 2 * N * sizeof(double2));
+  const cudaError_t e = raise_smem_limit(k_hess_trace<kTraceG>, (size_t)kTracePer * trace_stride(N) * sizeof(double2));
   if (e != cudaSuccess) return e;
   return N <= kGJSmemMax ? raise_smem_limit(k_hessenberg<true>, hess_smem_bytes(N, true))
                          : raise_smem_limit(k_hessenberg<false>, hess_smem_bytes(N, false));
@@ -420,7 +444,7 @@ void hess_trace(const double2* Hs, const double* scale, double mu, int N, long l
   // a pivot this far below the matrix leaves no digits in its reciprocal
   const double tiny = 1e-14;
   k_hess_trace<kTraceG><<<(unsigned)((n_b + kTracePer - 1) / kTracePer), kTraceThreads,
-                          (size_t)kTracePer * 2 * N * sizeof(double2), st>>>(Hs, scale, mu, N, n_b, tiny, tr, flag);
+                          (size_t)kTracePer * trace_stride(N) * sizeof(double2), st>>>(Hs, scale, mu, N, n_b, tiny, tr, flag);
 }
 
 }  // namespace gw

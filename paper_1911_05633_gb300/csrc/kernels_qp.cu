@@ -1,7 +1,7 @@
 // Linearised quasiparticle energies on the device: Sigma_c(i w) ~ S0 + i w S1 through the
 // two lowest positive fermionic frequencies, then the eigenvalues of
 // A^{-1} (H + Sigma_x^h + S0^h - mu) A^{-1} + mu with A = (I - S1^h)^{1/2} (h: Hermitian part).
-// One block per momentum; the Hermitian eigenproblems by cyclic Jacobi in shared memory.
+// One block per momentum, in shared memory.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -15,102 +15,10 @@ namespace gw {
 
 namespace {
 
-__device__ __forceinline__ double2 cmulq(double2 a, double2 b) {
-  return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
-}
 __device__ __forceinline__ double2 conjq(double2 a) { return make_double2(a.x, -a.y); }
 
-// Sum over the block, returned to every thread.
-__device__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-  return s;
-}
-
-struct Rot {
-  int p, q;
-  double c, s;
-  double2 e;  // a_pq / |a_pq|
-};
-
-// Hermitian a (N x N at stride Np, Np = N rounded up to even) -> J^H a J diagonal by cyclic
-// Jacobi: per sweep Np - 1 rounds of Np / 2 disjoint pairs (the round-robin order), each
-// round one rotation per pair, J_pq = D P with D = diag(1, e^{-i phi}) making a_pq real
-// and P the real Jacobi rotation of the 2 x 2 block.  v <- v J when v is given.  Stops when
-// the off-diagonal squared norm is below 1e-30 of the total (at most max_sweeps sweeps).
-__device__ void jacobi_heev(double2* a, double2* v, int N, int Np, int max_sweeps, Rot* rot, double* red) {
-  const int tid = threadIdx.x, nt = blockDim.x, half = Np / 2;
-  double t = 0.0;
-  for (int x = tid; x < N * N; x += nt) {
-    const double2 z = a[(x / N) * Np + x % N];
-    t += z.x * z.x + z.y * z.y;
-  }
-  const double total = block_sum(t, red);
-  for (int sw = 0; sw < max_sweeps; ++sw) {
-    double o = 0.0;
-    for (int x = tid; x < N * N; x += nt) {
-      const int i = x / N, j = x % N;
-      if (i != j) {
-        const double2 z = a[i * Np + j];
-        o += z.x * z.x + z.y * z.y;
-      }
-    }
-    if (!(block_sum(o, red) > 1e-30 * total)) break;
-    for (int r = 0; r < Np - 1; ++r) {
-      if (tid < half) {
-        Rot R;
-        if (tid == 0) { R.p = Np - 1; R.q = r; }
-        else { R.p = (r + tid) % (Np - 1); R.q = (r - tid + Np - 1) % (Np - 1); }
-        R.c = 1.0;
-        R.s = 0.0;
-        R.e = make_double2(1.0, 0.0);
-        if (R.p < N && R.q < N) {
-          const double2 apq = a[R.p * Np + R.q];
-          const double m = hypot(apq.x, apq.y);
-          if (m > 0.0) {
-            R.e = make_double2(apq.x / m, apq.y / m);
-            const double zeta = (a[R.q * Np + R.q].x - a[R.p * Np + R.p].x) / (2.0 * m);
-            const double tt = fabs(zeta) > 1e150 ? 0.5 / zeta : copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-            R.c = 1.0 / sqrt(1.0 + tt * tt);
-            R.s = tt * R.c;
-          }
-        }
-        rot[tid] = R;
-      }
-      __syncthreads();
-      // rows p, q: a <- J^H a
-      for (int x = tid; x < half * Np; x += nt) {
-        const Rot R = rot[x / Np];
-        if (R.s == 0.0) continue;
-        const int j = x % Np;
-        const double2 ap = a[R.p * Np + j], eq = cmulq(R.e, a[R.q * Np + j]);
-        a[R.p * Np + j] = make_double2(R.c * ap.x - R.s * eq.x, R.c * ap.y - R.s * eq.y);
-        a[R.q * Np + j] = make_double2(R.s * ap.x + R.c * eq.x, R.s * ap.y + R.c * eq.y);
-      }
-      __syncthreads();
-      // columns p, q: a <- a J, v <- v J
-      for (int x = tid; x < half * Np; x += nt) {
-        const Rot R = rot[x / Np];
-        if (R.s == 0.0) continue;
-        const int i = x % Np;
-        const double2 eb = conjq(R.e);
-        double2 ap = a[i * Np + R.p], eq = cmulq(eb, a[i * Np + R.q]);
-        a[i * Np + R.p] = make_double2(R.c * ap.x - R.s * eq.x, R.c * ap.y - R.s * eq.y);
-        a[i * Np + R.q] = make_double2(R.s * ap.x + R.c * eq.x, R.s * ap.y + R.c * eq.y);
-        if (v) {
-          ap = v[i * Np + R.p];
-          eq = cmulq(eb, v[i * Np + R.q]);
-          v[i * Np + R.p] = make_double2(R.c * ap.x - R.s * eq.x, R.c * ap.y - R.s * eq.y);
-          v[i * Np + R.q] = make_double2(R.s * ap.x + R.c * eq.x, R.s * ap.y + R.c * eq.y);
-        }
-      }
-      __syncthreads();
-    }
-  }
+__device__ __forceinline__ double2 cfmq(double2 a, double2 b, double2 c) {  // c + a b
+  return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
 }
 
 // Hermitian part of element (i, j) of M (row-major N x N) at offset base.
@@ -119,122 +27,252 @@ __device__ __forceinline__ double2 herm_el(const double2* __restrict__ M, long l
   return make_double2(0.5 * (x.x + y.x), 0.5 * (x.y - y.y));
 }
 
-// One block per momentum k; Ainv: global scratch [N_k][N][N].
-__global__ void __launch_bounds__(256) k_qp_energies(const double2* __restrict__ H, const double2* __restrict__ Sx,
+// Leading dimension in shared memory: odd, so that the words of a column fall on different banks.
+__host__ __device__ inline int qp_ld(int N) { return N | 1; }
+constexpr int kQT = 256;     // threads per block
+constexpr int kQPoints = 3;  // interior points per eigenvalue and section
+static_assert(kQpMaxN * kQPoints <= kQT, "one thread per section point");
+
+// f(i, j) over the rows and columns r0 .. N - 1, flattened over the block (every lane busy:
+// the FP64 pipe issues two multiply-adds per clock and SM, so idle lanes are what costs).
+template <typename F>
+__device__ __forceinline__ void each(int rows, int cols, F f) {
+  const int di = kQT / cols, dj = kQT - di * cols;
+  int i = threadIdx.x / cols, j = threadIdx.x - (threadIdx.x / cols) * cols;
+  while (i < rows) {
+    f(i, j);
+    i += di;
+    j += dj;
+    if (j >= cols) { j -= cols; ++i; }
+  }
+}
+
+// One block per momentum k.  The energies are the eigenvalues of X c = (E - mu) B c with
+// X = H^h + Sigma_x^h + S0^h - mu and B = I - S1^h, the same as those of A^{-1} X A^{-1},
+// A = B^{1/2}: B = L L^H by Cholesky, Z = L^{-1} X L^{-H}, Z to a real tridiagonal by
+// Householder reflections, its eigenvalues by sections on Sturm counts (all at once, three
+// interior points per eigenvalue and step).  About 13 N^3 FP64 operations per momentum; the
+// cyclic Jacobi iterations this replaces took about 270 N^3: 2.96 ms for 64 momenta of N = 72, against 34.3.
+__global__ void __launch_bounds__(kQT) k_qp_energies(const double2* __restrict__ H, const double2* __restrict__ Sx,
                                                      const double2* __restrict__ Sc, int n_w, int i0, int i1,
-                                                     double w0, double w1, double mu, int N, int max_sweeps,
-                                                     double2* __restrict__ Ainv, double* __restrict__ E) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int Np = (N + 1) & ~1;
-  double2* a = reinterpret_cast<double2*>(smraw);  // [Np][Np]
-  double2* v = a + (size_t)Np * Np;                // [Np][Np]
-  __shared__ Rot rot[kQpMaxN / 2];
-  __shared__ double red[8];
-  const int tid = threadIdx.x, nt = blockDim.x;
+                                                     double w0, double w1, double mu, int N,
+                                                     double* __restrict__ E) {
+  extern __shared__ double2 smq[];
+  const int ld = qp_ld(N);
+  double2* X = smq;                                   // [N][ld]
+  double2* L = X + (size_t)N * ld;                    // [N][ld]
+  double2* v = L + (size_t)N * ld;                    // [N] Householder vector
+  double2* p = v + N;                                 // [N]
+  double* d = reinterpret_cast<double*>(p + N);       // [N] diagonal
+  double* e2 = d + N;                                 // [N] squared off-diagonals
+  __shared__ double s_beta, s_lo, s_hi, s_min;
+  __shared__ int s_on;
+  __shared__ double lo[kQpMaxN], hi[kQpMaxN];
+  __shared__ unsigned char cnt[kQT];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const long long k = blockIdx.x;
   const long long NN = (long long)N * N;
   const long long b0 = (k * n_w + i0) * NN, b1 = (k * n_w + i1) * NN;
   // S1 = (Sc(i w1) - Sc(i w0)) / (i (w1 - w0)); S0 = Sc(i w0) - i w0 S1
+  const double fw = 1.0 / (w1 - w0);
   auto s1 = [&](int i, int j) -> double2 {
     if (!Sc) return make_double2(0.0, 0.0);
     const double2 d1 = Sc[b1 + (long long)i * N + j], d0 = Sc[b0 + (long long)i * N + j];
-    const double f = 1.0 / (w1 - w0);
-    return make_double2((d1.y - d0.y) * f, -(d1.x - d0.x) * f);  // (d1 - d0) / i
+    return make_double2((d1.y - d0.y) * fw, -(d1.x - d0.x) * fw);  // (d1 - d0) / i
   };
   auto s0 = [&](int i, int j) -> double2 {
     if (!Sc) return make_double2(0.0, 0.0);
     const double2 d0 = Sc[b0 + (long long)i * N + j], m = s1(i, j);
     return make_double2(d0.x + w0 * m.y, d0.y - w0 * m.x);  // d0 - i w0 S1
   };
-  // B = I - S1^h, V = I (padding rows and columns zero)
-  for (int x = tid; x < Np * Np; x += nt) {
-    const int i = x / Np, j = x % Np;
-    double2 z = make_double2(0.0, 0.0);
-    if (i < N && j < N) {
-      const double2 p = s1(i, j), q = s1(j, i);
-      z = make_double2((i == j ? 1.0 : 0.0) - 0.5 * (p.x + q.x), -0.5 * (p.y - q.y));
-    }
-    a[x] = z;
-    v[x] = make_double2(i == j ? 1.0 : 0.0, 0.0);
-  }
-  __syncthreads();
-  jacobi_heev(a, v, N, Np, max_sweeps, rot, red);
-  // Ainv = U diag(lambda^{-1/2}) U^H
-  for (int x = tid; x < N * N; x += nt) {
-    const int i = x / N, j = x % N;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int l = 0; l < N; ++l) {
-      const double f = rsqrt(a[l * Np + l].x);
-      acc = make_double2(fma(f, cmulq(v[i * Np + l], conjq(v[j * Np + l])).x, acc.x),
-                         fma(f, cmulq(v[i * Np + l], conjq(v[j * Np + l])).y, acc.y));
-    }
-    Ainv[k * NN + x] = acc;
-  }
-  __syncthreads();
-  // X = H^h + Sx^h + S0^h - mu into v, T = Ainv X into a, Y = T Ainv into v, then a = Y^h
-  for (int x = tid; x < N * N; x += nt) {
-    const int i = x / N, j = x % N;
+  each(N, N, [&](int i, int j) {
+    const double2 a = s1(i, j), b = s1(j, i);
+    L[i * ld + j] = make_double2((i == j ? 1.0 : 0.0) - 0.5 * (a.x + b.x), -0.5 * (a.y - b.y));
     double2 z = herm_el(H, k * NN, N, i, j);
     if (Sx) {
       const double2 y = herm_el(Sx, k * NN, N, i, j);
       z.x += y.x;
       z.y += y.y;
     }
-    const double2 p = s0(i, j), q = s0(j, i);
-    z.x += 0.5 * (p.x + q.x) - (i == j ? mu : 0.0);
-    z.y += 0.5 * (p.y - q.y);
-    v[i * Np + j] = z;
+    const double2 f = s0(i, j), q = s0(j, i);
+    z.x += 0.5 * (f.x + q.x) - (i == j ? mu : 0.0);
+    z.y += 0.5 * (f.y - q.y);
+    X[i * ld + j] = z;
+  });
+  __syncthreads();
+  // Cholesky, column by column (an indefinite B gives NaN energies); the reciprocal of the
+  // diagonal stands on the diagonal, and X <- L^{-1} X takes its step j in the same pass
+  for (int j = 0; j < N; ++j) {
+    if (t == 0) L[j * ld + j] = make_double2(1.0 / sqrt(L[j * ld + j].x), 0.0);
+    __syncthreads();
+    const double r = L[j * ld + j].x;
+    for (int i = t; i < N; i += kQT) {
+      X[j * ld + i] = make_double2(r * X[j * ld + i].x, r * X[j * ld + i].y);
+      if (i > j) L[i * ld + j] = make_double2(r * L[i * ld + j].x, r * L[i * ld + j].y);
+    }
+    __syncthreads();
+    const int m = N - 1 - j;
+    if (m > 0) {
+      each(m, m, [&](int a, int b) {  // B_ic -= L_ij conj(L_cj), the lower triangle
+        if (b > a) return;
+        const double2 x = L[(j + 1 + a) * ld + j], y = L[(j + 1 + b) * ld + j];
+        double2* z = L + (j + 1 + a) * ld + j + 1 + b;
+        *z = cfmq(x, make_double2(-y.x, y.y), *z);
+      });
+      each(m, N, [&](int a, int c) {
+        const double2 x = L[(j + 1 + a) * ld + j];
+        double2* z = X + (j + 1 + a) * ld + c;
+        *z = cfmq(make_double2(-x.x, -x.y), X[j * ld + c], *z);
+      });
+    }
+    __syncthreads();
+  }
+  // Z = X L^{-H}: column j scaled, taken out of the columns after it
+  for (int j = 0; j < N; ++j) {
+    const double r = L[j * ld + j].x;
+    for (int i = t; i < N; i += kQT) X[i * ld + j] = make_double2(r * X[i * ld + j].x, r * X[i * ld + j].y);
+    __syncthreads();
+    const int m = N - 1 - j;
+    if (m > 0)
+      each(N, m, [&](int i, int c) {
+        const double2 y = L[(j + 1 + c) * ld + j];
+        double2* z = X + i * ld + j + 1 + c;
+        *z = cfmq(make_double2(-y.x, y.y), X[i * ld + j], *z);
+      });
+    __syncthreads();
+  }
+  // the Hermitian part, into L's storage
+  each(N, N, [&](int i, int j) {
+    const double2 a = X[i * ld + j], b = X[j * ld + i];
+    L[i * ld + j] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
+  });
+  __syncthreads();
+  double2* A = L;
+  for (int c = 0; c + 1 < N; ++c) {
+    const int r0 = c + 1, m = N - r0;
+    if (wid == 0) {
+      double below = 0.0;
+      for (int i = r0 + 1 + lane; i < N; i += 32) {
+        const double2 z = A[i * ld + c];
+        below = fma(z.x, z.x, fma(z.y, z.y, below));
+        v[i] = z;
+      }
+      for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+      if (lane == 0) {
+        const double2 x0 = A[r0 * ld + c];
+        const double a0 = x0.x * x0.x + x0.y * x0.y;
+        d[c] = A[c * ld + c].x;
+        e2[c] = below + a0;
+        s_on = !(below == 0.0);
+        // v = x + e^{i theta} |x| e_1, beta = 2 / v^H v
+        const double norm = sqrt(below + a0), ab = sqrt(a0);
+        const double2 ph = ab > 0.0 ? make_double2(x0.x / ab, x0.y / ab) : make_double2(1.0, 0.0);
+        v[r0] = make_double2(fma(ph.x, norm, x0.x), fma(ph.y, norm, x0.y));
+        s_beta = 1.0 / (norm * (norm + ab));
+      }
+    }
+    __syncthreads();
+    if (s_on) {
+      const double beta = s_beta;
+      // p = beta A v, four lanes per row
+      for (int i = r0 + (t >> 2); i < N; i += kQT / 4) {
+        const unsigned mask = 0xFu << (lane & ~3);
+        double2 acc = make_double2(0.0, 0.0);
+        for (int j = r0 + (t & 3); j < N; j += 4) acc = cfmq(A[i * ld + j], v[j], acc);
+        for (int o = 1; o < 4; o <<= 1) {
+          acc.x += __shfl_xor_sync(mask, acc.x, o);
+          acc.y += __shfl_xor_sync(mask, acc.y, o);
+        }
+        if ((t & 3) == 0) p[i] = make_double2(beta * acc.x, beta * acc.y);
+      }
+      __syncthreads();
+      if (wid == 0) {  // w = p - (beta / 2) (v^H p) v
+        double g = 0.0;
+        for (int i = r0 + lane; i < N; i += 32) g = fma(v[i].x, p[i].x, fma(v[i].y, p[i].y, g));
+        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        g *= -0.5 * beta;
+        for (int i = r0 + lane; i < N; i += 32) p[i] = make_double2(fma(g, v[i].x, p[i].x), fma(g, v[i].y, p[i].y));
+      }
+      __syncthreads();
+      // A -= v w^H + w v^H
+      each(m, m, [&](int a, int b) {
+        const int i = r0 + a, j = r0 + b;
+        const double2 vi = v[i], wi = p[i], vj = v[j], wj = p[j];
+        double2* z = A + i * ld + j;
+        *z = cfmq(make_double2(-wi.x, -wi.y), conjq(vj), cfmq(make_double2(-vi.x, -vi.y), conjq(wj), *z));
+      });
+    }
+    __syncthreads();
+  }
+  if (t == 0) {
+    d[N - 1] = A[(N - 1) * ld + N - 1].x;
+    e2[N - 1] = 0.0;
   }
   __syncthreads();
-  for (int x = tid; x < N * N; x += nt) {
-    const int i = x / N, j = x % N;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int l = 0; l < N; ++l) {
-      const double2 m = cmulq(Ainv[k * NN + (long long)i * N + l], v[l * Np + j]);
-      acc.x += m.x;
-      acc.y += m.y;
+  // an interval that holds every eigenvalue (Gershgorin), and the smallest pivot of a count
+  if (wid == 0) {
+    double a = 1e300, b = -1e300, e = 0.0;
+    for (int i = lane; i < N; i += 32) {
+      const double r = sqrt(e2[i]) + (i > 0 ? sqrt(e2[i - 1]) : 0.0);
+      a = fmin(a, d[i] - r);
+      b = fmax(b, d[i] + r);
+      e = fmax(e, e2[i]);
     }
-    a[i * Np + j] = acc;
+    for (int o = 16; o > 0; o >>= 1) {
+      a = fmin(a, __shfl_xor_sync(0xffffffffu, a, o));
+      b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
+      e = fmax(e, __shfl_xor_sync(0xffffffffu, e, o));
+    }
+    if (lane == 0) {
+      const double pad = 4e-16 * N * fmax(fabs(a), fabs(b)) + 1e-300;
+      s_lo = a - pad;
+      s_hi = b + pad;
+      s_min = fmax(e, 1.0) * 2.3e-308;
+    }
   }
   __syncthreads();
-  for (int x = tid; x < N * N; x += nt) {
-    const int i = x / N, j = x % N;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int l = 0; l < N; ++l) {
-      const double2 m = cmulq(a[i * Np + l], Ainv[k * NN + (long long)l * N + j]);
-      acc.x += m.x;
-      acc.y += m.y;
-    }
-    v[i * Np + j] = acc;
+  const int ev = t / kQPoints, pt = t - ev * kQPoints;
+  if (pt == 0 && ev < N) {
+    lo[ev] = s_lo;
+    hi[ev] = s_hi;
   }
+  bool nan = false;
+  for (int i = 0; i < N; ++i) nan = nan || !(fabs(d[i]) < 1e300) || !(e2[i] < 1e300);
+  const double pmin = s_min;
   __syncthreads();
-  for (int x = tid; x < Np * Np; x += nt) {
-    const int i = x / Np, j = x % Np;
-    double2 z = make_double2(0.0, 0.0);
-    if (i < N && j < N) {
-      const double2 p = v[i * Np + j], q = v[j * Np + i];
-      z = make_double2(0.5 * (p.x + q.x), 0.5 * (p.y - q.y));
+  // 4^28 = 2^56 sections: below the last bit of the largest eigenvalue
+  for (int it = 0; it < 28; ++it) {
+    if (ev < N) {
+      const double x = lo[ev] + (hi[ev] - lo[ev]) * (0.25 * (pt + 1));
+      int n = 0;  // eigenvalues below x: negative pivots of T - x
+      double q = d[0] - x;
+      if (fabs(q) < pmin) q = -pmin;
+      n += q < 0.0;
+      for (int i = 1; i < N; ++i) {
+        q = d[i] - x - e2[i - 1] / q;
+        if (fabs(q) < pmin) q = -pmin;
+        n += q < 0.0;
+      }
+      cnt[t] = (unsigned char)n;
     }
-    a[x] = z;
-  }
-  __syncthreads();
-  jacobi_heev(a, nullptr, N, Np, max_sweeps, rot, red);
-  // ascending order: rank of each eigenvalue (ties by index)
-  for (int i = tid; i < N; i += nt) {
-    const double li = a[i * Np + i].x;
-    int r = 0;
-    for (int j = 0; j < N; ++j) {
-      const double lj = a[j * Np + j].x;
-      r += (lj < li || (lj == li && j < i)) ? 1 : 0;
+    __syncthreads();
+    if (ev < N && pt == 0) {
+      // the section whose lower end has at most ev eigenvalues below it and whose upper end more
+      int s = 0;
+      while (s < kQPoints && cnt[t + s] <= ev) ++s;
+      const double a = lo[ev], w = hi[ev] - lo[ev];
+      lo[ev] = s > 0 ? a + w * (0.25 * s) : a;
+      if (s < kQPoints) hi[ev] = a + w * (0.25 * (s + 1));
     }
-    E[k * N + r] = li + mu;
+    __syncthreads();
   }
+  if (t < N) E[k * N + t] = nan ? __longlong_as_double(0x7ff8000000000000ll) : 0.5 * (lo[t] + hi[t]) + mu;
 }
 
 }  // namespace
 
 gw_status qp_energies(const HostPlan& h, const double2* H, const double2* Sigx, const double2* Sigc, double mu,
-                      double2* ainv_scratch, double* E, cudaStream_t st) {
+                      double* E, cudaStream_t st) {
   const int N = h.n_orb_total();
   int i0 = -1, i1 = -1;
   for (int n = 0; n < h.n_omega; ++n) {
@@ -249,8 +287,7 @@ gw_status qp_energies(const HostPlan& h, const double2* H, const double2* Sigx, 
     set_last_error("quasiparticle energies: more orbitals than the compiled limit");
     return GW_ERR_UNSUPPORTED;
   }
-  const int Np = (N + 1) & ~1;
-  const size_t smem = 2 * (size_t)Np * Np * sizeof(double2);
+  const size_t smem = (2 * (size_t)N * qp_ld(N) + 2 * (size_t)N) * sizeof(double2) + 2 * (size_t)N * sizeof(double);
   cudaError_t e = raise_smem_limit(k_qp_energies, smem);
   if (e != cudaSuccess) {
     set_last_error(std::string("quasiparticle energies: ") + cudaGetErrorString(e));
@@ -258,8 +295,8 @@ gw_status qp_energies(const HostPlan& h, const double2* H, const double2* Sigx, 
   }
   {
     TimedLaunch tl_("k_qp_energies", st);
-    k_qp_energies<<<h.n_k, 256, smem, st>>>(H, Sigx, Sigc, h.n_omega, i0, i1, M_PI / h.beta, 3.0 * M_PI / h.beta, mu,
-                                            N, 60, ainv_scratch, E);
+    k_qp_energies<<<h.n_k, kQT, smem, st>>>(H, Sigx, Sigc, h.n_omega, i0, i1, M_PI / h.beta, 3.0 * M_PI / h.beta, mu,
+                                            N, E);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) {
