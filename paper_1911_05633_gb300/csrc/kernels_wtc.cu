@@ -3,13 +3,8 @@
 // residual I - A X evaluated to FP64 accuracy on tcgen05 from exact BF16 slices of A
 // and X (an Ozaki-type splitting): after a power-of-two scaling per row of A and per
 // column of X, every entry is a sum of slices a_s = alpha_s 2^-7(s+1), |alpha_s| <= 128,
-// each exact in BF16.  The products a_s x_t with s + t = L are multiples of 2^-7(L+2).
-// For K = N <= 384 terms their sums stay below 2^24 such units in these accumulators,
-// so FP32 accumulation is exact: levels 0, 1, 2 (Re: ArXr - AiXi, Im: ArXi + AiXr
-// together), levels 3 and 4 (one product type per accumulator).  The levels >= 5 share
-// one FP32 accumulator, whose rounding is ~2^-60 N of |A||X|.  The epilogue adds the
-// levels in FP64, level 0 first against the identity.  Two refinements take the FP32
-// inverse (error ~ kappa 1e-7) to ~1e-13 for kappa ~ 2e3.
+// each exact in BF16 (k_oz_product below).  Two refinements take the FP32 inverse (error
+// ~ kappa 1e-7) to ~1e-13 for kappa ~ 2e3.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -378,84 +373,138 @@ __global__ void k_slice_X(const float2* __restrict__ hi, const float2* __restric
   }
 }
 
-// Accumulator q (0..7) of one residual entry in units of 2^-52.  Accumulators 0..6
-// hold exact multiples of 2^-14, 2^-21, 2^-28, 2^-35, 2^-35, 2^-42, 2^-42 below 2^24
-// such units, so the scaled value is an exact integer (level 0 below 2^62); accumulator
-// 7 (levels >= 5) is rounded to 2^-52.
-__device__ __forceinline__ long long level_units52(float v, int q) {
-  switch (q) {
-    case 0: return (long long)__float2int_rn(v * 0x1p14f) << 38;
-    case 1: return (long long)__float2int_rn(v * 0x1p21f) << 31;
-    case 2: return (long long)__float2int_rn(v * 0x1p28f) << 24;
-    case 3:
-    case 4: return (long long)__float2int_rn(v * 0x1p35f) << 17;
-    case 5:
-    case 6: return (long long)__float2int_rn(v * 0x1p42f) << 10;
-    default: return __float2ll_rn(v * 0x1p52f);
+// ---- digit products on the tensor cores -------------------------------------------------
+//
+// One kernel for the residual R = I - A X of the refinements and for the panel products
+// C = A B, C -= A B of the block inverse.  A complex product runs as a real one of twice the
+// length: the Re rows are [Ar, -Ai] [Br; Bi] and the Im rows [Ai, Ar] [Br; Bi], so an output
+// row (Re or Im) takes one digit plane of A and one of B per 16-wide K step (-Ai through the
+// negate-A bit).  The digit products of level L = s + t (digit s of A, digit t of B) go to
+// accumulator L; for digit s of A the digits t of B feed consecutive accumulators, so a run
+// of up to four B planes, consecutive in shared memory, is one MMA of 64 x run columns: 11
+// MMAs per K step for eight levels, at the full rate of the tensor core (36 MMAs 64 wide run
+// at two thirds of it: their operand reads bound them).
+//
+// Exactness: the level sums over at most 512 real terms are integers in their unit
+// 2^-7(L+2) below 2^24 for L <= 5, exact in FP32 whatever rounding the tensor core applies;
+// levels 6 and 7 round far below 2^-52 of the scale.  A longer reduction (N = 384: 768 terms)
+// is taken in two halves: the accumulators are read out as exact 64-bit sums in units of
+// 2^-52 in between.  The sum of all levels is rounded once.
+constexpr int kPT = 512;          // threads: 4 warps per tensor-memory lane quadrant, 16 columns each
+constexpr int kPExact = 512;      // real terms per read-out
+
+// The integer of one level, |I| < 2^25 (the six-level residual keeps 768 terms in one sum):
+// split at a multiple of 8, both parts read by adding 1.5 2^k (a float-to-integer conversion
+// issues at the FP64 rate here: with eight of them per entry the read-out took as long as
+// the products).
+__device__ __forceinline__ int level_int(float v, float sc) {
+  const float x = v * sc;
+  const float y = x + 100663296.0f;                    // 1.5 2^26: x to a multiple of 8
+  return 8 * (__float_as_int(y) - 0x4CC00000) + (__float_as_int((x - (y - 100663296.0f)) + 12582912.0f) - 0x4B400000);
+}
+template <int L>
+__device__ __forceinline__ void add_level(long long& S, float v) {
+  S += (long long)level_int(v, __int_as_float((127 + 7 * (L + 2)) << 23)) << (38 - 7 * L);
+}
+// levels 6 and 7 together, rounded to 2^-52 (below 2^21 of them)
+__device__ __forceinline__ void add_67(long long& S, float v6, float v7) {
+  S += __float_as_int(fmaf(v6 + v7, 0x1p52f, 12582912.0f)) - 0x4B400000;
+}
+// levels 5 .. 7 of one accumulator, rounded to nearest at 2^-52
+__device__ __forceinline__ void add_tail(long long& S, float v) {
+  const float x = v * 0x1p52f;
+  S += fabsf(x) < 0x1p25f ? (long long)level_int(x, 1.0f) : __float2ll_rn(x);
+}
+// S 2^e rounded once to FP32 (ties to even), from the bit fields; below 2^-126: zero
+__device__ __forceinline__ float i2f_scaled(long long S, int e) {
+  if (S == 0) return 0.0f;
+  const uint32_t sign = S < 0 ? 0x80000000u : 0u;
+  unsigned long long m = S < 0 ? (unsigned long long)(-S) : (unsigned long long)S;
+  const int lz = __clzll((long long)m);
+  m <<= lz;  // leading one at bit 63
+  const uint32_t hi = (uint32_t)(m >> 32);
+  const bool rest = (hi & 0x7Fu) != 0u || (uint32_t)m != 0u;  // below the half unit
+  uint32_t f = hi >> 8;  // 24 bits with the leading one
+  if ((hi & 0x80u) && (rest || (f & 1u))) ++f;
+  int ex = 63 - lz + e;
+  if (f >> 24) { f >>= 1; ++ex; }
+  if (ex < -126) return __uint_as_float(sign);
+  if (ex > 127) return __uint_as_float(sign | 0x7F800000u);
+  return __uint_as_float(sign | ((uint32_t)(ex + 127) << 23) | (f & 0x7FFFFFu));
+}
+
+// The MMAs of one 16-wide K step.  `first`: the step's first product of each accumulator
+// writes it.  TAIL: the levels 5 .. LMAX share accumulator 5 (written by the step `first5`).
+template <int SX, int LMAX, bool TAIL>
+__device__ __forceinline__ void product_issue_step(uint32_t tm, uint64_t da0, uint64_t dx0, bool neg, bool first,
+                                                   bool first5) {
+  constexpr uint32_t PA = 128 * 16 * 2, PX = kWTN * 16 * 2;  // bytes per A / B plane
+  constexpr int LW = TAIL ? 4 : LMAX;                          // levels with an accumulator of their own
+  if (TAIL) {
+    const uint32_t id = neg ? idesc_bf16_f32_negA(128, kWTN) : idesc_bf16_f32(128, kWTN);
+    bool fresh = first5;
+#pragma unroll
+    for (int t = 0; t < SX; ++t)
+#pragma unroll
+      for (int s = 0; s <= LMAX; ++s)
+        if (s + t >= 5 && s + t <= LMAX) {
+          mma_bf16(tm + 5 * kWTN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t * PX) >> 4), id, fresh ? 0u : 1u);
+          fresh = false;
+        }
   }
-}
-
-// The residual as a real product of twice the length: the Re rows of A X are
-// [Ar, -Ai] [Xr; Xi] and the Im rows [Ai, Ar] [Xr; Xi], so one output row (Re or Im)
-// accumulates over 2N terms from one digit plane of A and one of X per 16-wide K step
-// (-Ai through the negate-A bit of the instruction descriptor).  The products a_s x_t of
-// level L = s + t go to accumulator q(L, half): levels 0, 1, 2 each one accumulator over
-// both halves of K (<= 2 N terms), levels 3 and 4 one accumulator per half (<= N terms),
-// levels >= 5 one accumulator.
-__host__ __device__ constexpr int ozaki_bucket(int L, int half) {
-  return L <= 2 ? L : L == 3 ? 3 + half : L == 4 ? 5 + half : 7;
-}
-
-// The MMAs of one 16-wide K step, fully unrolled.  `fresh` marks the accumulators whose
-// first product of the whole K loop is in this step (written, not added).
-template <int SX, int NA, int LMAX>
-__device__ __forceinline__ void ozaki_issue_step(uint32_t tm, uint64_t da0, uint64_t dx0, uint32_t id, int half,
-                                                 uint32_t fresh) {
-  constexpr uint32_t PA = 128 * 16 * 2, PX = kWTN * 16 * 2;  // bytes per A / X plane
-  uint32_t used = 0;
 #pragma unroll
-  for (int t = 0; t < SX; ++t) {
+  for (int s = 0; s <= LW; ++s) {
+    const int nt = (LW - s + 1) < SX ? (LW - s + 1) : SX;
 #pragma unroll
-    for (int s = 0; s < NA; ++s) {
-      if (s + t <= LMAX) {
-        const int q = ozaki_bucket(s + t, half);
-        const uint32_t acc = (((fresh & ~used) >> q) & 1u) ? 0u : 1u;
-        used |= 1u << q;
-        // descriptor start addresses are in 16-byte units in the low bits
-        mma_bf16(tm + (uint32_t)q * kWTN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t * PX) >> 4), id, acc);
-      }
+    for (int t0 = 0; t0 < nt; t0 += 4) {
+      const int n = (nt - t0) < 4 ? (nt - t0) : 4;
+      const uint32_t id = neg ? idesc_bf16_f32_negA(128, kWTN * n) : idesc_bf16_f32(128, kWTN * n);
+      // an accumulator's first product: digit 0 of A, or (levels beyond the digits of B) the
+      // smallest digit of A that reaches it, with B's last digit
+      const bool init = s == 0 || (s + t0 >= SX && t0 == SX - 1);
+      mma_bf16(tm + (uint32_t)(s + t0) * kWTN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t0 * PX) >> 4), id,
+               (first && init) ? 0u : 1u);
     }
   }
 }
 
-// R[b] = I - A[b] X[b] for one block of 128 output rows (Re rows for blockIdx.y < N/128,
-// else Im rows) x kWTN columns per block (128 threads), from the A digits s <= LMAX and
-// SX digits of X, products with s + t <= LMAX.  Eight FP32 accumulators of kWTN columns
-// fill the 512 tensor-memory columns.  kWStages shared-memory stages; while step kk runs,
-// the stage of step kk - 1 is refilled with step kk - 1 + kWStages.  The epilogue adds all
-// levels and the identity as one exact 64-bit integer in units of 2^-52 (the levels
-// cancel each other, so they are combined before any rounding), then rounds once to FP32
-// (R is small; FP32 keeps it to 2^-24 of itself) into the Re or Im part of R.
-template <int SX, int LMAX>
-__global__ void __launch_bounds__(128, 1)
-k_ozaki_residual(const uint16_t* __restrict__ Asl, const uint16_t* __restrict__ Xsl, const int* __restrict__ eA,
-                 const int* __restrict__ eX, float2* __restrict__ R, int N, int* status) {
-  static_assert(LMAX >= 5 && LMAX < kWSA, "every accumulator receives a product; A has kWSA digits");
-  constexpr int NA = LMAX + 1;                            // A digits used
+// One block of 128 output rows (Re rows for blockIdx.y < M/128, else Im rows) x kWTN columns
+// from the A digits s <= LMAX and SX digits of B, products with s + t <= LMAX.  kWStages
+// shared-memory stages; while step kk runs, the stage of step kk - 1 is refilled with step
+// kk - 1 + kWStages.  RES: R = I - A B in FP32 (R is small; FP32 keeps it to 2^-24 of itself),
+// else C = A B or C -= A B in FP64; row blocks [skip0, skip1) are left alone.  TAIL: the
+// levels 5 .. 7 in one accumulator, 21 narrow MMAs more per step (the residual of the second
+// refinement keeps the rounding it always had: where v^-1 - P is close to singular, W~ follows
+// the last bits of that residual).  A warp's 32 x
+// 16 results go through shared memory, so that a store covers two rows of 16 columns.
+// 264 complex products 768 x 256 by 256 x 1024 (a step of N = 1024): 3.88 ms, 4.54 with
+// float-to-integer conversions on four warps and 64-column MMAs for the residuals; 936
+// residuals of N = 384: six levels 3.54 ms (5.03), eight with TAIL 6.36 ms (7.07), eight
+// without 5.42 ms.  What bounds it now is the digits' way from L2: 48 KB per K step.
+template <int SX, int LMAX, bool RES, bool TAIL>
+__global__ void __launch_bounds__(kPT, 1) k_oz_product(const __grid_constant__ OzProductArgs g) {
+  constexpr int NL = LMAX + 1;
+  static_assert((NL == 8 && SX == 8) || (NL == 6 && SX == 5), "eight levels of eight digits, or six of five");
+  static_assert(!TAIL || NL == 8, "levels 5 .. 7");
+  static_assert(NL * kWTN <= 512, "the accumulators fit the tensor memory");
   constexpr uint32_t PA = 128 * 16 * 2, PX = kWTN * 16 * 2;
-  constexpr uint32_t AB = NA * PA, XB = SX * PX, SB = AB + XB;  // bytes per stage
+  constexpr uint32_t AB = NL * PA, XB = SX * PX, SB = AB + XB;  // bytes per stage
   constexpr uint32_t XC = wx_chunk(SX);
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t full[kWStages];
   __shared__ __align__(8) uint64_t mmad[kWStages];
+  __shared__ __align__(8) uint64_t gdone;
   const int jb = blockIdx.x;
-  const int NKS = N / 16, NIB = N / 128, NJB = N / kWTN;
+  const int NKS = g.K / 16, NIB = g.M / 128, NJB = g.Nc / kWTN;
   const bool imrow = (int)blockIdx.y >= NIB;
   const int ib = imrow ? (int)blockIdx.y - NIB : (int)blockIdx.y;
+  if (!RES && ib >= g.skip0 && ib < g.skip1) return;  // the whole block: before any barrier or allocation
   const long long b = blockIdx.z;
   const int NK2 = 2 * NKS;
+  const int n_groups = (2 * g.K > kPExact && NL > 6) ? 2 : 1;  // six levels need no exact last bits
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int* status = g.status;
   if (warp == 0) {
     tmem_alloc(&tmem_base, 512);
     tmem_relinquish();
@@ -465,15 +514,17 @@ k_ozaki_residual(const uint16_t* __restrict__ Asl, const uint16_t* __restrict__ 
       mbar_init(&full[s], 1);
       mbar_init(&mmad[s], 1);
     }
+    mbar_init(&gdone, 1);
     fence_mbar_init();
   }
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
   const uint32_t tm = tmem_base;
-  const unsigned char* Abase = reinterpret_cast<const unsigned char*>(Asl) + ((b * NIB + ib) * NKS) * (long long)kWAChunk;
-  const unsigned char* Xbase = reinterpret_cast<const unsigned char*>(Xsl) + ((b * NJB + jb) * NKS) * (long long)XC;
-  // step kk: half 0 takes (Ar | Ai for Im rows) with Xr, half 1 (Ai negated | Ar) with Xi
+  const unsigned char* Abase =
+      reinterpret_cast<const unsigned char*>(g.Asl) + ((b * NIB + ib) * NKS) * (long long)kWAChunk;
+  const unsigned char* Xbase = reinterpret_cast<const unsigned char*>(g.Bsl) + ((b * NJB + jb) * NKS) * (long long)XC;
+  // step kk: half 0 takes (Ar | Ai for Im rows) with Br, half 1 (Ai negated | Ar) with Bi
   auto load = [&](int kk, int st) {
     const int half = kk >= NKS ? 1 : 0, ks = kk - half * NKS;
     const int cA = imrow ? 1 - half : half;
@@ -482,73 +533,119 @@ k_ozaki_residual(const uint16_t* __restrict__ Asl, const uint16_t* __restrict__ 
     bulk_g2s(dst, Abase + (long long)ks * kWAChunk + (long long)cA * kWSA * PA, AB, &full[st]);
     bulk_g2s(dst + AB, Xbase + (long long)ks * XC + (long long)half * SX * PX, XB, &full[st]);
   };
+  const int quad = warp & 3, c0 = 16 * (warp >> 2);  // this warp's lanes 32 quad .. and columns c0 ..
+  const uint32_t t_addr = tm + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
+  long long S[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) S[c] = 0;
   bool ok = true;
-  if (tid == 0) {
-    const uint32_t id = idesc_bf16_f32(128, kWTN), idn = idesc_bf16_f32_negA(128, kWTN);
-    const uint32_t s0 = smem_u32(sm);
+  if (tid == 0)
     for (int s = 0; s < kWStages && s < NK2; ++s) load(s, s);
-    for (int kk = 0; kk < NK2; ++kk) {
-      const int st = kk % kWStages;
-      if (!mbar_wait(&full[st], (uint32_t)(kk / kWStages) & 1u, kWaitNs, status)) { ok = false; break; }
-      fence_after_sync();
-      const int half = kk >= NKS ? 1 : 0;
-      // first products: every accumulator at kk = 0, the second-half ones of levels 3, 4 at kk = NKS
-      const uint32_t fresh = kk == 0 ? 0xFFu : (kk == NKS ? ((1u << 4) | (1u << 6)) : 0u);
-      ozaki_issue_step<SX, NA, LMAX>(tm, smem_desc(s0 + st * SB, 128, 256), smem_desc(s0 + st * SB + AB, 128, 256),
-                                     (!imrow && half) ? idn : id, half, fresh);
-      mma_commit(&mmad[st]);
-      if (kk >= 1 && kk - 1 + kWStages < NK2) {
-        // the products of step kk - 1 are done once its commit arrives: refill its stage
-        const int so = (kk - 1) % kWStages;
-        if (!mbar_wait(&mmad[so], (uint32_t)((kk - 1) / kWStages) & 1u, kWaitNs, status)) { ok = false; break; }
-        load(kk - 1 + kWStages, so);
+  for (int grp = 0; grp < n_groups; ++grp) {
+    if (tid == 0 && ok) {
+      const uint32_t s0 = smem_u32(sm);
+      const int k_end = n_groups == 1 ? NK2 : NKS * (grp + 1);
+      const int k_begin = NKS * grp;
+      for (int kk = k_begin; kk < k_end; ++kk) {
+        const int st = kk % kWStages;
+        if (!mbar_wait(&full[st], (uint32_t)(kk / kWStages) & 1u, kWaitNs, status)) { ok = false; break; }
+        fence_after_sync();
+        product_issue_step<SX, LMAX, TAIL>(tm, smem_desc(s0 + st * SB, 128, 256),
+                                           smem_desc(s0 + st * SB + AB, 128, 256), !imrow && kk >= NKS, kk == k_begin,
+                                           kk == 0);
+        mma_commit(&mmad[st]);
+        if (kk >= 1 && kk - 1 + kWStages < NK2) {
+          // the products of step kk - 1 are done once its commit arrives: refill its stage
+          const int so = (kk - 1) % kWStages;
+          if (!mbar_wait(&mmad[so], (uint32_t)((kk - 1) / kWStages) & 1u, kWaitNs, status)) { ok = false; break; }
+          load(kk - 1 + kWStages, so);
+        }
+      }
+      mma_commit(&gdone);  // also on a failure: the products issued so far
+      if (!ok) atomicExch(status, 2);
+    }
+    __syncwarp();
+    const bool done = mbar_wait(&gdone, (uint32_t)grp & 1u, kWaitNs, status);
+    ok = __syncthreads_and(ok && done ? 1 : 0) != 0;
+    fence_after_sync();
+    if (!ok) break;
+    {
+      float v[32];
+      tmem_ld16x2(t_addr, kWTN, v);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) { add_level<0>(S[c], v[c]); add_level<1>(S[c], v[16 + c]); }
+      tmem_ld16x2(t_addr + 2 * kWTN, kWTN, v);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) { add_level<2>(S[c], v[c]); add_level<3>(S[c], v[16 + c]); }
+      tmem_ld16x2(t_addr + 4 * kWTN, kWTN, v);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        add_level<4>(S[c], v[c]);
+        if (!TAIL) add_level<5>(S[c], v[16 + c]);
+        else if (grp + 1 == n_groups) add_tail(S[c], v[16 + c]);
+      }
+      if (NL == 8 && !TAIL) {
+        tmem_ld16x2(t_addr + 6 * kWTN, kWTN, v);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) add_67(S[c], v[c], v[16 + c]);
       }
     }
+    if (grp + 1 < n_groups) {  // the next half writes the accumulators
+      fence_before_sync();
+      __syncthreads();
+      fence_after_sync();
+    }
   }
-  // every thread waits for the last products; one outcome for the block
-  const int last = NK2 - 1;
-  const bool done = ok && mbar_wait(&mmad[last % kWStages], (uint32_t)(last / kWStages) & 1u, kWaitNs, status);
-  ok = __syncthreads_and(done ? 1 : 0) != 0;
-  fence_after_sync();
   if (!ok) {
     if (tid == 0) atomicExch(status, 2);
   } else {
-    const int i = ib * 128 + 32 * warp + lane;
-    const int ea = eA[b * N + i];
-    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-    // The pipeline stages are free now: each warp stages its 32 x 16 results there, so
-    // that one store instruction covers two rows of 16 columns instead of 32 rows.
-    float* stg = reinterpret_cast<float*>(sm) + warp * (32 * 17);
-    float* Rw = reinterpret_cast<float*>(R + (b * N + ib * 128 + 32 * warp) * (long long)N) + (imrow ? 1 : 0);
-    bool range_ok = true;
-    for (int c0 = 0; c0 < kWTN; c0 += 16) {
-      float v[128];  // accumulator q, column c at v[16 q + c]
-      tmem_ld16x4(tm + lane_base + (uint32_t)c0, kWTN, v);
-      tmem_ld16x4(tm + lane_base + (uint32_t)(4 * kWTN + c0), kWTN, v + 64);
+    const int i = ib * 128 + 32 * quad + lane;
+    const int ea = g.eA[b * g.M + i];
+    const int* eb = g.eB + b * g.Nc + jb * kWTN + c0;
+    const int cc = lane & 15, r2 = lane >> 4;
+    // every product has read its stage: the stages are free for the results
+    if (RES) {
+      float* stg = reinterpret_cast<float*>(sm) + warp * (32 * 17);
+      bool range_ok = true;
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
-        long long val = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) val += level_units52(v[16 * q + c], q);
         const int j = jb * kWTN + c0 + c;
-        const int e = ea + eX[b * N + j];  // (A X)_ij = 2^e sum
+        const int e = ea + eb[c];  // (A X)_ij = 2^e sum
+        long long val = S[c];
         if (!imrow && i == j) {
           if (e < -10 || e > 52) range_ok = false;
           else val -= 1ll << (52 - e);  // 1 = 2^(52 - e) units of 2^(e - 52)
         }
         if (e < -126 || e > 126) range_ok = false;
-        const float sc = __int_as_float((127 + min(max(e, -126), 126)) << 23);  // 2^e
-        stg[lane * 17 + c] = -sc * ((float)val * 0x1p-52f);
+        const float res = i2f_scaled(-val, min(max(e, -126), 126) - 52);
+        stg[lane * 17 + c] = res;
       }
       __syncwarp();
-#pragma unroll 4
+      float* Rw = reinterpret_cast<float*>(g.R + (b * g.M + ib * 128 + 32 * quad) * (long long)g.Nc) + (imrow ? 1 : 0);
+#pragma unroll
       for (int t = 0; t < 16; ++t) {
-        const int rr = 2 * t + (lane >> 4), cc = lane & 15;
-        Rw[2 * ((long long)rr * N + jb * kWTN + c0 + cc)] = stg[rr * 17 + cc];
+        const int rr = 2 * t + r2;
+        Rw[2 * ((long long)rr * g.Nc + jb * kWTN + c0 + cc)] = stg[rr * 17 + cc];
       }
+      if (!range_ok) atomicExch(status, 4);  // scale outside the FP32 exponent range
+    } else {
+      double* stg = reinterpret_cast<double*>(sm) + warp * (32 * 17);
+      double* Cw = reinterpret_cast<double*>(g.C + b * g.c_ms + (long long)(ib * 128 + 32 * quad) * g.ldc) + (imrow ? 1 : 0);
+      // the old C values first: independent loads in flight while the sums are rounded
+      double cold[16];
+#pragma unroll
+      for (int t = 0; t < 16; ++t)
+        cold[t] = g.accumulate ? Cw[2 * ((long long)(2 * t + r2) * g.ldc + jb * kWTN + c0 + cc)] : 0.0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) stg[lane * 17 + c] = i2d_scaled(S[c], ea + eb[c] - 52);
       __syncwarp();
+#pragma unroll
+      for (int t = 0; t < 16; ++t) {
+        const int rr = 2 * t + r2;
+        const double pv = stg[rr * 17 + cc];
+        Cw[2 * ((long long)rr * g.ldc + jb * kWTN + c0 + cc)] = g.accumulate ? cold[t] - pv : pv;
+      }
     }
-    if (!range_ok) atomicExch(status, 4);  // scale outside the FP32 exponent range
   }
   fence_before_sync();
   __syncthreads();
@@ -760,8 +857,9 @@ k_refine_tc(const uint16_t* __restrict__ PX, const uint16_t* __restrict__ PR, co
 
 cudaError_t wtc_setup(size_t smem_gj32) {
   cudaError_t e = raise_smem_limit(k_gj_inverse_f32, smem_gj32);
-  if (e == cudaSuccess) e = raise_smem_limit(k_ozaki_residual<kWSX0, kWL0>, w_residual_smem(kWSX0, kWL0));
-  if (e == cudaSuccess) e = raise_smem_limit(k_ozaki_residual<kWSX1, kWLmax>, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX0, kWL0, true, false>, w_residual_smem(kWSX0, kWL0));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, true>, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, false>, w_residual_smem(kWSX1, kWLmax));
   if (e == cudaSuccess) e = raise_smem_limit(k_refine_tc<0>, w_refine_smem());
   if (e == cudaSuccess) e = raise_smem_limit(k_refine_tc<1>, w_refine_smem());
   if (e == cudaSuccess) e = raise_smem_limit(k_refine_tc<2>, w_refine_smem());
@@ -777,6 +875,14 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   const unsigned g8 = (unsigned)((t8 + 255) / 256 < 65535LL * 8 ? (t8 + 255) / 256 : 65535LL * 8);
   const dim3 gcol((unsigned)((N + 127) / 128), (unsigned)batch);
   const dim3 gres((unsigned)(N / kWTN), (unsigned)(2 * (N / 128)), (unsigned)batch);  // Re rows, then Im rows
+  OzProductArgs ga{};
+  ga.Asl = w.Asl;
+  ga.Bsl = w.Xsl;
+  ga.eA = w.eA;
+  ga.eB = w.eX;
+  ga.R = w.R;
+  ga.M = ga.Nc = ga.K = N;
+  ga.status = w.status;
   const dim3 gref((unsigned)(N / 128), (unsigned)(N / 128), (unsigned)batch);
   // X0: FP32 Gauss-Jordan
   {
@@ -807,8 +913,7 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_ozaki_residual<first>", st);
-    k_ozaki_residual<kWSX0, kWL0><<<gres, 128, w_residual_smem(kWSX0, kWL0), st>>>(w.Asl, w.Xsl, w.eA, w.eX, w.R, N,
-                                                                                  w.status);
+    k_oz_product<kWSX0, kWL0, true, false><<<gres, kPT, w_residual_smem(kWSX0, kWL0), st>>>(ga);
   }
   {
     gw::TimedLaunch tl_("k_split3_rows", st);
@@ -833,8 +938,7 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_ozaki_residual<second>", st);
-    k_ozaki_residual<kWSX1, kWLmax><<<gres, 128, w_residual_smem(kWSX1, kWLmax), st>>>(w.Asl, w.Xsl, w.eA, w.eX, w.R,
-                                                                                      N, w.status);
+    k_oz_product<kWSX1, kWLmax, true, true><<<gres, kPT, w_residual_smem(kWSX1, kWLmax), st>>>(ga);
   }
   {
     gw::TimedLaunch tl_("k_split3_cols", st);
@@ -866,8 +970,7 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
     }
     {
       gw::TimedLaunch tl_("k_ozaki_residual<third>", st);
-      k_ozaki_residual<kWSX1, kWLmax><<<gres, 128, w_residual_smem(kWSX1, kWLmax), st>>>(w.Asl, w.Xsl, w.eA, w.eX,
-                                                                                        w.R, N, w.status);
+      k_oz_product<kWSX1, kWLmax, true, false><<<gres, kPT, w_residual_smem(kWSX1, kWLmax), st>>>(ga);
     }
     {
       gw::TimedLaunch tl_("k_split3_cols", st);
@@ -1027,167 +1130,6 @@ __global__ void k_copy_panel(const double2* __restrict__ src, long long sms, int
 }
 
 
-// Level L of a panel product (accumulator L) in units of 2^-52.  With K <= kWblkMaxK
-// complex terms (2K real products per level) the sums of levels 0..5 are integers in their
-// unit 2^-7(L+2) below 2^24, so exact in FP32; levels 6 and 7 are rounded there and here,
-// far below 2^-52 of the scale.
-__device__ __forceinline__ long long panel_units52(float v, int L) {
-  switch (L) {
-    case 0: return (long long)__float2int_rn(v * 0x1p14f) << 38;
-    case 1: return (long long)__float2int_rn(v * 0x1p21f) << 31;
-    case 2: return (long long)__float2int_rn(v * 0x1p28f) << 24;
-    case 3: return (long long)__float2int_rn(v * 0x1p35f) << 17;
-    case 4: return (long long)__float2int_rn(v * 0x1p42f) << 10;
-    case 5: return (long long)__float2int_rn(v * 0x1p49f) << 3;
-    default: return __float2ll_rn(v * 0x1p52f);
-  }
-}
-
-// The MMAs of one 16-wide K step of a panel product: accumulator L holds level L, so for
-// digit s of A the digits t = 0 .. 7 - s of B feed the consecutive accumulators s .. 7, and
-// a run of up to four B planes (consecutive in shared memory) is one MMA of 64 x run
-// columns: 11 MMAs per K step, each A plane read at most twice.
-// `first`: the first K step, whose runs of digit 0 write their accumulators (every level
-// has one) and the later runs add to them.
-__device__ __forceinline__ void panel_issue_step(uint32_t tm, uint64_t da0, uint64_t dx0, bool neg, bool first) {
-  constexpr uint32_t PA = 128 * 16 * 2, PX = kWTN * 16 * 2;  // bytes per A / B plane
-#pragma unroll
-  for (int s = 0; s <= kWLmax; ++s) {
-#pragma unroll
-    for (int t0 = 0; t0 <= kWLmax - s; t0 += 4) {
-      const int n = (kWLmax - s - t0 + 1) < 4 ? (kWLmax - s - t0 + 1) : 4;
-      const uint32_t id = neg ? idesc_bf16_f32_negA(128, kWTN * n) : idesc_bf16_f32(128, kWTN * n);
-      mma_bf16(tm + (uint32_t)(s + t0) * kWTN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t0 * PX) >> 4), id,
-               (first && s == 0) ? 0u : 1u);
-    }
-  }
-}
-
-// C = A B (accumulate 0) or C = C - A B (accumulate 1) for an M x K panel A and a K x Nc
-// panel B given as digits (k_slice_panel_A / _B), K <= kWblkMaxK, FP64 out.  Blocks of
-// 128 output rows (Re rows for blockIdx.y < M/128, else Im rows) x kWTN columns, the
-// products a_s b_t with s + t <= 7 in eight level accumulators (one per level, both K
-// halves together); row blocks [skip0, skip1) are left alone.  The epilogue sums the
-// levels as one exact 64-bit integer in units of 2^(eA + eB - 52), rounds it once to FP64
-// and stages each warp's 32 x 16 results in shared memory so that a store covers two rows
-// of 16 columns.
-__global__ void __launch_bounds__(128, 1) k_oz_panel_gemm(const __grid_constant__ PanelGemmArgs g) {
-  constexpr int SX = kWSX1, LMAX = kWLmax, NA = LMAX + 1;
-  static_assert(LMAX == 7 && SX == 8, "eight levels, eight accumulators of kWTN columns");
-  static_assert(NA <= kWSA, "A has kWSA digits");
-  constexpr uint32_t PA = 128 * 16 * 2, PX = kWTN * 16 * 2;
-  constexpr uint32_t AB = NA * PA, XB = SX * PX, SB = AB + XB;
-  constexpr uint32_t XC = wx_chunk(SX);
-  extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ uint32_t tmem_base;
-  __shared__ __align__(8) uint64_t full[kWStages];
-  __shared__ __align__(8) uint64_t mmad[kWStages];
-  const int jb = blockIdx.x;
-  const int NKS = g.K / 16, NIB = g.M / 128, NJB = g.Nc / kWTN;
-  const bool imrow = (int)blockIdx.y >= NIB;
-  const int ib = imrow ? (int)blockIdx.y - NIB : (int)blockIdx.y;
-  if (ib >= g.skip0 && ib < g.skip1) return;  // the whole block: before any barrier or allocation
-  const long long b = blockIdx.z;
-  const int NK2 = 2 * NKS;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int* status = g.status;
-  if (warp == 0) {
-    tmem_alloc(&tmem_base, 512);
-    tmem_relinquish();
-  }
-  if (tid == 0) {
-    for (int s = 0; s < kWStages; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&mmad[s], 1);
-    }
-    fence_mbar_init();
-  }
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  const uint32_t tm = tmem_base;
-  const unsigned char* Abase =
-      reinterpret_cast<const unsigned char*>(g.Asl) + ((b * NIB + ib) * NKS) * (long long)kWAChunk;
-  const unsigned char* Xbase = reinterpret_cast<const unsigned char*>(g.Bsl) + ((b * NJB + jb) * NKS) * (long long)XC;
-  // step kk: half 0 takes (Ar | Ai for Im rows) with Br, half 1 (Ai negated | Ar) with Bi
-  auto load = [&](int kk, int st) {
-    const int half = kk >= NKS ? 1 : 0, ks = kk - half * NKS;
-    const int cA = imrow ? 1 - half : half;
-    unsigned char* dst = sm + st * SB;
-    mbar_arrive_expect_tx(&full[st], SB);
-    bulk_g2s(dst, Abase + (long long)ks * kWAChunk + (long long)cA * kWSA * PA, AB, &full[st]);
-    bulk_g2s(dst + AB, Xbase + (long long)ks * XC + (long long)half * SX * PX, XB, &full[st]);
-  };
-  bool ok = true;
-  if (tid == 0) {
-    const uint32_t s0 = smem_u32(sm);
-    for (int s = 0; s < kWStages && s < NK2; ++s) load(s, s);
-    for (int kk = 0; kk < NK2; ++kk) {
-      const int st = kk % kWStages;
-      if (!mbar_wait(&full[st], (uint32_t)(kk / kWStages) & 1u, kWaitNs, status)) { ok = false; break; }
-      fence_after_sync();
-      const int half = kk >= NKS ? 1 : 0;
-      panel_issue_step(tm, smem_desc(s0 + st * SB, 128, 256), smem_desc(s0 + st * SB + AB, 128, 256), !imrow && half,
-                       kk == 0);
-      mma_commit(&mmad[st]);
-      if (kk >= 1 && kk - 1 + kWStages < NK2) {
-        const int so = (kk - 1) % kWStages;
-        if (!mbar_wait(&mmad[so], (uint32_t)((kk - 1) / kWStages) & 1u, kWaitNs, status)) { ok = false; break; }
-        load(kk - 1 + kWStages, so);
-      }
-    }
-  }
-  const int last = NK2 - 1;
-  const bool done = ok && mbar_wait(&mmad[last % kWStages], (uint32_t)(last / kWStages) & 1u, kWaitNs, status);
-  ok = __syncthreads_and(done ? 1 : 0) != 0;
-  fence_after_sync();
-  if (!ok) {
-    if (tid == 0) atomicExch(status, 2);
-  } else {
-    const int i = ib * 128 + 32 * warp + lane;
-    const int ea = g.eA[b * g.M + i];
-    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-    double* stg = reinterpret_cast<double*>(sm) + warp * (32 * 17);
-    double* Cw = reinterpret_cast<double*>(g.C + b * g.c_ms + (long long)(ib * 128 + 32 * warp) * g.ldc) + (imrow ? 1 : 0);
-    const int* eBj = g.eB + b * g.Nc + jb * kWTN;
-    for (int c0 = 0; c0 < kWTN; c0 += 16) {
-      // this group's old C values and column exponents first: independent loads in flight
-      // while the accumulators are read (a load after each store would wait out its latency)
-      double cold[16];
-      int eb[16];
-      const int cc = lane & 15;
-#pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        const int rr = 2 * t + (lane >> 4);
-        cold[t] = g.accumulate ? Cw[2 * ((long long)rr * g.ldc + jb * kWTN + c0 + cc)] : 0.0;
-        eb[t] = eBj[c0 + t];
-      }
-      float v[128];  // accumulator q, column c at v[16 q + c]
-      tmem_ld16x4(tm + lane_base + (uint32_t)c0, kWTN, v);
-      tmem_ld16x4(tm + lane_base + (uint32_t)(4 * kWTN + c0), kWTN, v + 64);
-#pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        long long val = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) val += panel_units52(v[16 * q + c], q);
-        stg[lane * 17 + c] = i2d_scaled(val, ea + eb[c] - 52);
-      }
-      __syncwarp();
-#pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        const int rr = 2 * t + (lane >> 4);
-        const double pv = stg[rr * 17 + cc];
-        Cw[2 * ((long long)rr * g.ldc + jb * kWTN + c0 + cc)] = g.accumulate ? cold[t] - pv : pv;
-      }
-      __syncwarp();
-    }
-  }
-  fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tm, 512);
-}
-
-
 namespace {
 
 unsigned grid_for(long long n_thr) {
@@ -1218,7 +1160,7 @@ void panel_gemm(const WblkBuffers& w, const double2* A, long long a_ms, int lda,
     k_slice_panel_B<<<grid_for((long long)batch * K * Nc / 8), 256, 0, st>>>(B, b_ms, ldb, w.eB, w.Bsl, K, Nc,
                                                                               (long long)batch * K * Nc / 8);
   }
-  PanelGemmArgs g{};
+  OzProductArgs g{};
   g.Asl = w.Asl;
   g.Bsl = w.Bsl;
   g.eA = w.eA;
@@ -1235,8 +1177,8 @@ void panel_gemm(const WblkBuffers& w, const double2* A, long long a_ms, int lda,
   g.status = w.inner.status;
   {
     gw::TimedLaunch tl_("k_oz_panel_gemm", st);
-    k_oz_panel_gemm<<<dim3((unsigned)(Nc / kWTN), (unsigned)(2 * (M / 128)), (unsigned)batch), 128,
-                      w_residual_smem(kWSX1, kWLmax), st>>>(g);
+    k_oz_product<kWSX1, kWLmax, false, false><<<dim3((unsigned)(Nc / kWTN), (unsigned)(2 * (M / 128)), (unsigned)batch), kPT,
+                                         w_residual_smem(kWSX1, kWLmax), st>>>(g);
   }
 }
 
@@ -1258,7 +1200,7 @@ int wblk_block_size(int N) {
 
 cudaError_t wblk_setup(size_t smem_gj32_bs) {
   cudaError_t e = wtc_setup(smem_gj32_bs);
-  if (e == cudaSuccess) e = raise_smem_limit(k_oz_panel_gemm, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, false, false>, w_residual_smem(kWSX1, kWLmax));
   return e;
 }
 

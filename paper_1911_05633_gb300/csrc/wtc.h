@@ -64,17 +64,18 @@ struct WtcBuffers {
 cudaError_t wtc_setup(size_t smem_gj32);
 
 // ---- block Gauss-Jordan for N beyond kWNmax (kernels_wtc.cu) ----------------------
-// Arguments of k_oz_panel_gemm: C = A B (accumulate 0) or C -= A B (1) from the digits
-// of an M x K and a K x Nc panel (M a multiple of 128, Nc of kWTN, K of 16 and <= kWblkMaxK).
-struct PanelGemmArgs {
+// Arguments of k_oz_product: the digits of an M x K and a K x Nc matrix (M a multiple of
+// 128, Nc of kWTN, K of 16; for an FP64 result K <= kWblkMaxK or an even split of it).
+struct OzProductArgs {
   const uint16_t* Asl;
   const uint16_t* Bsl;
   const int* eA;
   const int* eB;
-  double2* C;
+  int M, Nc, K;
+  float2* R;       // residual I - A B [batch][M][Nc] in FP32, or
+  double2* C;      // C = A B (accumulate 0) or C -= A B (1)
   long long c_ms;  // matrix stride of C (elements)
   int ldc;         // row stride of C (elements)
-  int M, Nc, K;
   int skip0, skip1;  // 128-row blocks of C left alone
   int accumulate;
   int* status;
