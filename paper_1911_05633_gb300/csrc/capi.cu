@@ -19,6 +19,7 @@
 #include "contract.h"
 #include "wtc.h"
 #include "oz.h"
+#include "chain.h"
 #include "ktimer.h"
 #include "dyson.h"
 #include "gj.h"
@@ -96,6 +97,7 @@ struct gw_plan_s {
   gw::OzSigma oz;
   gw::OzTransform ozt;  // FP64-accurate structured transforms on the tensor cores
   gw::OzPol ozp;        // FP64-accurate stage 3 of P on the tensor cores
+  gw::ChainPlan chain;  // FP64 P and Sigma over symmetric pairs (in place of oz and ozp when it fits)
   gw::KernelTimer timer;  // optional per-kernel event timing (gw_timing_*)
   gw::DysonPlan dyson;    // Eq. G_1 scratch, allocated by the first Dyson call
 };
@@ -165,6 +167,7 @@ void free_device(gw_plan_s* p) {
   gw::oz_sigma_free(p->oz);
   gw::oz_transform_free(p->ozt);
   gw::oz_pol_free(p->ozp);
+  gw::chain_free(p->chain);
   gw::dyson_free(p->dyson);
 }
 
@@ -403,6 +406,10 @@ static gw_status alloc_w_scratch(gw_plan_s* p) {
 
 // The FP64 digit-GEMM scratch of the Sigma stage W~ C^b and of the P stage Y C^b.
 static gw_status alloc_oz_sigma(gw_plan_s* p) {
+  if (p->chain.ok) {
+    p->oz_pending = false;
+    return gw::chain_alloc_s(p->chain, p->h, (size_t)4 << 30);
+  }
   const gw_status st = gw::oz_sigma_init(p->oz, p->h, (size_t)4 << 30);
   p->oz_pending = false;
   if (st != GW_OK) return st;
@@ -411,6 +418,10 @@ static gw_status alloc_oz_sigma(gw_plan_s* p) {
   return GW_OK;
 }
 static gw_status alloc_oz_pol(gw_plan_s* p) {
+  if (p->chain.ok) {
+    p->ozp_pending = false;
+    return gw::chain_alloc_p(p->chain, p->h, (size_t)4 << 30);
+  }
   const gw_status st = gw::oz_pol_init(p->ozp, p->h, (size_t)4 << 30);
   p->ozp_pending = false;
   if (st == GW_OK && gw::uploads_landed() != cudaSuccess) return GW_ERR_CUDA;
@@ -595,6 +606,7 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
     if ((st = upload(&p->d_counter, nullptr, 16)) != GW_OK) return fail(st);
     gw::set_last_error("");
   }
+  if (!(opt && opt->fp64_products == 1) && (st = gw::chain_init(p->chain, h)) != GW_OK) return fail(st);
   if (p->sigma_tensor) {
     if (defer) p->oz_pending = true;
     else if ((st = alloc_oz_sigma(p)) != GW_OK) return fail(st);
@@ -652,7 +664,7 @@ gw_status gw_plan_query(gw_plan_t p, gw_plan_info* info) {
   info->w_tensor = p->w_tensor ? 1 : 0;
   info->w_block = p->w_bs;
   info->sigma_tensor = p->sigma_tensor ? 1 : 0;
-  info->p_tensor = (p->ozp.ready || p->ozp_pending) ? 1 : 0;  // pending: planned at the first call
+  info->p_tensor = (p->ozp.ready || p->ozp_pending || p->chain.ok) ? 1 : 0;  // pending: planned at the first call
   info->mixed_queue = (p->contract_p ? 1 : 0) | (p->contract_s ? 2 : 0);
   info->transform_tensor = (p->ozt.ready_w ? 1 : 0) | (p->ozt.ready_p ? 2 : 0);
   info->n_q_solved = p->n_qh;
@@ -849,6 +861,8 @@ gw_status gw_polarizability_tau(gw_plan_t p, const void* G_R, void* P_R, gw_prec
   g.mirror_tau = h.c_symmetric;
   const int nt_eff = h.c_symmetric ? (h.n_tau + 1) / 2 : h.n_tau;
   if (p->ozp_pending && (st = alloc_oz_pol(p)) != GW_OK) return st;
+  if (p->chain.p_ready)
+    return gw::chain_polarizability(p->chain, h, p->d_ent, (const double2*)G_R, (double2*)P_R, p->d_status, S(stream));
   if (p->ozp.ready) {
     // stages 1 and 2 in FP64 (Y to the pass buffer), stage 3 on the tensor cores, per pass
     for (int s0 = 0; s0 < nt_eff; s0 += p->ozp.tau_c) {
@@ -908,7 +922,11 @@ gw_status gw_self_energy_tau(gw_plan_t p, const void* G_R, const void* Wt_R, con
     g.out_n_slices = h.n_tau;
     g.sign = -1.0;
     if (p->oz_pending && (st = alloc_oz_sigma(p)) != GW_OK) return st;
-    if (p->sigma_tensor) {
+    if (p->chain.s_ready) {
+      if ((st = gw::chain_self_energy(p->chain, h, p->d_ent, (const double2*)G_R, (const double2*)Wt_R, h.n_tau, -1, -1.0,
+                                      (double2*)Sig_R, p->d_status, S(stream))) != GW_OK)
+        return st;
+    } else if (p->sigma_tensor) {
       // stage A (W~ C^b) on the tensor cores per pass of tau slices, stages B and C in FP64
       for (int s0 = 0; s0 < h.n_tau; s0 += p->oz.tau_c) {
         const int te = std::min(p->oz.tau_c, h.n_tau - s0);
@@ -949,6 +967,10 @@ gw_status gw_self_energy_tau(gw_plan_t p, const void* G_R, const void* Wt_R, con
     b.s[0].sign = +1.0;
     return gw::contract_launch(true, p->cfgS, b, p->d_unitsX, p->n_unitsX, p->d_counter, p->d_status, S(stream));
   }
+  if (v_R && Sigx_R && prec == GW_FP64 && p->chain.s_ready)
+    // exchange: W~ -> v, G(tau) -> -G(beta-), one slice
+    return gw::chain_self_energy(p->chain, h, p->d_ent, (const double2*)G_R, (const double2*)v_R, 1, h.n_tau - 1, 1.0,
+                                 (double2*)Sigx_R, p->d_status, S(stream));
   if (v_R && Sigx_R) {
     // exchange: W~ -> v, G(tau) -> -G(beta-): +C G(beta-) v C in FP64
     gw::ContractArgs g{};
