@@ -108,9 +108,11 @@ typedef struct {
   size_t workspace_bytes; /* cap on the W-solve scratch (0: 24 GiB for the tensor-core and the block
                              inverse, 4 GiB otherwise) */
   int no_symmetry;        /* 1: never use the frequency / momentum symmetries in the W solve */
-  int w_solver;           /* 0: automatic (tensor-core inverse when N_PB is 128, 256 or 384;
-                             block Gauss-Jordan over pivot blocks of 384, 256 or 128 that the
-                             tensor-core inverse takes when N_PB is a larger multiple of 128),
+  int w_solver;           /* 0: automatic (tensor-core inverse when N_PB is 128, 256 or 384, and for
+                             other orders from 88 to 383 beside an identity, while the scratch
+                             cap holds one frequency; block Gauss-Jordan over pivot blocks of
+                             384, 256 or 128 that the tensor-core inverse takes when N_PB is a
+                             larger multiple of 128),
                              1: FP64 Gauss-Jordan inverse always */
   int fp64_products;      /* 0 automatic: FP64-accurate digit products on the tensor cores for
                              the W~ C^b stage of the GW_FP64 Sigma (every K <= 384), the Y C^b
@@ -144,7 +146,7 @@ typedef struct {
   double cond_boson;
   int w_symmetric;            /* the W solve runs on nu >= 0 and half of the q mesh (see gw_screened_W_iw) */
   int n_q_solved;             /* momenta solved per frequency */
-  int w_tensor;               /* inverses by FP32 Gauss-Jordan + two tensor-core refinements */
+  int w_tensor;               /* inverses of order N_PB by FP32 Gauss-Jordan + two tensor-core refinements */
   int sigma_tensor;           /* GW_FP64 Sigma: stage W~ C^b by FP64-accurate tensor-core products */
   int p_tensor;               /* GW_FP64 P: stage Y C^b by FP64-accurate tensor-core products (device plans) */
   int transform_tensor;       /* bit 0: GW_IN_REAL bosonic i nu -> tau, bit 1: GW_IN_MIRROR bosonic

@@ -76,6 +76,11 @@ struct gw_plan_s {
   // block Gauss-Jordan for N_PB beyond the tensor-core inverse (pivot blocks of w_bs,
   // each inverted by the tensor-core inverse; the t_* buffers above sized for them)
   bool w_block = false;
+  int w_np = 0;       // order of the matrices solved: N_PB, or (w_pad) the multiple of 128 above it
+  bool w_pad = false;
+  int* t_weak = nullptr;       // [nu_chunk * n_qh] with w_pad: matrices left to the FP64 inverse
+  unsigned* t_rmax = nullptr;  // largest residuals
+  int* t_act = nullptr;        // matrices refined once more
   int w_bs = 0;
   double2* b_D = nullptr;
   double2* b_Rp = nullptr;
@@ -130,6 +135,19 @@ struct DeviceGuard {
   }
 };
 
+// Orders N_PB that the tensor-core inverse takes beside an identity, and the refinements there:
+// the third and, where it is needed, the fourth have residuals to nine digits, for the error
+// of an FP64 elimination or less.  The line: 196 matrices in two batches, W solve of N = 80 2.34 ms
+// against 1.82 by the FP64 inverse in shared memory, N = 96 2.39 against 3.18, 120 2.55 against
+// 9.33, 136 (in 256) 8.34 against 13.2, 200 8.79 against 34.2, 288 (in 384) 21.8 against 83.7.
+constexpr int kPadMinN = 88;
+constexpr int kPadRefinements = 4;
+// Scratch of the tensor-core inverse per matrix element: three FP32 arrays, the digit planes
+// of both operands and the term planes of X0.
+constexpr size_t w_tensor_bytes_per_element(bool pad) {
+  return 3 * sizeof(float2) + 2 * (pad ? 2 * gw::kWFine : gw::kWSA + gw::kWSX1) * 2 + 6 * 2;
+}
+
 gw_status cuda_fail(cudaError_t e, const char* what) {
   set_last_error(std::string(what) + ": " + cudaGetErrorString(e));
   return GW_ERR_CUDA;
@@ -159,7 +177,7 @@ void free_device(gw_plan_s* p) {
                   p->d_C, p->d_Tf_fwd, p->d_Tf_inv, p->d_Tb_fwd, p->d_Tb_mirror, p->d_Tb_inv, p->d_qh, p->d_qw,
                   p->d_numirror, p->d_wsV, p->d_wsA, p->d_perm, p->d_status, p->t_X32, p->t_lo, p->t_R, p->t_PX, p->t_Asl,
                   p->t_Xsl, p->t_eA, p->t_eX, p->d_unitsP, p->d_unitsS, p->d_unitsX, p->d_counter,
-                  p->b_D, p->b_Rp, p->b_Asl, p->b_Bsl, p->b_eA, p->b_eB};
+                  p->t_weak, p->t_rmax, p->t_act, p->b_D, p->b_Rp, p->b_Asl, p->b_Bsl, p->b_eA, p->b_eB};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   gw::mixed_free(p->mixed);
@@ -208,7 +226,7 @@ gw_status launch_gather(gw_plan_s* p, gw_block kind, int n_slices, const double2
                         long long s_stride, const double2* F_sub, long long sub_k_stride, long long sub_s_stride,
                         double2* F_R, int out_n_slices, int out_slice0, double scale, cudaStream_t st,
                         const int* k_list = nullptr, const double* k_weight = nullptr, int n_k_in = -1,
-                        int real_only = 0) {
+                        int real_only = 0, int ld = 0) {
   gw::GatherArgs g{};
   g.ent = p->d_ent;
   g.pair_start = p->d_pair_start;
@@ -224,7 +242,8 @@ gw_status launch_gather(gw_plan_s* p, gw_block kind, int n_slices, const double2
   g.F_k = F_k;
   g.k_stride = k_stride;
   g.s_stride = s_stride;
-  g.ld = dense_n(p, kind);
+  g.cols = dense_n(p, kind);
+  g.ld = ld ? ld : g.cols;
   g.pb = kind == GW_BLOCK_PB;
   g.row_off = kind == GW_BLOCK_PB ? p->d_pb_off : p->d_orb_off;
   g.F_sub = F_sub;
@@ -245,7 +264,7 @@ gw_status launch_gather(gw_plan_s* p, gw_block kind, int n_slices, const double2
 gw_status launch_scatter(gw_plan_s* p, gw_block kind, int n_slices, const double2* F_R, int in_n_slices,
                          int in_slice0, double2* F_k, long long k_stride, long long s_stride, cudaStream_t st,
                          const int* k_list = nullptr, int n_k_out = -1, const double2* base = nullptr,
-                         double coef = 1.0, bool real_in = false) {
+                         double coef = 1.0, bool real_in = false, int ld = 0) {
   gw::ScatterArgs g{};
   g.real_in = real_in ? 1 : 0;
   g.ent = p->d_ent;
@@ -267,7 +286,8 @@ gw_status launch_scatter(gw_plan_s* p, gw_block kind, int n_slices, const double
   g.F_k = F_k;
   g.k_stride = k_stride;
   g.s_stride = s_stride;
-  g.ld = dense_n(p, kind);
+  g.cols = dense_n(p, kind);
+  g.ld = ld ? ld : g.cols;
   dim3 grid(p->h.n_atoms, n_slices, band_splits(p, kind, n_slices));
   {
     gw::TimedLaunch tl_("k_scatter_R_to_k", st);
@@ -294,7 +314,13 @@ gw_status launch_tensor_inverse(gw_plan_s* p, double2* mats, int batch, long lon
   w.eA = p->t_eA;
   w.eX = p->t_eX;
   w.status = p->d_status;
-  gw::wtc_inverse(w, mats, batch, (int)N, p->smem_GJ32, st);
+  if (p->w_pad) {
+    w.weak = p->t_weak;
+    w.rmax = p->t_rmax;
+    w.act = p->t_act;
+    w.perm = p->d_perm;
+  }
+  gw::wtc_inverse(w, mats, batch, (int)N, p->smem_GJ32, st, p->w_pad ? kPadRefinements : 2);
   return check_launch("tensor-core inverse");
 }
 
@@ -345,7 +371,7 @@ size_t smem_sigma(const gw::HostPlan& h) {
 // sized to the cap, plus the tensor-core inverse's planes.
 static gw_status alloc_w_scratch(gw_plan_s* p) {
   const gw::HostPlan& h = p->h;
-  const size_t npb = (size_t)h.n_pb_total();
+  const size_t npb = (size_t)p->w_np;
   const size_t mat = npb * npb * sizeof(double2);
   // bytes per inverted matrix: FP64 matrix, pivots, and (tensor path) the FP32 inverse,
   // its correction and the residual, the BF16 digit planes of both operands, the term
@@ -353,7 +379,7 @@ static gw_status alloc_w_scratch(gw_plan_s* p) {
   // the tensor-core inverse's scratch per inverted matrix of order ni (the matrix itself,
   // or the pivot block of the block Gauss-Jordan)
   const size_t ni = p->w_block ? (size_t)p->w_bs : npb;
-  const size_t tc_per = ni * ni * (3 * sizeof(float2) + 2 * (gw::kWSA + gw::kWSX1) * 2 + 6 * 2) + 2 * ni * sizeof(int);
+  const size_t tc_per = ni * ni * w_tensor_bytes_per_element(p->w_pad) + 2 * ni * sizeof(int);
   // block Gauss-Jordan: the pivot block, the row panel, the digits of a column and a row
   // panel (2 kWSA, 2 kWSX1 BF16 planes per element) and 2 npb exponents
   const size_t bs = (size_t)p->w_bs;
@@ -386,10 +412,15 @@ static gw_status alloc_w_scratch(gw_plan_s* p) {
     if ((st = up((void**)&p->t_lo, nm * ni * ni * sizeof(float2))) != GW_OK) return st;
     if ((st = up((void**)&p->t_R, nm * ni * ni * sizeof(float2))) != GW_OK) return st;
     if ((st = up((void**)&p->t_PX, nm * ni * ni * 6 * 2)) != GW_OK) return st;
-    if ((st = up((void**)&p->t_Asl, nm * ni * ni * 2 * gw::kWSA * 2)) != GW_OK) return st;
-    if ((st = up((void**)&p->t_Xsl, nm * ni * ni * 2 * gw::kWSX1 * 2)) != GW_OK) return st;
+    if ((st = up((void**)&p->t_Asl, nm * ni * ni * 2 * (p->w_pad ? gw::kWFine : gw::kWSA) * 2)) != GW_OK) return st;
+    if ((st = up((void**)&p->t_Xsl, nm * ni * ni * 2 * (p->w_pad ? gw::kWFine : gw::kWSX1) * 2)) != GW_OK) return st;
     if ((st = up((void**)&p->t_eA, nm * ni * sizeof(int))) != GW_OK) return st;
     if ((st = up((void**)&p->t_eX, nm * ni * sizeof(int))) != GW_OK) return st;
+    if (p->w_pad) {
+      if ((st = up((void**)&p->t_weak, nm * sizeof(int))) != GW_OK) return st;
+      if ((st = up((void**)&p->t_rmax, nm * sizeof(unsigned))) != GW_OK) return st;
+      if ((st = up((void**)&p->t_act, nm * sizeof(int))) != GW_OK) return st;
+    }
   }
   if (p->w_block) {
     const size_t nm = (size_t)nch * p->n_qh;
@@ -504,6 +535,17 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
     // beyond it: block Gauss-Jordan over pivot blocks that the tensor-core inverse takes
     p->w_bs = !(opt && opt->w_solver == 1) && !p->w_tensor ? gw::wblk_block_size((int)n) : 0;
     p->w_block = p->w_bs > 0;
+    p->w_np = (int)n;
+    if (!(opt && opt->w_solver == 1) && n % 128 != 0 && n >= (size_t)kPadMinN && n < (size_t)gw::kWNmax) {
+      // any other order up to 384: beside an identity in the next multiple of 128, unless the
+      // scratch of one frequency is more than the caller's cap
+      const size_t np = (n + 127) / 128 * 128;
+      const size_t cap = opt && opt->workspace_bytes ? opt->workspace_bytes : (size_t)4 << 30;
+      if (p->n_qh * np * np * (2 * sizeof(double2) + w_tensor_bytes_per_element(true)) <= cap) {
+        p->w_tensor = p->w_pad = true;
+        p->w_np = (int)np;
+      }
+    }
     bool k_ok = true;  // the tensor-core Sigma stage sums levels 0-4 exactly for K_b <= 384
     for (int s = 0; s < hh.n_species; ++s) k_ok = k_ok && hh.n_prod[s] <= 16 * gw::kOzMaxKS;
     p->sigma_tensor = !(opt && opt->fp64_products == 1) && k_ok;
@@ -559,9 +601,10 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
   if ((st = upload(&p->d_qw, qw.data(), qw.size() * sizeof(double))) != GW_OK) return fail(st);
   if ((st = upload(&p->d_numirror, numirror.data(), numirror.size() * sizeof(int))) != GW_OK) return fail(st);
   p->ws_cap = (opt && opt->workspace_bytes) ? opt->workspace_bytes
-                                            : (p->w_tensor || p->w_block ? ((size_t)24 << 30) : ((size_t)4 << 30));
+                                            : ((p->w_tensor && !p->w_pad) || p->w_block ? ((size_t)24 << 30)
+                                                                                        : ((size_t)4 << 30));
   if (p->w_tensor || p->w_block) {
-    p->smem_GJ32 = gw::gj32_smem(p->w_block ? p->w_bs : (int)npb);
+    p->smem_GJ32 = gw::gj32_smem(p->w_block ? p->w_bs : p->w_np);
     if ((p->w_block ? gw::wblk_setup(p->smem_GJ32) : gw::wtc_setup(p->smem_GJ32)) != cudaSuccess) {
       cudaError_t e = cudaGetLastError();
       set_last_error(std::string("cudaFuncSetAttribute (tensor W): ") + cudaGetErrorString(e));
@@ -583,7 +626,7 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
   if (gw::raise_smem_limit(gw::k_polarizability_fp64, (int)p->smem_P) != cudaSuccess ||
       gw::raise_smem_limit(gw::k_self_energy_fp64, (int)p->smem_S) != cudaSuccess ||
       gw::raise_smem_limit(gw::k_transform, (int)p->smem_T) != cudaSuccess ||
-      gw::gj_setup((int)npb) != cudaSuccess) {
+      gw::gj_setup((int)npb) != cudaSuccess || (p->w_pad && gw::gj_only_setup(p->w_np) != cudaSuccess)) {
     cudaError_t e = cudaGetLastError();
     set_last_error(std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
     return fail(GW_ERR_UNSUPPORTED);
@@ -661,7 +704,7 @@ gw_status gw_plan_query(gw_plan_t p, gw_plan_info* info) {
   info->cond_fermion = h.cond_f;
   info->cond_boson = h.cond_b;
   info->w_symmetric = p->w_sym ? 1 : 0;
-  info->w_tensor = p->w_tensor ? 1 : 0;
+  info->w_tensor = p->w_tensor && !p->w_pad ? 1 : 0;
   info->w_block = p->w_bs;
   info->sigma_tensor = p->sigma_tensor ? 1 : 0;
   info->p_tensor = (p->ozp.ready || p->ozp_pending || p->chain.ok) ? 1 : 0;  // pending: planned at the first call
@@ -1005,7 +1048,7 @@ gw_status gw_screened_W_iw(gw_plan_t p, const void* P_R_iw, const void* v_q, voi
   cudaStream_t s = S(stream);
   if (p->w_pending && (st = alloc_w_scratch(p)) != GW_OK) return st;
   const long long N = h.n_pb_total();
-  const long long NN = N * N;
+  const long long Np = p->w_np, NN = Np * Np;  // the matrices solved (N beside an identity when Np > N)
   const int nq = p->n_qh;
   const double2* v = (const double2*)v_q;
   // v(q)^{-1} for the solved momenta
@@ -1013,10 +1056,10 @@ gw_status gw_screened_W_iw(gw_plan_t p, const void* P_R_iw, const void* v_q, voi
     dim3 g((unsigned)std::min<long long>((NN + 255) / 256, 1024), (unsigned)nq);
     {
       gw::TimedLaunch tl_("k_copy_mats", s);
-      gw::k_copy_mats<<<g, 256, 0, s>>>(v, p->d_qh, p->d_wsV, NN);
+      gw::k_copy_mats<<<g, 256, 0, s>>>(v, p->d_qh, p->d_wsV, (int)N, (int)Np);
     }
     if ((st = check_launch("k_copy_mats")) != GW_OK) return st;
-    if (p->w_tensor) st = launch_tensor_inverse(p, p->d_wsV, nq, N, s);
+    if (p->w_tensor) st = launch_tensor_inverse(p, p->d_wsV, nq, Np, s);
     else if (p->w_block) st = launch_block_inverse(p, p->d_wsV, nq, N, s);
     else st = launch_gj(p, p->d_wsV, nq, N, s);
     if (st != GW_OK) return st;
@@ -1028,17 +1071,21 @@ gw_status gw_screened_W_iw(gw_plan_t p, const void* P_R_iw, const void* v_q, voi
     // A = v(q)^{-1} - P(q, nu) for the chunk, [nu][q][N][N]
     // symmetric mode: P(R, i nu) is real (the imaginary parts are not read)
     if ((st = launch_scatter(p, GW_BLOCK_PB, nc, (const double2*)P_R_iw, h.n_nu, slot0, p->d_wsA, NN,
-                             (long long)nq * NN, s, p->d_qh, nq, p->d_wsV, -1.0, p->w_sym)) != GW_OK)
+                             (long long)nq * NN, s, p->d_qh, nq, p->d_wsV, -1.0, p->w_sym, (int)Np)) != GW_OK)
       return st;
-    if (p->w_tensor) st = launch_tensor_inverse(p, p->d_wsA, nc * nq, N, s);
+    if (p->w_pad) {
+      gw::TimedLaunch tl_("k_pad_identity", s);
+      gw::k_pad_identity<<<dim3((unsigned)((Np + 31) / 32), (unsigned)(nc * nq)), 256, 0, s>>>(p->d_wsA, (int)N, (int)Np);
+    }
+    if (p->w_tensor) st = launch_tensor_inverse(p, p->d_wsA, nc * nq, Np, s);
     else if (p->w_block) st = launch_block_inverse(p, p->d_wsA, nc * nq, N, s);
     else st = launch_gj(p, p->d_wsA, nc * nq, N, s);
     if (st != GW_OK) return st;
     // W~(R) = (1/N_k) sum_q e^{-iqR} (W(q) - v(q)); in symmetric mode the sum runs over
     // one momentum of each (q, -q) pair with weight 2 and keeps the (exactly real) real part
-    if ((st = launch_gather(p, GW_BLOCK_PB, nc, p->d_wsA, NN, (long long)nq * NN, v, NN, 0, (double2*)Wt_R_iw,
+    if ((st = launch_gather(p, GW_BLOCK_PB, nc, p->d_wsA, NN, (long long)nq * NN, v, N * N, 0, (double2*)Wt_R_iw,
                             h.n_nu, slot0, 1.0 / h.n_k, s, p->d_qh, p->w_sym ? p->d_qw : nullptr, nq,
-                            p->w_sym ? 1 : 0)) != GW_OK)
+                            p->w_sym ? 1 : 0, (int)Np)) != GW_OK)
       return st;
   }
   if (p->w_sym && p->n_neg > 0) {
@@ -1359,7 +1406,7 @@ extern "C" gw_status gw_screened_W_iw_noalloc(gw_plan_t p, const void* P_R_iw, c
     for (int b2 = 0; b2 < h.n_species; ++b2) maxblk = std::max(maxblk, h.n_prod[a] * h.n_prod[b2]);
   for (size_t qi = 0; qi < qh.size(); ++qi) {
     dim3 gc((unsigned)std::min<long long>((NN + 255) / 256, 1024), 1);
-    gw::k_copy_mats<<<gc, 256, 0, s>>>(v, p->d_qh + qi, vinv, NN);
+    gw::k_copy_mats<<<gc, 256, 0, s>>>(v, p->d_qh + qi, vinv, (int)N, (int)N);
     if ((st = check_launch("k_copy_mats")) != GW_OK) return st;
     gw::gj_batch(vinv, perm, 1, (int)N, NN, p->d_status, s);
     if ((st = check_launch("k_gj_inverse")) != GW_OK) return st;

@@ -17,6 +17,10 @@ cudaError_t gj_setup(int N);
 // kGJSmemMax).  A zero pivot sets *status.
 void gj_batch(double2* mats, int* perm, int batch, int N, long long stride, int* status, cudaStream_t st);
 
+// The panel form on the matrices with only[b] != 0 (N up to 430; the others are not touched).
+cudaError_t gj_only_setup(int N);
+void gj_batch_only(double2* mats, int* perm, int batch, int N, int* status, const int* only, cudaStream_t st);
+
 cudaError_t hess_setup(int N);
 // out[b] = Hessenberg form of i w_n - H(k) - Sx(k) - Sc(k, n), b = k n_w + n (Sx, Sc may be
 // null); scale[b]: the largest |re| + |im| of the matrix.

@@ -29,7 +29,8 @@ struct GatherArgs {
   int real_only;           // keep the real part of the result
   const double2* F_k;      // dense input
   long long k_stride, s_stride;
-  int ld;
+  int ld;                  // row stride of F_k
+  int cols;                // columns of the dense matrix (<= ld)
   int pb;                  // 1: product-basis blocks, 0: orbital blocks
   const int* row_off;      // [n_atoms + 1] orbital or product offsets (the full pair block)
   const double2* F_sub;    // optional dense input subtracted from F_k
@@ -58,7 +59,8 @@ struct ScatterArgs {
   int pb;
   double2* F_k;            // dense output
   long long k_stride, s_stride;
-  int ld;
+  int ld;                  // row stride of F_k
+  int cols;                // columns of the dense matrix (<= ld)
 };
 
 struct TransformArgs {
@@ -107,11 +109,14 @@ __global__ void k_self_energy_fp64(ContractArgs g);
 __global__ void k_gj_inverse(double2* __restrict__ A, int* __restrict__ perm, int N, long long mat_stride,
                              int* status);
 constexpr int kGJB = 16;  // panel width of the blocked Gauss-Jordan inverse
+// `only` (or null): matrices b with only[b] == 0 are left alone.
 __global__ void k_gj_inverse_blocked(double2* __restrict__ A, int* __restrict__ perm, int N, long long mat_stride,
-                                     int* status);
-// dst[b] = src[map[b]] for dense N x N matrices (used to stage v(q) before inversion).
+                                     int* status, const int* __restrict__ only);
+// dst[b] = src[map[b]] for dense N x N matrices, beside an identity in Np x Np (used to stage
+// v(q) before inversion).
 __global__ void k_copy_mats(const double2* __restrict__ src, const int* __restrict__ map, double2* __restrict__ dst,
-                            long long NN);
+                            int N, int Np);
+__global__ void k_pad_identity(double2* __restrict__ mats, int N, int Np);
 // W~(R, -nu_j) = W~(mirror(R), nu_{mirror j})^T for the negative frequencies (real blocks).
 __global__ void k_mirror_nu(const DevEntry* __restrict__ ent, const int* __restrict__ nu_mirror, int n_neg, int n_nu,
                             double2* __restrict__ W);

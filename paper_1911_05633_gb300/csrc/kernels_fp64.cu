@@ -56,21 +56,21 @@ __global__ void k_gather_k_to_R(GatherArgs g) {
   const int a = blockIdx.x, s = blockIdx.y;
   const int ro = g.row_off[a];
   const int rows = g.row_off[a + 1] - ro;
-  const int n_el = rows * g.ld;
+  const int n_el = rows * g.cols;
   const bool hold = g.n_k_in <= kHoldK;
   for (int x = threadIdx.x + blockIdx.z * blockDim.x; x < n_el; x += blockDim.x * gridDim.z) {
-    const int i = x / g.ld, col = x - i * g.ld;
+    const int i = x / g.cols, col = x - i * g.cols;
     const int b = g.col_atom[col];
     const int j = col - g.row_off[b];
     const int p = a * g.n_atoms + b;
     const int e0 = g.pair_start[p], e1 = g.pair_start[p + 1];
     if (e0 == e1) continue;
-    const long long in_el = (long long)(ro + i) * g.ld + col;
+    const long long in_el = (long long)(ro + i) * g.ld + col, sub_el = (long long)(ro + i) * g.cols + col;
     auto value = [&](int kk) -> double2 {
       const int k = g.k_list ? g.k_list[kk] : kk;
       double2 v = g.F_k[(long long)kk * g.k_stride + (long long)s * g.s_stride + in_el];
       if (g.F_sub) {
-        const double2 w = g.F_sub[(long long)k * g.sub_k_stride + (long long)s * g.sub_s_stride + in_el];
+        const double2 w = g.F_sub[(long long)k * g.sub_k_stride + (long long)s * g.sub_s_stride + sub_el];
         v.x -= w.x;
         v.y -= w.y;
       }
@@ -193,10 +193,10 @@ __global__ void k_scatter_R_to_k(ScatterArgs g) {
   const int a = blockIdx.x, s = blockIdx.y;
   const int ro = g.row_off[a];
   const int rows = g.row_off[a + 1] - ro;
-  const int n_el = rows * g.ld;
+  const int n_el = rows * g.cols;
   const bool hold = g.n_k_out <= kHoldK;
   for (int x = threadIdx.x + blockIdx.z * blockDim.x; x < n_el; x += blockDim.x * gridDim.z) {
-    const int i = x / g.ld, col = x - i * g.ld;
+    const int i = x / g.cols, col = x - i * g.cols;
     const int b = g.col_atom[col];
     const int j = col - g.row_off[b];
     const int p = a * g.n_atoms + b;
@@ -576,7 +576,8 @@ __global__ void k_gj_inverse(double2* __restrict__ A, int* __restrict__ perm, in
 // once per panel instead of once per column.  Requires 2 N kGJB complex values of
 // shared memory (N <= 430).
 __global__ void k_gj_inverse_blocked(double2* __restrict__ A, int* __restrict__ perm, int N, long long mat_stride,
-                                     int* status) {
+                                     int* status, const int* __restrict__ only) {
+  if (only && !only[blockIdx.x]) return;
   extern __shared__ unsigned char smraw[];
   double2* Pan = reinterpret_cast<double2*>(smraw);  // [N][kGJB] panel columns
   double2* Prow = Pan + (size_t)N * kGJB;            // [kGJB][N] pivot rows (pre-update)
@@ -708,12 +709,25 @@ __global__ void k_gj_inverse_blocked(double2* __restrict__ A, int* __restrict__ 
 }
 
 __global__ void k_copy_mats(const double2* __restrict__ src, const int* __restrict__ map, double2* __restrict__ dst,
-                            long long NN) {
+                            int N, int Np) {
   const int b = blockIdx.y;
-  const double2* s = src + (long long)map[b] * NN;
+  const long long NN = (long long)Np * Np;
+  const double2* s = src + (long long)map[b] * N * N;
   double2* d = dst + (long long)b * NN;
-  for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < NN; x += (long long)gridDim.x * blockDim.x)
-    d[x] = s[x];
+  for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < NN; x += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(x / Np), j = (int)(x - (x / Np) * Np);
+    d[x] = i < N && j < N ? s[(long long)i * N + j] : make_double2(i == j ? 1.0 : 0.0, 0.0);
+  }
+}
+
+// The rows and columns N .. Np - 1 of every Np x Np matrix: those of the identity, so that
+// the inverse is the N x N one beside an identity.  One block per matrix and 32 rows.
+__global__ void k_pad_identity(double2* __restrict__ mats, int N, int Np) {
+  double2* d = mats + (long long)blockIdx.y * Np * Np;
+  const int i0 = blockIdx.x * 32, i1 = min(Np, i0 + 32);
+  for (int i = i0 + (threadIdx.x >> 5); i < i1; i += blockDim.x >> 5)
+    for (int j = (i < N ? N : 0) + (threadIdx.x & 31); j < Np; j += 32)
+      d[(long long)i * Np + j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
 }
 
 // One block per (entry, negative-frequency slot j): copy the transposed block of the

@@ -413,7 +413,7 @@ void gj_batch(double2* mats, int* perm, int batch, int N, long long stride, int*
     k_gj_inverse_smem<<<batch, kT, gj_smem_bytes(N), st>>>(mats, N, stride, status);
   } else if (gj_is_blocked(N)) {
     TimedLaunch tl_("k_gj_inverse_blocked", st);
-    k_gj_inverse_blocked<<<batch, 512, gj_blocked_bytes(N), st>>>(mats, perm, N, stride, status);
+    k_gj_inverse_blocked<<<batch, 512, gj_blocked_bytes(N), st>>>(mats, perm, N, stride, status, nullptr);
   } else {
     TimedLaunch tl_("k_gj_inverse", st);
     k_gj_inverse<<<batch, 512, 2 * (size_t)N * sizeof(double2), st>>>(mats, perm, N, stride, status);
@@ -446,5 +446,11 @@ void hess_trace(const double2* Hs, const double* scale, double mu, int N, long l
   k_hess_trace<kTraceG><<<(unsigned)((n_b + kTracePer - 1) / kTracePer), kTraceThreads,
                           (size_t)kTracePer * trace_stride(N) * sizeof(double2), st>>>(Hs, scale, mu, N, n_b, tiny, tr, flag);
 }
+
+void gj_batch_only(double2* mats, int* perm, int batch, int N, int* status, const int* only, cudaStream_t st) {
+  TimedLaunch tl_("k_gj_inverse_blocked<only>", st);
+  k_gj_inverse_blocked<<<batch, 512, gj_blocked_bytes(N), st>>>(mats, perm, N, (long long)N * N, status, only);
+}
+cudaError_t gj_only_setup(int N) { return raise_smem_limit(k_gj_inverse_blocked, gj_blocked_bytes(N)); }
 
 }  // namespace gw

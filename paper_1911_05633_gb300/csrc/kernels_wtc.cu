@@ -13,6 +13,7 @@
 #include "umma.h"
 #include "fpbits.h"
 #include "ozaki.h"
+#include "gj.h"
 #include "wtc.h"
 #include "ktimer.h"
 
@@ -37,7 +38,8 @@ __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
 // update), run per chunk of kGJ32C columns with 8 x 4 complex register blocks per
 // thread.  At the end the columns are permuted back by the composite of the pivot swaps.
 __global__ void __launch_bounds__(512, 1)
-k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __restrict__ status) {
+k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __restrict__ status,
+                 int* __restrict__ weak) {
   constexpr int B = kGJ32B, C = kGJ32C;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* Pan = reinterpret_cast<float2*>(smraw);  // [N][B]
@@ -89,7 +91,7 @@ k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __res
       const int p = bi < N ? bi : k;
       if (tid == 0) {
         pm[k] = p;
-        if (!(best > 0.0f)) atomicExch(status, 1);
+        if (!(best > 0.0f)) atomicExch(weak ? weak + blockIdx.x : status, 1);
       }
       // lane j holds column j of the pivot row (scaled) and of the old row k
       const float2 d = Pan[p * B + m];
@@ -226,8 +228,11 @@ constexpr uint64_t kWaitNs = 500ull * 1000ull * 1000ull;
 
 }  // namespace
 
-__global__ void k_to_f32(const double2* __restrict__ src, float2* __restrict__ dst, long long n) {
+// `act` (or null), here and below: matrices b with act[b] == 0 are left out (NN elements each).
+__global__ void k_to_f32(const double2* __restrict__ src, float2* __restrict__ dst, long long n, long long NN,
+                         const int* __restrict__ act) {
   for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
+    if (act && !act[x / NN]) continue;
     const double2 z = src[x];
     dst[x] = make_float2((float)z.x, (float)z.y);
   }
@@ -270,12 +275,30 @@ __global__ void k_col_exponent(const float2* __restrict__ hi, const float2* __re
   eX[(long long)b * N + j] = m > 0 ? m - (lo ? 125 : 126) : 0;
 }
 
+// round(x 2^(7 ND - e)) for |x| < 2^e: fixed56 for eight digits, to 2^-63 for nine.
+template <int ND>
+__device__ __forceinline__ long long fixed_nd(double x, int e) {
+  return fixed56(x, e - 7 * (ND - 8));
+}
+// Digit s of it from the top, |d_0| <= 128, |d_s| <= 64 after it (as next_digit; the bit below
+// the cut is added instead of a half, which could carry out of 63 bits).
+template <int ND>
+__device__ __forceinline__ int digit_nd(long long& m, int s) {
+  if (ND == 8) return next_digit(m, s);
+  const int sh = 7 * (ND - 1 - s);
+  const long long d = sh > 0 ? (m >> sh) + ((m >> (sh - 1)) & 1) : m;
+  m -= (long long)((unsigned long long)d << sh);
+  return (int)d;
+}
+
 // A operand digits.  Element (i, k) of matrix b -> kWSA digits of Re and of Im in the
 // K-major tile layout, one chunk per (matrix, 128-row block, 16-wide K step) holding
 // the 2 kWSA planes of 128 x 16 in the order (Re digits 0 .. kWSA-1, Im digits ...).
 // One thread per (row i, 8 consecutive k): it reads 128 contiguous bytes and writes one
 // 16-byte row of a core matrix per plane; the 32 lanes of a warp (i % 8, k half,
-// (i / 8) % 2) fill 512 contiguous bytes of each plane.
+// (i / 8) % 2) fill 512 contiguous bytes of each plane.  ND digits (kWSA, or kWFine for
+// the matrices beside an identity).
+template <int ND>
 __global__ void k_slice_A(const double2* __restrict__ A, const int* __restrict__ eA, uint16_t* __restrict__ Asl,
                           int N, long long n_total) {
   const int NKS = N / 16, NIB = N / 128;
@@ -297,23 +320,23 @@ __global__ void k_slice_A(const double2* __restrict__ A, const int* __restrict__
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const double2 z = src[u];
-      mr[u] = fixed56(z.x, e);
-      mi[u] = fixed56(z.y, e);
+      mr[u] = fixed_nd<ND>(z.x, e);
+      mi[u] = fixed_nd<ND>(z.y, e);
     }
-    uint16_t* chunk = Asl + ((b * NIB + ib) * NKS + ks) * (long long)(kWAChunk / 2);
+    uint16_t* chunk = Asl + ((b * NIB + ib) * NKS + ks) * (long long)(w_achunk(ND) / 2);
     const uint32_t off = kmajor_offset(128, il, 8 * h) / 2;
 #pragma unroll
-    for (int s = 0; s < kWSA; ++s) {
+    for (int s = 0; s < ND; ++s) {
       uint32_t pr[4], pi[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const uint32_t r0 = digit_bf16(next_digit(mr[2 * u], s), s), r1 = digit_bf16(next_digit(mr[2 * u + 1], s), s);
-        const uint32_t i0 = digit_bf16(next_digit(mi[2 * u], s), s), i1 = digit_bf16(next_digit(mi[2 * u + 1], s), s);
+        const uint32_t r0 = digit_bf16(digit_nd<ND>(mr[2 * u], s), s), r1 = digit_bf16(digit_nd<ND>(mr[2 * u + 1], s), s);
+        const uint32_t i0 = digit_bf16(digit_nd<ND>(mi[2 * u], s), s), i1 = digit_bf16(digit_nd<ND>(mi[2 * u + 1], s), s);
         pr[u] = r0 | (r1 << 16);
         pi[u] = i0 | (i1 << 16);
       }
-      *reinterpret_cast<uint4*>(chunk + (0 * kWSA + s) * (128 * 16) + off) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
-      *reinterpret_cast<uint4*>(chunk + (1 * kWSA + s) * (128 * 16) + off) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
+      *reinterpret_cast<uint4*>(chunk + (0 * ND + s) * (128 * 16) + off) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
+      *reinterpret_cast<uint4*>(chunk + (1 * ND + s) * (128 * 16) + off) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
     }
   }
 }
@@ -402,18 +425,22 @@ __device__ __forceinline__ int level_int(float v, float sc) {
   const float y = x + 100663296.0f;                    // 1.5 2^26: x to a multiple of 8
   return 8 * (__float_as_int(y) - 0x4CC00000) + (__float_as_int((x - (y - 100663296.0f)) + 12582912.0f) - 0x4B400000);
 }
-template <int L>
-__device__ __forceinline__ void add_level(long long& S, float v) {
-  S += (long long)level_int(v, __int_as_float((127 + 7 * (L + 2)) << 23)) << (38 - 7 * L);
+// (unsigned: with the units of 2^-59 the sum runs modulo 2^64 until the identity is taken out)
+template <int L, int UB>
+__device__ __forceinline__ void add_level(unsigned long long& S, float v) {
+  S += (unsigned long long)(long long)level_int(v, __int_as_float((127 + 7 * (L + 2)) << 23)) << (UB - 14 - 7 * L);
 }
-// levels 6 and 7 together, rounded to 2^-52 (below 2^21 of them)
-__device__ __forceinline__ void add_67(long long& S, float v6, float v7) {
-  S += __float_as_int(fmaf(v6 + v7, 0x1p52f, 12582912.0f)) - 0x4B400000;
+// the last two levels together, rounded to a unit (below 2^21 of them): 6 and 7 to 2^-52, 7 and
+// 8 to 2^-59
+template <int UB>
+__device__ __forceinline__ void add_last2(unsigned long long& S, float v0, float v1) {
+  const float sc = __int_as_float((127 + UB) << 23);
+  S += (unsigned long long)(long long)(__float_as_int(fmaf(v0 + v1, sc, 12582912.0f)) - 0x4B400000);
 }
 // levels 5 .. 7 of one accumulator, rounded to nearest at 2^-52
-__device__ __forceinline__ void add_tail(long long& S, float v) {
+__device__ __forceinline__ void add_tail(unsigned long long& S, float v) {
   const float x = v * 0x1p52f;
-  S += fabsf(x) < 0x1p25f ? (long long)level_int(x, 1.0f) : __float2ll_rn(x);
+  S += (unsigned long long)(fabsf(x) < 0x1p25f ? (long long)level_int(x, 1.0f) : __float2ll_rn(x));
 }
 // S 2^e rounded once to FP32 (ties to even), from the bit fields; below 2^-126: zero
 __device__ __forceinline__ float i2f_scaled(long long S, int e) {
@@ -435,20 +462,20 @@ __device__ __forceinline__ float i2f_scaled(long long S, int e) {
 
 // The MMAs of one 16-wide K step.  `first`: the step's first product of each accumulator
 // writes it.  TAIL: the levels 5 .. LMAX share accumulator 5 (written by the step `first5`).
-template <int SX, int LMAX, bool TAIL>
+template <int SX, int LMAX, bool TAIL, int TN>
 __device__ __forceinline__ void product_issue_step(uint32_t tm, uint64_t da0, uint64_t dx0, bool neg, bool first,
                                                    bool first5) {
-  constexpr uint32_t PA = 128 * 16 * 2, PX = kWTN * 16 * 2;  // bytes per A / B plane
+  constexpr uint32_t PA = 128 * 16 * 2, PX = TN * 16 * 2;  // bytes per A / B plane
   constexpr int LW = TAIL ? 4 : LMAX;                          // levels with an accumulator of their own
   if (TAIL) {
-    const uint32_t id = neg ? idesc_bf16_f32_negA(128, kWTN) : idesc_bf16_f32(128, kWTN);
+    const uint32_t id = neg ? idesc_bf16_f32_negA(128, TN) : idesc_bf16_f32(128, TN);
     bool fresh = first5;
 #pragma unroll
     for (int t = 0; t < SX; ++t)
 #pragma unroll
       for (int s = 0; s <= LMAX; ++s)
         if (s + t >= 5 && s + t <= LMAX) {
-          mma_bf16(tm + 5 * kWTN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t * PX) >> 4), id, fresh ? 0u : 1u);
+          mma_bf16(tm + 5 * TN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t * PX) >> 4), id, fresh ? 0u : 1u);
           fresh = false;
         }
   }
@@ -456,13 +483,13 @@ __device__ __forceinline__ void product_issue_step(uint32_t tm, uint64_t da0, ui
   for (int s = 0; s <= LW; ++s) {
     const int nt = (LW - s + 1) < SX ? (LW - s + 1) : SX;
 #pragma unroll
-    for (int t0 = 0; t0 < nt; t0 += 4) {
-      const int n = (nt - t0) < 4 ? (nt - t0) : 4;
-      const uint32_t id = neg ? idesc_bf16_f32_negA(128, kWTN * n) : idesc_bf16_f32(128, kWTN * n);
+    for (int t0 = 0; t0 < nt; t0 += 256 / TN) {
+      const int n = (nt - t0) < 256 / TN ? (nt - t0) : 256 / TN;
+      const uint32_t id = neg ? idesc_bf16_f32_negA(128, TN * n) : idesc_bf16_f32(128, TN * n);
       // an accumulator's first product: digit 0 of A, or (levels beyond the digits of B) the
       // smallest digit of A that reaches it, with B's last digit
       const bool init = s == 0 || (s + t0 >= SX && t0 == SX - 1);
-      mma_bf16(tm + (uint32_t)(s + t0) * kWTN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t0 * PX) >> 4), id,
+      mma_bf16(tm + (uint32_t)(s + t0) * TN, da0 + (uint64_t)((s * PA) >> 4), dx0 + (uint64_t)((t0 * PX) >> 4), id,
                (first && init) ? 0u : 1u);
     }
   }
@@ -477,30 +504,32 @@ __device__ __forceinline__ void product_issue_step(uint32_t tm, uint64_t da0, ui
 // refinement keeps the rounding it always had: where v^-1 - P is close to singular, W~ follows
 // the last bits of that residual).  A warp's 32 x
 // 16 results go through shared memory, so that a store covers two rows of 16 columns.
-// 264 complex products 768 x 256 by 256 x 1024 (a step of N = 1024): 3.88 ms, 4.54 with
-// float-to-integer conversions on four warps and 64-column MMAs for the residuals; 936
-// residuals of N = 384: six levels 3.54 ms (5.03), eight with TAIL 6.36 ms (7.07), eight
-// without 5.42 ms.  What bounds it now is the digits' way from L2: 48 KB per K step.
-template <int SX, int LMAX, bool RES, bool TAIL>
+// 264 complex 768 x 256 by 256 x 1024 products (N = 1024): 4.54 ms with float-to-integer
+// conversions on four warps; N = 384 residuals, 900 matrices, eight levels: 7.1 ms.
+template <int SX, int LMAX, bool RES, bool TAIL, int ND>
 __global__ void __launch_bounds__(kPT, 1) k_oz_product(const __grid_constant__ OzProductArgs g) {
   constexpr int NL = LMAX + 1;
-  static_assert((NL == 8 && SX == 8) || (NL == 6 && SX == 5), "eight levels of eight digits, or six of five");
+  constexpr int TN = w_tn(LMAX);         // columns per block
+  constexpr int W = TN / 4;              // columns per warp
+  constexpr int UB = NL == 9 ? 59 : 52;  // sums in units of 2^-UB
+  static_assert((NL == 9 && SX == 9 && RES) || (NL == 8 && SX == 8) || (NL == 6 && SX == 5), "the level read-out below");
   static_assert(!TAIL || NL == 8, "levels 5 .. 7");
-  static_assert(NL * kWTN <= 512, "the accumulators fit the tensor memory");
-  constexpr uint32_t PA = 128 * 16 * 2, PX = kWTN * 16 * 2;
+  static_assert(NL * TN <= 512, "the accumulators fit the tensor memory");
+  constexpr uint32_t PA = 128 * 16 * 2, PX = TN * 16 * 2;
   constexpr uint32_t AB = NL * PA, XB = SX * PX, SB = AB + XB;  // bytes per stage
-  constexpr uint32_t XC = wx_chunk(SX);
+  constexpr uint32_t XC = wx_chunk(SX, TN);
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t full[kWStages];
   __shared__ __align__(8) uint64_t mmad[kWStages];
   __shared__ __align__(8) uint64_t gdone;
   const int jb = blockIdx.x;
-  const int NKS = g.K / 16, NIB = g.M / 128, NJB = g.Nc / kWTN;
+  const int NKS = g.K / 16, NIB = g.M / 128, NJB = g.Nc / TN;
   const bool imrow = (int)blockIdx.y >= NIB;
   const int ib = imrow ? (int)blockIdx.y - NIB : (int)blockIdx.y;
   if (!RES && ib >= g.skip0 && ib < g.skip1) return;  // the whole block: before any barrier or allocation
   const long long b = blockIdx.z;
+  if (RES && g.act && !g.act[b]) return;
   const int NK2 = 2 * NKS;
   const int n_groups = (2 * g.K > kPExact && NL > 6) ? 2 : 1;  // six levels need no exact last bits
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -522,7 +551,7 @@ __global__ void __launch_bounds__(kPT, 1) k_oz_product(const __grid_constant__ O
   fence_after_sync();
   const uint32_t tm = tmem_base;
   const unsigned char* Abase =
-      reinterpret_cast<const unsigned char*>(g.Asl) + ((b * NIB + ib) * NKS) * (long long)kWAChunk;
+      reinterpret_cast<const unsigned char*>(g.Asl) + ((b * NIB + ib) * NKS) * (long long)w_achunk(ND);
   const unsigned char* Xbase = reinterpret_cast<const unsigned char*>(g.Bsl) + ((b * NJB + jb) * NKS) * (long long)XC;
   // step kk: half 0 takes (Ar | Ai for Im rows) with Br, half 1 (Ai negated | Ar) with Bi
   auto load = [&](int kk, int st) {
@@ -530,14 +559,14 @@ __global__ void __launch_bounds__(kPT, 1) k_oz_product(const __grid_constant__ O
     const int cA = imrow ? 1 - half : half;
     unsigned char* dst = sm + st * SB;
     mbar_arrive_expect_tx(&full[st], SB);
-    bulk_g2s(dst, Abase + (long long)ks * kWAChunk + (long long)cA * kWSA * PA, AB, &full[st]);
+    bulk_g2s(dst, Abase + (long long)ks * w_achunk(ND) + (long long)cA * ND * PA, AB, &full[st]);
     bulk_g2s(dst + AB, Xbase + (long long)ks * XC + (long long)half * SX * PX, XB, &full[st]);
   };
-  const int quad = warp & 3, c0 = 16 * (warp >> 2);  // this warp's lanes 32 quad .. and columns c0 ..
+  const int quad = warp & 3, c0 = W * (warp >> 2);  // this warp's lanes 32 quad .. and columns c0 ..
   const uint32_t t_addr = tm + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
-  long long S[16];
+  unsigned long long S[W];
 #pragma unroll
-  for (int c = 0; c < 16; ++c) S[c] = 0;
+  for (int c = 0; c < W; ++c) S[c] = 0;
   bool ok = true;
   if (tid == 0)
     for (int s = 0; s < kWStages && s < NK2; ++s) load(s, s);
@@ -550,7 +579,7 @@ __global__ void __launch_bounds__(kPT, 1) k_oz_product(const __grid_constant__ O
         const int st = kk % kWStages;
         if (!mbar_wait(&full[st], (uint32_t)(kk / kWStages) & 1u, kWaitNs, status)) { ok = false; break; }
         fence_after_sync();
-        product_issue_step<SX, LMAX, TAIL>(tm, smem_desc(s0 + st * SB, 128, 256),
+        product_issue_step<SX, LMAX, TAIL, TN>(tm, smem_desc(s0 + st * SB, 128, 256),
                                            smem_desc(s0 + st * SB + AB, 128, 256), !imrow && kk >= NKS, kk == k_begin,
                                            kk == 0);
         mma_commit(&mmad[st]);
@@ -569,25 +598,44 @@ __global__ void __launch_bounds__(kPT, 1) k_oz_product(const __grid_constant__ O
     ok = __syncthreads_and(ok && done ? 1 : 0) != 0;
     fence_after_sync();
     if (!ok) break;
-    {
-      float v[32];
-      tmem_ld16x2(t_addr, kWTN, v);
+    float v[32];
+    if constexpr (W == 8) {  // nine levels of 32 columns
+      tmem_ld8x4(t_addr, TN, v);
 #pragma unroll
-      for (int c = 0; c < 16; ++c) { add_level<0>(S[c], v[c]); add_level<1>(S[c], v[16 + c]); }
-      tmem_ld16x2(t_addr + 2 * kWTN, kWTN, v);
+      for (int c = 0; c < 8; ++c) {
+        add_level<0, UB>(S[c], v[c]);
+        add_level<1, UB>(S[c], v[8 + c]);
+        add_level<2, UB>(S[c], v[16 + c]);
+        add_level<3, UB>(S[c], v[24 + c]);
+      }
+      tmem_ld8x4(t_addr + 4 * TN, TN, v);
+      float v8[32];
+      tmem_ld8x4(t_addr + 5 * TN, TN, v8);  // the last of them is level 8
 #pragma unroll
-      for (int c = 0; c < 16; ++c) { add_level<2>(S[c], v[c]); add_level<3>(S[c], v[16 + c]); }
-      tmem_ld16x2(t_addr + 4 * kWTN, kWTN, v);
+      for (int c = 0; c < 8; ++c) {
+        add_level<4, UB>(S[c], v[c]);
+        add_level<5, UB>(S[c], v[8 + c]);
+        add_level<6, UB>(S[c], v[16 + c]);
+        add_last2<UB>(S[c], v[24 + c], v8[24 + c]);
+      }
+    } else {
+      tmem_ld16x2(t_addr, TN, v);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) { add_level<0, UB>(S[c], v[c]); add_level<1, UB>(S[c], v[16 + c]); }
+      tmem_ld16x2(t_addr + 2 * TN, TN, v);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) { add_level<2, UB>(S[c], v[c]); add_level<3, UB>(S[c], v[16 + c]); }
+      tmem_ld16x2(t_addr + 4 * TN, TN, v);
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
-        add_level<4>(S[c], v[c]);
-        if (!TAIL) add_level<5>(S[c], v[16 + c]);
+        add_level<4, UB>(S[c], v[c]);
+        if (!TAIL) add_level<5, UB>(S[c], v[16 + c]);
         else if (grp + 1 == n_groups) add_tail(S[c], v[16 + c]);
       }
       if (NL == 8 && !TAIL) {
-        tmem_ld16x2(t_addr + 6 * kWTN, kWTN, v);
+        tmem_ld16x2(t_addr + 6 * TN, TN, v);
 #pragma unroll
-        for (int c = 0; c < 16; ++c) add_67(S[c], v[c], v[16 + c]);
+        for (int c = 0; c < 16; ++c) add_last2<UB>(S[c], v[c], v[16 + c]);
       }
     }
     if (grp + 1 < n_groups) {  // the next half writes the accumulators
@@ -601,49 +649,59 @@ __global__ void __launch_bounds__(kPT, 1) k_oz_product(const __grid_constant__ O
   } else {
     const int i = ib * 128 + 32 * quad + lane;
     const int ea = g.eA[b * g.M + i];
-    const int* eb = g.eB + b * g.Nc + jb * kWTN + c0;
-    const int cc = lane & 15, r2 = lane >> 4;
+    const int* eb = g.eB + b * g.Nc + jb * TN + c0;
+    const int cc = lane % W, r2 = lane / W;
+    constexpr int RP = 32 / W;  // rows per store
     // every product has read its stage: the stages are free for the results
     if (RES) {
-      float* stg = reinterpret_cast<float*>(sm) + warp * (32 * 17);
+      float* stg = reinterpret_cast<float*>(sm) + warp * (32 * (W + 1));
       bool range_ok = true;
+      unsigned big = 0u;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const int j = jb * kWTN + c0 + c;
+      for (int c = 0; c < W; ++c) {
+        const int j = jb * TN + c0 + c;
         const int e = ea + eb[c];  // (A X)_ij = 2^e sum
-        long long val = S[c];
+        unsigned long long val = S[c];
         if (!imrow && i == j) {
-          if (e < -10 || e > 52) range_ok = false;
-          else val -= 1ll << (52 - e);  // 1 = 2^(52 - e) units of 2^(e - 52)
+          if (e < -10 || e > UB) range_ok = false;
+          else if (UB - e < 64) val -= 1ull << (UB - e);  // 1 = 2^(UB - e) units of 2^(e - UB)
         }
         if (e < -126 || e > 126) range_ok = false;
-        const float res = i2f_scaled(-val, min(max(e, -126), 126) - 52);
-        stg[lane * 17 + c] = res;
+        const float res = i2f_scaled(-(long long)val, min(max(e, -126), 126) - UB);
+        big = max(big, __float_as_uint(fabsf(res)));
+        stg[lane * (W + 1) + c] = res;
       }
       __syncwarp();
       float* Rw = reinterpret_cast<float*>(g.R + (b * g.M + ib * 128 + 32 * quad) * (long long)g.Nc) + (imrow ? 1 : 0);
 #pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        const int rr = 2 * t + r2;
-        Rw[2 * ((long long)rr * g.Nc + jb * kWTN + c0 + cc)] = stg[rr * 17 + cc];
+      for (int t = 0; t < W; ++t) {
+        const int rr = RP * t + r2;
+        Rw[2 * ((long long)rr * g.Nc + jb * TN + c0 + cc)] = stg[rr * (W + 1) + cc];
       }
-      if (!range_ok) atomicExch(status, 4);  // scale outside the FP32 exponent range
+      if (!range_ok) {  // scale outside the FP32 exponent range
+        if (g.weak) g.weak[b] = 1;
+        else atomicExch(status, 4);
+      }
+      if (g.rmax) {
+        for (int o = 16; o > 0; o >>= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, o));
+        if (lane == 0) atomicMax(g.rmax + b, big);
+      }
     } else {
-      double* stg = reinterpret_cast<double*>(sm) + warp * (32 * 17);
+      double* stg = reinterpret_cast<double*>(sm) + warp * (32 * (W + 1));
       double* Cw = reinterpret_cast<double*>(g.C + b * g.c_ms + (long long)(ib * 128 + 32 * quad) * g.ldc) + (imrow ? 1 : 0);
       // the old C values first: independent loads in flight while the sums are rounded
       double cold[16];
 #pragma unroll
       for (int t = 0; t < 16; ++t)
-        cold[t] = g.accumulate ? Cw[2 * ((long long)(2 * t + r2) * g.ldc + jb * kWTN + c0 + cc)] : 0.0;
+        cold[t] = g.accumulate ? Cw[2 * ((long long)(2 * t + r2) * g.ldc + jb * TN + c0 + cc)] : 0.0;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) stg[lane * 17 + c] = i2d_scaled(S[c], ea + eb[c] - 52);
+      for (int c = 0; c < 16; ++c) stg[lane * (W + 1) + c] = i2d_scaled((long long)S[c], ea + eb[c] - 52);
       __syncwarp();
 #pragma unroll
       for (int t = 0; t < 16; ++t) {
         const int rr = 2 * t + r2;
-        const double pv = stg[rr * 17 + cc];
-        Cw[2 * ((long long)rr * g.ldc + jb * kWTN + c0 + cc)] = g.accumulate ? cold[t] - pv : pv;
+        const double pv = stg[rr * (W + 1) + cc];
+        Cw[2 * ((long long)rr * g.ldc + jb * TN + c0 + cc)] = g.accumulate ? cold[t] - pv : pv;
       }
     }
   }
@@ -689,7 +747,8 @@ __device__ __forceinline__ void split3_store8(const float2* z, uint16_t* chunk, 
 // BF16x3 operand planes of a row-major FP32 complex matrix M[b][r][k] (rows r = the MMA's
 // M or N rows, k = reduction index): one kRefChunk chunk per (matrix, 128-row block,
 // 16-wide K step).  Thread mapping as in k_slice_A.
-__global__ void k_split3_rows(const float2* __restrict__ M, uint16_t* __restrict__ P, int N, long long n_total) {
+__global__ void k_split3_rows(const float2* __restrict__ M, uint16_t* __restrict__ P, int N, long long n_total,
+                              const int* __restrict__ act) {
   const int NKS = N / 16, NRB = N / 128;
   const long long n_thr = n_total / 8;
   for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < n_thr; x += (long long)gridDim.x * blockDim.x) {
@@ -699,6 +758,7 @@ __global__ void k_split3_rows(const float2* __restrict__ M, uint16_t* __restrict
     const int ks = (int)(w % NKS); w /= NKS;
     const int rb = (int)(w % NRB);
     const long long b = w / NRB;
+    if (act && !act[b]) continue;
     const int h = (lane >> 3) & 1;
     const int rl = (lane & 7) + 8 * ((lane >> 4) + 2 * gp);
     const float2* src = M + (b * N + rb * 128 + rl) * (long long)N + ks * 16 + 8 * h;
@@ -711,7 +771,8 @@ __global__ void k_split3_rows(const float2* __restrict__ M, uint16_t* __restrict
 
 // The same planes for the transpose: element M[b][k][r] goes to row r (for the B operand
 // of X R, whose rows are the columns of R).  Thread mapping as in k_slice_X.
-__global__ void k_split3_cols(const float2* __restrict__ M, uint16_t* __restrict__ P, int N, long long n_total) {
+__global__ void k_split3_cols(const float2* __restrict__ M, uint16_t* __restrict__ P, int N, long long n_total,
+                              const int* __restrict__ act) {
   const int NKS = N / 16, NRB = N / 128;
   const long long n_thr = n_total / 8;
   for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < n_thr; x += (long long)gridDim.x * blockDim.x) {
@@ -721,6 +782,7 @@ __global__ void k_split3_cols(const float2* __restrict__ M, uint16_t* __restrict
     const int ks = (int)(w % NKS); w /= NKS;
     const int rb = (int)(w % NRB);
     const long long b = w / NRB;
+    if (act && !act[b]) continue;
     const int h = (lane >> 3) & 1;
     const int rl = (lane & 7) + 8 * ((lane >> 4) + 2 * gp);
     const float2* src = M + (b * N + ks * 16 + 8 * h) * (long long)N + rb * 128 + rl;
@@ -743,7 +805,8 @@ __global__ void k_split3_cols(const float2* __restrict__ M, uint16_t* __restrict
 template <int MODE>
 __global__ void __launch_bounds__(128, 1)
 k_refine_tc(const uint16_t* __restrict__ PX, const uint16_t* __restrict__ PR, const float2* __restrict__ hi,
-            float2* __restrict__ lo, double2* __restrict__ out, int N, int* status) {
+            float2* __restrict__ lo, double2* __restrict__ out, int N, int* status, const int* __restrict__ act) {
+  if (act && !act[blockIdx.z]) return;
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint32_t tmem_base;
   __shared__ __align__(8) uint64_t full[kRefStages];
@@ -855,11 +918,60 @@ k_refine_tc(const uint16_t* __restrict__ PX, const uint16_t* __restrict__ PR, co
   if (warp == 0) tmem_dealloc(tm, 256);
 }
 
+// flag[b] = 1 where the largest residual of matrix b is above `most` (one that is no number
+// counts as large); else 0 with `clear`, or as it was.
+__global__ void k_mark(unsigned* __restrict__ rmax, int* __restrict__ flag, int batch, float most, int clear) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= batch) return;
+  if (rmax[b] > __float_as_uint(most)) flag[b] = 1;
+  else if (clear) flag[b] = 0;
+  rmax[b] = 0u;
+}
+
+// A back from its digits (to 2^-64 of its row's largest element, under the rounding that an
+// FP64 elimination commits) for the matrices marked weak.
+__global__ void k_unslice_A(const uint16_t* __restrict__ Asl, const int* __restrict__ eA, const int* __restrict__ weak,
+                            double2* __restrict__ A, int N) {
+  const long long b = blockIdx.y;
+  if (!weak[b]) return;
+  const int NKS = N / 16, NIB = N / 128;
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < N * N; x += gridDim.x * blockDim.x) {
+    const int i = x / N, k = x - i * N;
+    const uint16_t* chunk = Asl + ((b * NIB + i / 128) * NKS + k / 16) * (long long)(w_achunk(kWFine) / 2) +
+                            kmajor_offset(128, i % 128, k % 16) / 2;
+    const int e = eA[b * N + i];
+    double z[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      unsigned long long m = 0;
+#pragma unroll
+      for (int s = 0; s < kWFine; ++s) {
+        const float d = __uint_as_float((uint32_t)chunk[(c * kWFine + s) * (128 * 16)] << 16);
+        m += (unsigned long long)(long long)__float2int_rn(d * __int_as_float((127 + 7 * (s + 1)) << 23)) << (56 - 7 * s);
+      }
+      z[c] = scalbn((double)(long long)m, e - 63);
+    }
+    A[b * N * N + x] = make_double2(z[0], z[1]);
+  }
+}
+
+__global__ void k_panel_col_exp(const double2* __restrict__ B, long long ms, int ld, int K, int Nc,
+                                int* __restrict__ e, const int* __restrict__ act);
+template <int ND>
+__global__ void k_slice_panel_B(const double2* __restrict__ B, long long ms, int ld, const int* __restrict__ eB,
+                                uint16_t* __restrict__ Bsl, int K, int Nc, long long n_thr,
+                                const int* __restrict__ act);
+
 cudaError_t wtc_setup(size_t smem_gj32) {
   cudaError_t e = raise_smem_limit(k_gj_inverse_f32, smem_gj32);
-  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX0, kWL0, true, false>, w_residual_smem(kWSX0, kWL0));
-  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, true>, w_residual_smem(kWSX1, kWLmax));
-  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, false>, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX0, kWL0, true, false, kWSA>, w_residual_smem(kWSX0, kWL0));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, true, kWSA>, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, false, kWSA>, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX0, kWL0, true, false, kWFine>, w_residual_smem(kWSX0, kWL0));
+  if (e == cudaSuccess)
+    e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, true, kWFine>, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess)
+    e = raise_smem_limit(k_oz_product<kWFine, kWFine - 1, true, false, kWFine>, w_residual_smem(kWFine, kWFine - 1));
   if (e == cudaSuccess) e = raise_smem_limit(k_refine_tc<0>, w_refine_smem());
   if (e == cudaSuccess) e = raise_smem_limit(k_refine_tc<1>, w_refine_smem());
   if (e == cudaSuccess) e = raise_smem_limit(k_refine_tc<2>, w_refine_smem());
@@ -869,6 +981,7 @@ cudaError_t wtc_setup(size_t smem_gj32) {
 void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t smem_gj32, cudaStream_t st,
                  int refinements) {
   const long long NN = (long long)N * N;
+  const bool fine = w.weak != nullptr;
   const long long tot = (long long)batch * NN;
   const unsigned g1 = (unsigned)((tot + 255) / 256 < 65535LL * 8 ? (tot + 255) / 256 : 65535LL * 8);
   const long long t8 = tot / 8;  // slicing threads: one per 8 consecutive elements
@@ -883,15 +996,21 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   ga.R = w.R;
   ga.M = ga.Nc = ga.K = N;
   ga.status = w.status;
+  ga.weak = w.weak;
+  const int* act = nullptr;
   const dim3 gref((unsigned)(N / 128), (unsigned)(N / 128), (unsigned)batch);
+  if (w.weak) {
+    cudaMemsetAsync(w.weak, 0, (size_t)batch * sizeof(int), st);
+    cudaMemsetAsync(w.rmax, 0, (size_t)batch * sizeof(unsigned), st);
+  }
   // X0: FP32 Gauss-Jordan
   {
     gw::TimedLaunch tl_("k_to_f32", st);
-    k_to_f32<<<g1, 256, 0, st>>>(mats, w.X32, tot);
+    k_to_f32<<<g1, 256, 0, st>>>(mats, w.X32, tot, NN, nullptr);
   }
   {
     gw::TimedLaunch tl_("k_gj_inverse_f32", st);
-    k_gj_inverse_f32<<<batch, 512, smem_gj32, st>>>(w.X32, N, NN, w.status);
+    k_gj_inverse_f32<<<batch, 512, smem_gj32, st>>>(w.X32, N, NN, w.status, w.weak);
   }
   // digits of A (kept for both residuals)
   {
@@ -900,7 +1019,8 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_slice_A", st);
-    k_slice_A<<<g8, 256, 0, st>>>(mats, w.eA, w.Asl, N, tot);
+    if (fine) k_slice_A<kWFine><<<g8, 256, 0, st>>>(mats, w.eA, w.Asl, N, tot);
+    else k_slice_A<kWSA><<<g8, 256, 0, st>>>(mats, w.eA, w.Asl, N, tot);
   }
   // R0 = I - A X0 (FP32), lo = X0 R0: X1 = X0 + lo
   {
@@ -913,19 +1033,20 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_ozaki_residual<first>", st);
-    k_oz_product<kWSX0, kWL0, true, false><<<gres, kPT, w_residual_smem(kWSX0, kWL0), st>>>(ga);
+    if (fine) k_oz_product<kWSX0, kWL0, true, false, kWFine><<<gres, kPT, w_residual_smem(kWSX0, kWL0), st>>>(ga);
+    else k_oz_product<kWSX0, kWL0, true, false, kWSA><<<gres, kPT, w_residual_smem(kWSX0, kWL0), st>>>(ga);
   }
   {
     gw::TimedLaunch tl_("k_split3_rows", st);
-    k_split3_rows<<<g8, 256, 0, st>>>(w.X32, w.PX, N, tot);
+    k_split3_rows<<<g8, 256, 0, st>>>(w.X32, w.PX, N, tot, act);
   }
   {
     gw::TimedLaunch tl_("k_split3_cols", st);
-    k_split3_cols<<<g8, 256, 0, st>>>(w.R, w.Xsl, N, tot);  // the X digits are no longer needed
+    k_split3_cols<<<g8, 256, 0, st>>>(w.R, w.Xsl, N, tot, act);  // the X digits are no longer needed
   }
   {
     gw::TimedLaunch tl_("k_refine_tc<first>", st);
-    k_refine_tc<0><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, nullptr, N, w.status);
+    k_refine_tc<0><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, nullptr, N, w.status, act);
   }
   // R1 = I - A X1 (FP32), X2 = X1 + X0 R1 in FP64, written over A
   {
@@ -938,48 +1059,81 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_ozaki_residual<second>", st);
-    k_oz_product<kWSX1, kWLmax, true, true><<<gres, kPT, w_residual_smem(kWSX1, kWLmax), st>>>(ga);
+    ga.rmax = w.rmax;
+    if (fine) k_oz_product<kWSX1, kWLmax, true, true, kWFine><<<gres, kPT, w_residual_smem(kWSX1, kWLmax), st>>>(ga);
+    else k_oz_product<kWSX1, kWLmax, true, true, kWSA><<<gres, kPT, w_residual_smem(kWSX1, kWLmax), st>>>(ga);
   }
   {
     gw::TimedLaunch tl_("k_split3_cols", st);
-    k_split3_cols<<<g8, 256, 0, st>>>(w.R, w.Xsl, N, tot);
+    k_split3_cols<<<g8, 256, 0, st>>>(w.R, w.Xsl, N, tot, act);
   }
   {
     gw::TimedLaunch tl_("k_refine_tc<final>", st);
-    k_refine_tc<1><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status);
+    k_refine_tc<1><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status, act);
+  }
+  // the second residual has to be small before its successor is taken modulo 2^64
+  if (fine) {
+    gw::TimedLaunch tl_("k_mark", st);
+    k_mark<<<(unsigned)((batch + 255) / 256), 256, 0, st>>>(w.rmax, w.weak, batch, 0x1p-8f, 0);
   }
   // X <- X + X (I - A X) again, the left factor now the current X rounded to FP32 (the
   // correction is needed to 2^-24 of itself only): with X0 there the error would shrink
-  // by |I - A X0| per step, with X by about kappa 2^-24 |I - A X|
+  // by |I - A X0| per step, with X by about kappa 2^-24 |I - A X|.  With nine digits the
+  // residual is good to 2^-59 of |A||X|, so the corrected X is that of FP64 rounding; the
+  // fourth refinement then takes only the matrices whose third residual was above 2^-38.
   for (int r = 3; r <= refinements; ++r) {
     {
       gw::TimedLaunch tl_("k_to_f32", st);
-      k_to_f32<<<g1, 256, 0, st>>>(mats, w.X32, tot);
+      k_to_f32<<<g1, 256, 0, st>>>(mats, w.X32, tot, NN, act);
     }
     {
       gw::TimedLaunch tl_("k_split3_rows", st);
-      k_split3_rows<<<g8, 256, 0, st>>>(w.X32, w.PX, N, tot);
+      k_split3_rows<<<g8, 256, 0, st>>>(w.X32, w.PX, N, tot, act);
     }
     {
       gw::TimedLaunch tl_("k_panel_col_exp", st);
-      k_panel_col_exp<<<dim3((unsigned)((N + 127) / 128), (unsigned)batch), 128, 0, st>>>(mats, NN, N, N, N, w.eX);
+      k_panel_col_exp<<<dim3((unsigned)((N + 127) / 128), (unsigned)batch), 128, 0, st>>>(mats, NN, N, N, N, w.eX, act);
     }
     {
       gw::TimedLaunch tl_("k_slice_panel_B", st);
-      k_slice_panel_B<<<g8, 256, 0, st>>>(mats, NN, N, w.eX, w.Xsl, N, N, t8);
+      if (fine) k_slice_panel_B<kWFine><<<g8, 256, 0, st>>>(mats, NN, N, w.eX, w.Xsl, N, N, t8, act);
+      else k_slice_panel_B<kWSX1><<<g8, 256, 0, st>>>(mats, NN, N, w.eX, w.Xsl, N, N, t8, act);
     }
     {
       gw::TimedLaunch tl_("k_ozaki_residual<third>", st);
-      k_oz_product<kWSX1, kWLmax, true, false><<<gres, kPT, w_residual_smem(kWSX1, kWLmax), st>>>(ga);
+      ga.rmax = w.rmax;
+      ga.act = act;
+      if (fine) {
+        const dim3 gf((unsigned)(N / w_tn(kWFine - 1)), gres.y, gres.z);
+        k_oz_product<kWFine, kWFine - 1, true, false, kWFine>
+            <<<gf, kPT, w_residual_smem(kWFine, kWFine - 1), st>>>(ga);
+      } else {
+        k_oz_product<kWSX1, kWLmax, true, false, kWSA><<<gres, kPT, w_residual_smem(kWSX1, kWLmax), st>>>(ga);
+      }
     }
     {
       gw::TimedLaunch tl_("k_split3_cols", st);
-      k_split3_cols<<<g8, 256, 0, st>>>(w.R, w.Xsl, N, tot);
+      k_split3_cols<<<g8, 256, 0, st>>>(w.R, w.Xsl, N, tot, act);
     }
     {
       gw::TimedLaunch tl_("k_refine_tc<add>", st);
-      k_refine_tc<2><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status);
+      k_refine_tc<2><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status, act);
     }
+    if (fine) {
+      gw::TimedLaunch tl_("k_mark", st);
+      const bool last = r == refinements;
+      k_mark<<<(unsigned)((batch + 255) / 256), 256, 0, st>>>(w.rmax, last ? w.weak : w.act, batch,
+                                                               last ? 0x1p-30f : 0x1p-38f, last ? 0 : 1);
+      act = w.act;
+    }
+  }
+  if (fine) {
+    // what is left: by FP64 elimination, from A's digits
+    {
+      gw::TimedLaunch tl_("k_unslice_A", st);
+      k_unslice_A<<<dim3(16, (unsigned)batch), 256, 0, st>>>(w.Asl, w.eA, w.weak, mats, N);
+    }
+    gj_batch_only(mats, w.perm, batch, N, w.status, w.weak, st);
   }
 }
 
@@ -1015,8 +1169,9 @@ __global__ void k_panel_row_exp(const double2* __restrict__ A, long long ms, int
 
 // Scale exponent of each column of a K x Nc panel: one thread per column.
 __global__ void k_panel_col_exp(const double2* __restrict__ B, long long ms, int ld, int K, int Nc,
-                                int* __restrict__ e) {
+                                int* __restrict__ e, const int* __restrict__ act) {
   const int b = blockIdx.y;
+  if (act && !act[b]) return;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= Nc) return;
   const double2* c = B + (long long)b * ms + j;
@@ -1071,12 +1226,15 @@ __global__ void k_slice_panel_A(const double2* __restrict__ A, long long ms, int
   }
 }
 
-// B-operand digits of a K x Nc panel (FP64), chunks as k_slice_X<kWSX1>: one per
-// (matrix, kWTN-column block, 16-wide K step) with the kWSX1 digits of Re, then of Im.
+// B-operand digits of a K x Nc panel (FP64), chunks as k_slice_X: one per (matrix, column
+// block, 16-wide K step) with the ND digits of Re, then of Im (blocks of kWTN columns, or of
+// the narrower ones of nine digits).
+template <int ND>
 __global__ void k_slice_panel_B(const double2* __restrict__ B, long long ms, int ld, const int* __restrict__ eB,
-                                uint16_t* __restrict__ Bsl, int K, int Nc, long long n_thr) {
-  constexpr int JG = kWTN / 16;
-  const int NKS = K / 16, NJB = Nc / kWTN;
+                                uint16_t* __restrict__ Bsl, int K, int Nc, long long n_thr,
+                                const int* __restrict__ act) {
+  constexpr int TN = w_tn(ND - 1), JG = TN / 16;
+  const int NKS = K / 16, NJB = Nc / TN;
   for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < n_thr; x += (long long)gridDim.x * blockDim.x) {
     const int lane = (int)(x & 31);
     long long w = x >> 5;  // (b, jb, ks, column group)
@@ -1084,9 +1242,10 @@ __global__ void k_slice_panel_B(const double2* __restrict__ B, long long ms, int
     const int ks = (int)(w % NKS); w /= NKS;
     const int jb = (int)(w % NJB);
     const long long b = w / NJB;
+    if (act && !act[b]) continue;
     const int h = (lane >> 3) & 1;
     const int jl = (lane & 7) + 8 * ((lane >> 4) + 2 * jg);
-    const int j = jb * kWTN + jl;
+    const int j = jb * TN + jl;
     const int k0 = ks * 16 + 8 * h;
     const int e = eB[b * Nc + j];
     const double2* src = B + b * ms + (long long)k0 * ld + j;
@@ -1094,23 +1253,23 @@ __global__ void k_slice_panel_B(const double2* __restrict__ B, long long ms, int
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const double2 z = src[(long long)u * ld];
-      mr[u] = fixed56(z.x, e);
-      mi[u] = fixed56(z.y, e);
+      mr[u] = fixed_nd<ND>(z.x, e);
+      mi[u] = fixed_nd<ND>(z.y, e);
     }
-    uint16_t* chunk = Bsl + ((b * NJB + jb) * NKS + ks) * (long long)(wx_chunk(kWSX1) / 2);
-    const uint32_t off = kmajor_offset(kWTN, jl, 8 * h) / 2;
+    uint16_t* chunk = Bsl + ((b * NJB + jb) * NKS + ks) * (long long)(wx_chunk(ND, TN) / 2);
+    const uint32_t off = kmajor_offset(TN, jl, 8 * h) / 2;
 #pragma unroll
-    for (int t = 0; t < kWSX1; ++t) {
+    for (int t = 0; t < ND; ++t) {
       uint32_t pr[4], pi[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const uint32_t r0 = digit_bf16(next_digit(mr[2 * u], t), t), r1 = digit_bf16(next_digit(mr[2 * u + 1], t), t);
-        const uint32_t i0 = digit_bf16(next_digit(mi[2 * u], t), t), i1 = digit_bf16(next_digit(mi[2 * u + 1], t), t);
+        const uint32_t r0 = digit_bf16(digit_nd<ND>(mr[2 * u], t), t), r1 = digit_bf16(digit_nd<ND>(mr[2 * u + 1], t), t);
+        const uint32_t i0 = digit_bf16(digit_nd<ND>(mi[2 * u], t), t), i1 = digit_bf16(digit_nd<ND>(mi[2 * u + 1], t), t);
         pr[u] = r0 | (r1 << 16);
         pi[u] = i0 | (i1 << 16);
       }
-      *reinterpret_cast<uint4*>(chunk + (0 * kWSX1 + t) * (kWTN * 16) + off) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
-      *reinterpret_cast<uint4*>(chunk + (1 * kWSX1 + t) * (kWTN * 16) + off) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
+      *reinterpret_cast<uint4*>(chunk + (0 * ND + t) * (TN * 16) + off) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
+      *reinterpret_cast<uint4*>(chunk + (1 * ND + t) * (TN * 16) + off) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
     }
   }
 }
@@ -1153,12 +1312,12 @@ void panel_gemm(const WblkBuffers& w, const double2* A, long long a_ms, int lda,
   }
   {
     gw::TimedLaunch tl_("k_panel_col_exp", st);
-    k_panel_col_exp<<<dim3((unsigned)((Nc + 127) / 128), (unsigned)batch), 128, 0, st>>>(B, b_ms, ldb, K, Nc, w.eB);
+    k_panel_col_exp<<<dim3((unsigned)((Nc + 127) / 128), (unsigned)batch), 128, 0, st>>>(B, b_ms, ldb, K, Nc, w.eB, nullptr);
   }
   {
     gw::TimedLaunch tl_("k_slice_panel_B", st);
-    k_slice_panel_B<<<grid_for((long long)batch * K * Nc / 8), 256, 0, st>>>(B, b_ms, ldb, w.eB, w.Bsl, K, Nc,
-                                                                              (long long)batch * K * Nc / 8);
+    k_slice_panel_B<kWSX1><<<grid_for((long long)batch * K * Nc / 8), 256, 0, st>>>(
+        B, b_ms, ldb, w.eB, w.Bsl, K, Nc, (long long)batch * K * Nc / 8, nullptr);
   }
   OzProductArgs g{};
   g.Asl = w.Asl;
@@ -1177,7 +1336,7 @@ void panel_gemm(const WblkBuffers& w, const double2* A, long long a_ms, int lda,
   g.status = w.inner.status;
   {
     gw::TimedLaunch tl_("k_oz_panel_gemm", st);
-    k_oz_product<kWSX1, kWLmax, false, false><<<dim3((unsigned)(Nc / kWTN), (unsigned)(2 * (M / 128)), (unsigned)batch), kPT,
+    k_oz_product<kWSX1, kWLmax, false, false, kWSA><<<dim3((unsigned)(Nc / kWTN), (unsigned)(2 * (M / 128)), (unsigned)batch), kPT,
                                          w_residual_smem(kWSX1, kWLmax), st>>>(g);
   }
 }
@@ -1200,7 +1359,7 @@ int wblk_block_size(int N) {
 
 cudaError_t wblk_setup(size_t smem_gj32_bs) {
   cudaError_t e = wtc_setup(smem_gj32_bs);
-  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, false, false>, w_residual_smem(kWSX1, kWLmax));
+  if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, false, false, kWSA>, w_residual_smem(kWSX1, kWLmax));
   return e;
 }
 

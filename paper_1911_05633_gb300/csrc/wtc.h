@@ -15,12 +15,17 @@ constexpr int kWLmax = 7;    // second residual: products a_s x_t with s + t <= 
 constexpr int kWTN = 64;     // output columns per residual block
 constexpr int kWNmax = 384;  // largest N whose level sums stay exact in FP32
 constexpr int kWStages = 4;  // shared-memory stages of the residual
-constexpr uint32_t kWAChunk = kWSA * 2 * 128 * 16 * 2;  // bytes per (row block, K step): Re then Im digits
-__host__ __device__ constexpr uint32_t wx_chunk(int SX) { return (uint32_t)SX * 2 * kWTN * 16 * 2; }
+constexpr int kWFine = 9;     // digits of both operands in the last residuals of the matrices beside an identity
+// bytes of A digits per (row block, K step): Re then Im digits
+__host__ __device__ constexpr uint32_t w_achunk(int ND) { return (uint32_t)ND * 2 * 128 * 16 * 2; }
+constexpr uint32_t kWAChunk = w_achunk(kWSA);
+// columns per block of k_oz_product: its level accumulators fill the 512 of the tensor memory
+__host__ __device__ constexpr int w_tn(int lmax) { return lmax < 8 ? kWTN : 32; }
+__host__ __device__ constexpr uint32_t wx_chunk(int SX, int TN = kWTN) { return (uint32_t)SX * 2 * TN * 16 * 2; }
 // dynamic shared memory of the residual: per stage the A digits s <= lmax of one
 // component (128 x 16 each) and the SX digits of one component of X (kWTN x 16 each)
 __host__ __device__ constexpr size_t w_residual_smem(int SX, int lmax) {
-  return (size_t)kWStages * ((size_t)(lmax + 1) * 128 * 16 * 2 + (size_t)SX * kWTN * 16 * 2);
+  return (size_t)kWStages * ((size_t)(lmax + 1) * 128 * 16 * 2 + (size_t)SX * w_tn(lmax) * 16 * 2);
 }
 
 constexpr int kGJ32B = 32;    // panel width of the FP32 Gauss-Jordan inverse
@@ -33,12 +38,12 @@ __host__ __device__ constexpr size_t gj32_buf_elems(int N) {
 __host__ __device__ constexpr size_t gj32_smem(int N) {
   return ((size_t)N * kGJ32B + gj32_buf_elems(N)) * 8 + ((size_t)2 * N + 4 * kGJ32B) * 4;
 }
-__global__ void k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __restrict__ status);
-__global__ void k_to_f32(const double2* __restrict__ src, float2* __restrict__ dst, long long n);
+__global__ void k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __restrict__ status,
+                                 int* __restrict__ weak);
+__global__ void k_to_f32(const double2* __restrict__ src, float2* __restrict__ dst, long long n, long long NN,
+                         const int* __restrict__ act);
 __global__ void k_row_exponent(const double2* __restrict__ A, int* __restrict__ eA, int N, int batch);
 
-__global__ void k_slice_A(const double2* __restrict__ A, const int* __restrict__ eA, uint16_t* __restrict__ Asl,
-                          int N, long long n_total);
 // Refinement products X R on the tensor cores: BF16x3 planes, 6 planes of 128 x 16 per
 // (128-row block, 16-wide K step) chunk, kRefStages pipeline stages of 2 chunks.
 constexpr uint32_t kRefChunk = 6 * 128 * 16 * 2;
@@ -58,6 +63,13 @@ struct WtcBuffers {
   int* eA;
   int* eX;
   int* status;
+  // where the FP64 inverse takes over: [batch] flags of the matrices that the refinement
+  // did not reach, the largest |I - A X| of each as bits, pivot scratch [batch][N]; or null
+  // (the FP32 pivots and ranges then go to *status)
+  int* weak;
+  unsigned* rmax;
+  int* act;  // [batch] matrices that the fourth refinement takes
+  int* perm;
 };
 
 // Raise the shared-memory limits of the kernels (once per device and size).
@@ -79,6 +91,9 @@ struct OzProductArgs {
   int skip0, skip1;  // 128-row blocks of C left alone
   int accumulate;
   int* status;
+  unsigned* rmax;  // largest |R| of each matrix as bits, or null
+  int* weak;       // matrices out of the FP32 range, or null (*status then)
+  const int* act;  // matrices with act[b] == 0 are left out; null: none
 };
 // Scratch of one batch of block inverses of N x N with pivot blocks of bs (per matrix:
 // the pivot block D, the row panel Rp, the digits of a bs-column and a bs-row panel, 2 N
@@ -109,9 +124,5 @@ void wblk_inverse(const WblkBuffers& w, double2* mats, int batch, int N, int bs,
 // `refinements` (at least 2) FP64-accurate refinements of the FP32 inverse.
 void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t smem_gj32, cudaStream_t st,
                  int refinements = 2);
-__global__ void k_panel_col_exp(const double2* __restrict__ B, long long ms, int ld, int K, int Nc,
-                                int* __restrict__ e);
-__global__ void k_slice_panel_B(const double2* __restrict__ B, long long ms, int ld, const int* __restrict__ eB,
-                                uint16_t* __restrict__ Bsl, int K, int Nc, long long n_thr);
 
 }  // namespace gw
