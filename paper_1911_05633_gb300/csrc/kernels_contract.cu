@@ -23,6 +23,12 @@
 // stores.  Every wait on the tensor core or on a bulk copy is bounded: after the limit
 // the group records the failure (status 2) and waits once more, bounded, for its
 // products in flight before the block releases its tensor memory and ends.
+//
+// Both kernels wait on their CUDA-core stages (four warps per scheduler; DRAM at 10 to 20 %
+// of its rate): what helps is fewer trips to shared memory and more loads in flight.  72-atom
+// cell, 64 nodes: Sigma 16.4 -> 15.0 ms with rows of the dense stage at an odd stride, G
+// read 16 bytes at a time and eight values of W~ in flight per thread; P 9.13 -> 8.59 ms with
+// G's transpose read 16 bytes at a time and four rows of its store in flight.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -97,6 +103,9 @@ __device__ __forceinline__ void split3x2(float x0, float x1, uint32_t& h, uint32
   m = *reinterpret_cast<uint32_t*>(&mm);
   l = *reinterpret_cast<uint32_t*>(&ll);
 }
+
+// Complex FP32 values per row of n that make rows of 16-byte words.
+__device__ __forceinline__ int row16(int n) { return (n + 1) & ~1; }
 
 // Shared-memory layout of one group (byte offsets from the group's base).
 struct GLayout {
@@ -235,6 +244,7 @@ __device__ bool p_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
   // G(tau) and conj(G(beta - tau)) transposed, in FP32
   float2* G1 = c.Gs;
   float2* G2t = c.Gs + kCMaxOrb * kCMaxOrb;
+  const int gst = row16(na);  // row stride of the transpose: rows start on 16 bytes
   {
     const double2* Gin = S.G + E.off_orb * nt;
     for (int x = t; x < na * nb; x += kTG) {
@@ -242,7 +252,7 @@ __device__ bool p_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
       const double2 g2 = __ldg(Gin + (long long)im * na * nb + x);
       G1[x] = make_float2(d2f(g1.x), d2f(g1.y));
       const int L2 = x / nb, L3 = x - L2 * nb;
-      G2t[L3 * na + L2] = make_float2(d2f(g2.x), -d2f(g2.y));
+      G2t[L3 * gst + L2] = make_float2(d2f(g2.x), -d2f(g2.y));
     }
   }
   group_sync(c.g);
@@ -295,13 +305,19 @@ __device__ bool p_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
                   }
                   cur = L1;
                 }
-                const float2* g2 = G2t + L3 * na;
+                // conj(G(beta - tau)[L''][L''']), two values per load: one 8-byte broadcast per four
+                // multiply-adds kept the load-store pipe as busy as the FP32 pipes
+                const float4* g2 = reinterpret_cast<const float4*>(G2t + L3 * gst);
 #pragma unroll
-                for (int L2 = 0; L2 < NA; ++L2) {
+                for (int L2 = 0; L2 < NA; L2 += 2) {
                   if (EXACT || L2 < na) {
-                    const float2 b = g2[L2];  // conj(G(beta - tau)[L''][L'''])
+                    const float4 b = g2[L2 / 2];
                     yr = fmaf(xr[L2], b.x, fmaf(-xi[L2], b.y, yr));
                     yi = fmaf(xr[L2], b.y, fmaf(xi[L2], b.x, yi));
+                    if (L2 + 1 < NA && (EXACT || L2 + 1 < na)) {
+                      yr = fmaf(xr[L2 + 1], b.z, fmaf(-xi[L2 + 1], b.w, yr));
+                      yi = fmaf(xr[L2 + 1], b.w, fmaf(xi[L2 + 1], b.z, yi));
+                    }
                   }
                 }
               }
@@ -350,15 +366,24 @@ __device__ bool p_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
       double2* Pt = Pout + (long long)it * Ka * Kb + (long long)K0 * Kb;
       double2* Pm = Pout + (long long)im * Ka * Kb + (long long)K0 * Kb;
       // rows over the group's warps, columns over the lanes (consecutive stores)
-      for (int klx = t >> 5; klx < KL; klx += kTG / 32)
-        for (int Kp = t & 31; Kp < Kb; Kp += 32) {
-          const float2 p = Ps[klx * ldp + Kp];
+      for (int Kp = t & 31; Kp < Kb; Kp += 32) {
+        auto put = [&](int klx, float2 p) {
           const float zr = msf * p.x, zi = msf * p.y;  // -s is a power of two: exact
           const double dr = f2d(zr), di = f2d(zi);
           const int x = klx * Kb + Kp;
           Pt[x] = make_double2(dr, di);
           if (mirror) Pm[x] = make_double2(dr, dneg(di));
+        };
+        int klx = t >> 5;
+        for (; klx + 3 * (kTG / 32) < KL; klx += 4 * (kTG / 32)) {  // four rows' reads in flight
+          float2 p[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) p[u] = Ps[(klx + u * (kTG / 32)) * ldp + Kp];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) put(klx + u * (kTG / 32), p[u]);
         }
+        for (; klx < KL; klx += kTG / 32) put(klx, Ps[klx * ldp + Kp]);
+      }
     }
     // a staging wider than the A buffer overwrote the B operand
     if (t == 0 && (uint32_t)(64 * ldp * 8) > c.a_bytes) c.gs->bkey = -1;
@@ -384,12 +409,13 @@ __device__ bool s_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
   const int bkey = (sys << 12) | (sb << 2) | E.tier;
   const int t = c.t;
   const double2* Win = S.W + E.off_pb * S.w_slices + (long long)it * Ka * Kb;
+  const int gst = row16(nb);  // row stride of G(tau): rows start on 16 bytes
   {
     const int gs = S.g_fixed >= 0 ? S.g_fixed : it;
     const double2* Gin = S.G + E.off_orb * S.g_slices + (long long)gs * na * nb;
     for (int x = t; x < na * nb; x += kTG) {
       const double2 gv = __ldg(Gin + x);
-      c.Gs[x] = make_float2(d2f(gv.x), d2f(gv.y));
+      c.Gs[(x / nb) * gst + x % nb] = make_float2(d2f(gv.x), d2f(gv.y));
     }
   }
   group_sync(c.g);
@@ -414,14 +440,13 @@ __device__ bool s_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
         const int kk = k0 + 8 * q8;
         uint32_t pk[6][4];
         const double2* wrow = Win + (long long)(K0 + kl) * Kb;
+        double2 w[8];  // all eight loads in flight before the first conversion
+#pragma unroll
+        for (int u = 0; u < 8; ++u) w[u] = kk + u < Kb ? __ldg(wrow + kk + u) : make_double2(0.0, 0.0);
 #pragma unroll
         for (int u2 = 0; u2 < 4; ++u2) {
-          float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
-          const int k = kk + 2 * u2;
-          if (k < Kb) { const double2 w = __ldg(wrow + k); a0 = d2f(w.x); b0 = d2f(w.y); }
-          if (k + 1 < Kb) { const double2 w = __ldg(wrow + k + 1); a1 = d2f(w.x); b1 = d2f(w.y); }
-          split3x2(a0, a1, pk[0][u2], pk[1][u2], pk[2][u2]);
-          split3x2(b0, b1, pk[3][u2], pk[4][u2], pk[5][u2]);
+          split3x2(d2f(w[2 * u2].x), d2f(w[2 * u2 + 1].x), pk[0][u2], pk[1][u2], pk[2][u2]);
+          split3x2(d2f(w[2 * u2].y), d2f(w[2 * u2 + 1].y), pk[3][u2], pk[4][u2], pk[5][u2]);
         }
         const uint32_t o_r = kmajor_offset(128, kl, kk - k0), o_i = kmajor_offset(128, 64 + kl, kk - k0);
 #pragma unroll
@@ -436,11 +461,13 @@ __device__ bool s_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
     // Bm[kl][L'][L'''] (complex FP32) from tensor memory into the A buffer, in passes over L'
     const int n_used = min(unit_n_hh(NJ), KD / 16);
     float2* Bm = reinterpret_cast<float2*>(c.A);
-    const int ldb = (nb + 1) & ~1;  // padded L''' stride (float2): rows 16-byte aligned
-    const int cap = (int)(c.a_bytes / 8u) / (64 * ldb);
-    const int per_pass = max(1, min(nb, cap));
+    // a row of K holds np_ nb complex values and, when that is even, one more: the lanes of
+    // stage C read the same column of consecutive rows, and an odd stride of 8-byte words
+    // spreads 16 of them over all banks (at 90 they took two turns, and with G's 8-byte
+    // reads that was most of the unit's time in the load-store pipe)
+    const int per_pass = max(1, min(nb, ((int)(c.a_bytes / 8u) / 64 - 1) / nb));
     for (int l0 = 0; l0 < nb; l0 += per_pass) {
-      const int l1 = min(nb, l0 + per_pass), np_ = l1 - l0;
+      const int l1 = min(nb, l0 + per_pass), np_ = l1 - l0, ldk_b = (np_ * nb) | 1;
       const int jlo = l0 * nb, jhi = l1 * nb;
       {
         const int wq = c.warp & 3, wsub = (c.warp >> 2) & 1;
@@ -452,14 +479,11 @@ __device__ bool s_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
           acc_sum16(c, lane_off, c0, NJ, n_used, v);
           const int kl = r & 63;
           if (kl < KL) {
-            float* dst = reinterpret_cast<float*>(Bm + kl * (np_ * ldb)) + (r >> 6);
+            float* dst = reinterpret_cast<float*>(Bm + kl * ldk_b) + (r >> 6);
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
               const int j = c0 + k;
-              if (j >= jlo && j < jhi) {
-                const int L1 = j / nb, L3 = j - L1 * nb;
-                dst[2 * ((L1 - l0) * ldb + L3)] = v[k];
-              }
+              if (j >= jlo && j < jhi) dst[2 * (j - jlo)] = v[k];
             }
           }
         }
@@ -476,22 +500,26 @@ __device__ bool s_unit(const GCtx& c, const CSys& S, const DevEntry& E, int it, 
           for (int L2 = 0; L2 < NA; ++L2) {
             if (EXACT || L2 < na) {
               const float cv = __ldg(CK + (long long)L2 * ldk);
-              const float2* gr = c.Gs + L2 * nb;
+              const float4* gr = reinterpret_cast<const float4*>(c.Gs + L2 * gst);  // two values per load
 #pragma unroll
-              for (int L3 = 0; L3 < NB; ++L3) {
+              for (int L3 = 0; L3 < NB; L3 += 2) {
                 if (EXACT || L3 < nb) {
-                  const float2 gv = gr[L3];
+                  const float4 gv = gr[L3 / 2];
                   hr[L3] = fmaf(cv, gv.x, hr[L3]);
                   hi[L3] = fmaf(cv, gv.y, hi[L3]);
+                  if (L3 + 1 < NB && (EXACT || L3 + 1 < nb)) {
+                    hr[L3 + 1] = fmaf(cv, gv.z, hr[L3 + 1]);
+                    hi[L3 + 1] = fmaf(cv, gv.w, hi[L3 + 1]);
+                  }
                 }
               }
             }
           }
-          const float2* bk = Bm + kl * (np_ * ldb);
+          const float2* bk = Bm + kl * ldk_b;
 #pragma unroll
           for (int L1 = 0; L1 < NB; ++L1) {
             if (L1 >= l0 && L1 < l1) {
-              const float2* b = bk + (L1 - l0) * ldb;
+              const float2* b = bk + (L1 - l0) * nb;
               float sr = 0.f, si = 0.f;
 #pragma unroll
               for (int L3 = 0; L3 < NB; ++L3) {
