@@ -20,6 +20,7 @@
 #include "wtc.h"
 #include "oz.h"
 #include "chain.h"
+#include "lattice.h"
 #include "ktimer.h"
 #include "dyson.h"
 #include "gj.h"
@@ -102,6 +103,7 @@ struct gw_plan_s {
   gw::OzSigma oz;
   gw::OzTransform ozt;  // FP64-accurate structured transforms on the tensor cores
   gw::OzPol ozp;        // FP64-accurate stage 3 of P on the tensor cores
+  gw::LatticePlan lattice;  // R <-> k on meshes with general phases
   gw::ChainPlan chain;  // FP64 P and Sigma over symmetric pairs (in place of oz and ozp when it fits)
   gw::KernelTimer timer;  // optional per-kernel event timing (gw_timing_*)
   gw::DysonPlan dyson;    // Eq. G_1 scratch, allocated by the first Dyson call
@@ -186,6 +188,7 @@ void free_device(gw_plan_s* p) {
   gw::oz_transform_free(p->ozt);
   gw::oz_pol_free(p->ozp);
   gw::chain_free(p->chain);
+  gw::lattice_free(p->lattice);
   gw::dyson_free(p->dyson);
 }
 
@@ -220,6 +223,13 @@ unsigned band_splits(const gw_plan_s* p, gw_block kind, int n_slices) {
   const long long base = (long long)p->h.n_atoms * std::max(1, n_slices);
   const long long want = (4LL * std::max(1, sms) + base - 1) / base;
   return (unsigned)std::max<long long>(1, std::min<long long>({want, (el + 255) / 256, 65535}));
+}
+
+// Whether a transform of n_slices slices goes to the tensor cores (lattice.h): from about
+// 8 million FP64 multiply-adds on, 15 us of the chip; below that either way is launch latency.
+bool lattice_takes(const gw_plan_s* p, gw_block kind, int n_slices) {
+  const double len = (double)(kind == GW_BLOCK_PB ? p->h.off_pb : p->h.off_orb).back();
+  return p->lattice.ok && len * n_slices * p->h.n_k * 4.0 >= 8e6;
 }
 
 gw_status launch_gather(gw_plan_s* p, gw_block kind, int n_slices, const double2* F_k, long long k_stride,
@@ -649,7 +659,10 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
     if ((st = upload(&p->d_counter, nullptr, 16)) != GW_OK) return fail(st);
     gw::set_last_error("");
   }
-  if (!(opt && opt->fp64_products == 1) && (st = gw::chain_init(p->chain, h)) != GW_OK) return fail(st);
+  if (!(opt && opt->fp64_products == 1)) {
+    if ((st = gw::chain_init(p->chain, h)) != GW_OK) return fail(st);
+    if ((st = gw::lattice_init(p->lattice, h)) != GW_OK) return fail(st);
+  }
   if (p->sigma_tensor) {
     if (defer) p->oz_pending = true;
     else if ((st = alloc_oz_sigma(p)) != GW_OK) return fail(st);
@@ -757,6 +770,10 @@ gw_status gw_fourier_k_to_R(gw_plan_t p, gw_block kind, int n_slices, const void
   if (!F_k || !F_R || n_slices <= 0) { set_last_error("bad argument"); return GW_ERR_ARG; }
   DeviceGuard guard(p->device);
   gw::ActiveTimer timing(&p->timer);
+  if (lattice_takes(p, kind, n_slices))
+    return gw::lattice_run(p->lattice, p->h, p->d_ent, kind == GW_BLOCK_PB ? p->d_pb_off : p->d_orb_off,
+                           kind == GW_BLOCK_PB, n_slices, false, (double2*)const_cast<void*>(F_k), (double2*)F_R,
+                           p->d_status, S(stream));
   const long long N = dense_n(p, kind);
   return launch_gather(p, kind, n_slices, (const double2*)F_k, (long long)n_slices * N * N, N * N, nullptr, 0, 0,
                        (double2*)F_R, n_slices, 0, 1.0 / p->h.n_k, S(stream));
@@ -773,6 +790,10 @@ gw_status gw_fourier_R_to_k(gw_plan_t p, gw_block kind, int n_slices, const void
   if (!F_k || !F_R || n_slices <= 0) { set_last_error("bad argument"); return GW_ERR_ARG; }
   DeviceGuard guard(p->device);
   gw::ActiveTimer timing(&p->timer);
+  if (lattice_takes(p, kind, n_slices))
+    return gw::lattice_run(p->lattice, p->h, p->d_ent, kind == GW_BLOCK_PB ? p->d_pb_off : p->d_orb_off,
+                           kind == GW_BLOCK_PB, n_slices, true, (double2*)F_k, (double2*)const_cast<void*>(F_R),
+                           p->d_status, S(stream));
   const long long N = dense_n(p, kind);
   return launch_scatter(p, kind, n_slices, (const double2*)F_R, n_slices, 0, (double2*)F_k,
                         (long long)n_slices * N * N, N * N, S(stream));
