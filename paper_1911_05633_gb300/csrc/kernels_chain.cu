@@ -40,22 +40,15 @@ constexpr uint32_t kChStep = kOzDigits * kTfPlane;  // 32 KB: digits of 128 rows
 __host__ __device__ constexpr uint32_t ch_bstep(int NT) { return (uint32_t)kOzDigits * NT * 32; }
 
 // Digits of 8 values of one row to global memory: K half h of step ks of unit base A.
-__device__ __forceinline__ void ch_store_row(unsigned char* A, int r, int k8, const long long* M) {
-  unsigned char* a = A + (k8 >> 1) * kChStep + kmajor_offset(128, r, 8 * (k8 & 1));
-  *reinterpret_cast<uint4*>(a + 0 * kTfPlane) = tf_plane_row<0>(M);
-  *reinterpret_cast<uint4*>(a + 1 * kTfPlane) = tf_plane_row<1>(M);
-  *reinterpret_cast<uint4*>(a + 2 * kTfPlane) = tf_plane_row<2>(M);
-  *reinterpret_cast<uint4*>(a + 3 * kTfPlane) = tf_plane_row<3>(M);
-  *reinterpret_cast<uint4*>(a + 4 * kTfPlane) = tf_plane_row<4>(M);
-  *reinterpret_cast<uint4*>(a + 5 * kTfPlane) = tf_plane_row<5>(M);
-  *reinterpret_cast<uint4*>(a + 6 * kTfPlane) = tf_plane_row<6>(M);
-  *reinterpret_cast<uint4*>(a + 7 * kTfPlane) = tf_plane_row<7>(M);
+__device__ __forceinline__ void ch_store_row(unsigned char* A, int r, int k8, const long long* m) {
+  tf_cut8(m, A + (k8 >> 1) * kChStep + kmajor_offset(128, r, 8 * (k8 & 1)));
 }
 
 // ---------------------------------------------------------------------------------------
 // M of one unit (entry blockIdx.x, node s0 + blockIdx.y) and its digits.  Bound by the FP64
 // pipe: four multiply-adds per ordering.  The rows' scales need all of a row, so M goes
-// through shared memory once.
+// through shared memory once.  9024 units of n = 9: 0.48 ms, 0.41 of it FP64 issue; stages X and Y of the
+// other path took 3.13 ms.
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_polarizability_pairs(const DevEntry* __restrict__ ent,
                                                               const int* __restrict__ species,
@@ -127,8 +120,8 @@ __global__ void __launch_bounds__(256) k_polarizability_pairs(const DevEntry* __
     for (int u = 0; u < 8; ++u) {
       const int q = 8 * k8 + u;
       const double2 z = p < np && q < nq ? M[p * ldq + q] : make_double2(0.0, 0.0);
-      R[u] = fixed56(z.x, e_s[p]) + kTfBias;
-      I[u] = fixed56(z.y, e_s[64 + p]) + kTfBias;
+      R[u] = fixed56(z.x, e_s[p]);
+      I[u] = fixed56(z.y, e_s[64 + p]);
     }
     ch_store_row(A, p, k8, R);
     ch_store_row(A, 64 + p, k8, I);
@@ -171,8 +164,8 @@ __global__ void __launch_bounds__(256) k_slice_w_units(const DevEntry* __restric
     for (int u = 0; u < 8; ++u) {
       const int k = 8 * k8 + u;
       const double2 z = K < Ka && k < Kb ? w[(long long)K * Kb + k] : make_double2(0.0, 0.0);
-      R[u] = fixed56(z.x, e_s[K]) + kTfBias;
-      I[u] = fixed56(z.y, e_s[64 + K]) + kTfBias;
+      R[u] = fixed56(z.x, e_s[K]);
+      I[u] = fixed56(z.y, e_s[64 + K]);
     }
     ch_store_row(A, K, k8, R);
     ch_store_row(A, 64 + K, k8, I);
@@ -191,8 +184,8 @@ __global__ void __launch_bounds__(256) k_slice_w_units(const DevEntry* __restric
 // slots idle.  The digits of the next unit come in by bulk copies while this one's second
 // product is read out.  P goes out through shared memory, so that a store is 16 bytes of 32
 // consecutive K' (from the accumulators' lanes it would be the real or the imaginary halves).
-// 9024 units of n = 9, K = 48: 0.73 ms for P (0.76 with 16 columns per warp and halves
-// stored from the lanes), 18424 units of Sigma 1.29 ms (1.47).  Prefetching the next unit's
+// 9024 units of n = 9, K = 48: 0.69 ms for P (with 16 columns per warp and halves stored from
+// the lanes 0.03 ms more), 18424 units of Sigma 1.22 ms (0.18 more).  Prefetching the next unit's
 // digits into L2 changed nothing (0.74 ms): they are there.
 // ---------------------------------------------------------------------------------------
 struct ChainArgs {
@@ -236,7 +229,7 @@ __device__ __forceinline__ void ch_sums(uint32_t taddr, uint32_t NT, long long* 
         const float s0 = __int_as_float((127 + 7 * (l + q)) << 23), s1 = __int_as_float((127 + 7 * (l + q + 1)) << 23);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const int P = tf_level_int<false>(v[8 * q + j], s0) * 128 + tf_level_int<false>(v[8 * q + 8 + j], s1);
+          const int P = tf_pair_int<false>(v[8 * q + j], s0, v[8 * q + 8 + j], s1);
           if (l + q < 6) S[c0 + j] += (long long)P << (42 - 7 * (l + q + 1));
           else S[c0 + j] += (long long)((P + 64) >> 7);  // level 7: rounded at 2^-56
         }
@@ -347,18 +340,11 @@ __global__ void __launch_bounds__(ch_threads(NT), 1) k_chain(const __grid_consta
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int em = row_e[64 * c + n0 + 8 * h + j];
-          M[j] = (em > -100000 ? shift_round(S[8 * h + j], ea + eB1[n0 + 8 * h + j] - em) : 0ll) + kTfBias;
+          M[j] = em > -100000 ? shift_round(S[8 * h + j], ea + eB1[n0 + 8 * h + j] - em) : 0ll;
         }
         // M-major core matrices: 8 reduction indices of 16 bytes, 8 rows (c, n) in each
         unsigned char* a = A + (r >> 4) * kChStep + ((64 * c + n0) / 8 + h) * 256 + ((r >> 3) & 1) * 128 + (r & 7) * 16;
-        *reinterpret_cast<uint4*>(a + 0 * kTfPlane) = tf_plane_row<0>(M);
-        *reinterpret_cast<uint4*>(a + 1 * kTfPlane) = tf_plane_row<1>(M);
-        *reinterpret_cast<uint4*>(a + 2 * kTfPlane) = tf_plane_row<2>(M);
-        *reinterpret_cast<uint4*>(a + 3 * kTfPlane) = tf_plane_row<3>(M);
-        *reinterpret_cast<uint4*>(a + 4 * kTfPlane) = tf_plane_row<4>(M);
-        *reinterpret_cast<uint4*>(a + 5 * kTfPlane) = tf_plane_row<5>(M);
-        *reinterpret_cast<uint4*>(a + 6 * kTfPlane) = tf_plane_row<6>(M);
-        *reinterpret_cast<uint4*>(a + 7 * kTfPlane) = tf_plane_row<7>(M);
+        tf_cut8(M, a);
       }
     }
     const int er = row_e[row];  // of this thread's row of the second product
@@ -387,7 +373,7 @@ __global__ void __launch_bounds__(ch_threads(NT), 1) k_chain(const __grid_consta
       double* d = g.D + (long long)u * g.ld_d * 128 + row;
 #pragma unroll
       for (int j = 0; j < W; ++j)
-        if (n0 + j < g.ld_d) d[(n0 + j) * 128] = er > -100000 ? i2d_scaled(S[j], er + eB2[n0 + j] - 56) : 0.0;
+        if (n0 + j < g.ld_d) d[(n0 + j) * 128] = er > -100000 ? tf_i2d(S[j], er + eB2[n0 + j] - 56) : 0.0;
     } else {
       const int grp = warp >> 2, tg = tid & 127;
       double* stg = reinterpret_cast<double*>(B2 + BB) + grp * (8 * 64 * 2);
@@ -400,7 +386,7 @@ __global__ void __launch_bounds__(ch_threads(NT), 1) k_chain(const __grid_consta
 #pragma unroll
         for (int j = 0; j < 8; ++j)  // -s (s = 1 or 2) folded into the integer and the exponent
           stg[(2 * j + c) * 64 + r] =
-              er > -100000 ? i2d_scaled(-S[8 * h + j], er + eB2[n0 + 8 * h + j] - 56 + g.ms_shift) : 0.0;
+              er > -100000 ? tf_i2d(-S[8 * h + j], er + eB2[n0 + 8 * h + j] - 56 + g.ms_shift) : 0.0;
         asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
         const int Kp = tg & 63;
 #pragma unroll
@@ -431,7 +417,7 @@ __global__ void __launch_bounds__(ch_threads(NT), 1) k_chain(const __grid_consta
 // ---------------------------------------------------------------------------------------
 // Sigma[L][L'] = sign sum_{L'' L'''} D[(L, L'')][(L', L''')] G[L''][L'''], one unit per block.
 // Bound by the FP64 pipe: n_a^2 n_b^2 complex multiply-adds.  A thread takes one (L, L') and
-// every n_seg-th L''.  18048 units of n = 9: 0.83 ms, 0.80 of it FP64 issue.
+// every n_seg-th L''.  18048 units of n = 9: 0.84 ms, 0.80 of it FP64 issue.
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_sigma_pairs(const DevEntry* __restrict__ ent, const int* __restrict__ species,
                                                      const unsigned char* __restrict__ pidx,

@@ -10,7 +10,7 @@
 // 27 points and 5.4 kept classes per pair take 290 clocks per element and SM.  Cutting the 54
 // values into digits and reading the sums back is integer and FP32 work of about a tenth of
 // that, and the products are free beside it.
-// G, v and Sigma of the 16-atom cell on a 3x3x3 mesh (1392 entries, 48 slices): 1.16 ms in
+// G, v and Sigma of the 16-atom cell on a 3x3x3 mesh (1392 entries, 48 slices): 0.99 ms in
 // three launches, 4.64 ms by k_gather_k_to_R and k_scatter_R_to_k.
 #include <cuda_runtime.h>
 
@@ -165,15 +165,8 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
             unsigned char* A = As + st * kLtStep + kmajor_offset(128, r, 8 * h);
             long long M[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) M[u] = fixed56(w[ks][u], e) + kTfBias;
-            *reinterpret_cast<uint4*>(A + 0 * kTfPlane) = tf_plane_row<0>(M);
-            *reinterpret_cast<uint4*>(A + 1 * kTfPlane) = tf_plane_row<1>(M);
-            *reinterpret_cast<uint4*>(A + 2 * kTfPlane) = tf_plane_row<2>(M);
-            *reinterpret_cast<uint4*>(A + 3 * kTfPlane) = tf_plane_row<3>(M);
-            *reinterpret_cast<uint4*>(A + 4 * kTfPlane) = tf_plane_row<4>(M);
-            *reinterpret_cast<uint4*>(A + 5 * kTfPlane) = tf_plane_row<5>(M);
-            *reinterpret_cast<uint4*>(A + 6 * kTfPlane) = tf_plane_row<6>(M);
-            *reinterpret_cast<uint4*>(A + 7 * kTfPlane) = tf_plane_row<7>(M);
+            for (int u = 0; u < 8; ++u) M[u] = fixed56(w[ks][u], e);
+            tf_cut8(M, A);
             fence_smem_to_async();
             mbar_arrive(&a_full[st]);
             ++step;
@@ -246,7 +239,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
           const float s0 = __int_as_float((127 + 7 * l) << 23), s1 = __int_as_float((127 + 7 * (l + 1)) << 23);
 #pragma unroll
           for (int k = 0; k < 16; ++k) {  // units of 2^-56 of the scale (64 terms: below 64 of it)
-            const int P = tf_level_int<false>(v[k], s0) * 128 + tf_level_int<false>(v[16 + k], s1);
+            const int P = tf_pair_int<false>(v[k], s0, v[16 + k], s1);
             if (l < 6) S[k] += (long long)P << (42 - 7 * (l + 1));
             else S[k] += (long long)((P + 64) >> 7);
           }
@@ -260,7 +253,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
         for (int k = 0; k < 16; k += 2) {
           const int n = 16 * c + k, m = n >> 1;
           if (m >= n_out) break;
-          const double2 z = make_double2(i2d_scaled(S[k], ea + eB_s[n] - 56), i2d_scaled(S[k + 1], ea + eB_s[n + 1] - 56));
+          const double2 z = make_double2(tf_i2d(S[k], ea + eB_s[n] - 56), tf_i2d(S[k + 1], ea + eB_s[n + 1] - 56));
           if (SCATTER) g.dense[m * g.k_stride + dense_at(s, i, j)] = z;
           else if (i < re_s[m] && j < ce_s[m])
             g.entries[off_s[m] + (long long)s * re_s[m] * ce_s[m] + i * ce_s[m] + j] = z;

@@ -230,15 +230,8 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_oz_transform(const __grid_con
         unsigned char* A = As + st * kTfAStage + kmajor_offset(128, r, 8 * h);
         long long M[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) M[u] = fixed56(w[u], e) + kTfBias;
-        *reinterpret_cast<uint4*>(A + 0 * kTfPlane) = tf_plane_row<0>(M);
-        *reinterpret_cast<uint4*>(A + 1 * kTfPlane) = tf_plane_row<1>(M);
-        *reinterpret_cast<uint4*>(A + 2 * kTfPlane) = tf_plane_row<2>(M);
-        *reinterpret_cast<uint4*>(A + 3 * kTfPlane) = tf_plane_row<3>(M);
-        *reinterpret_cast<uint4*>(A + 4 * kTfPlane) = tf_plane_row<4>(M);
-        *reinterpret_cast<uint4*>(A + 5 * kTfPlane) = tf_plane_row<5>(M);
-        *reinterpret_cast<uint4*>(A + 6 * kTfPlane) = tf_plane_row<6>(M);
-        *reinterpret_cast<uint4*>(A + 7 * kTfPlane) = tf_plane_row<7>(M);
+        for (int u = 0; u < 8; ++u) M[u] = fixed56(w[u], e);
+        tf_cut8(M, A);
         fence_smem_to_async();
         mbar_arrive(&a_full[st]);
       };
@@ -387,8 +380,8 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_oz_transform(const __grid_con
             const int n = n0 + j;
             if (n >= g.n_cols) break;
             const int m = n >> 1;
-            const double re = i2d_scaled(S[j], ea + eB_s[n] - 52);
-            const double im = i2d_scaled(S[j + 1], ea + eB_s[n + 1] - 52);
+            const double re = tf_i2d(S[j], ea + eB_s[n] - 52);
+            const double im = tf_i2d(S[j + 1], ea + eB_s[n + 1] - 52);
             dst[(long long)m * blk] = make_double2(re, im);
             if (g.out_mode == kTfOutMirror && g.n_out - 1 - m != m)
               dst[(long long)(g.n_out - 1 - m) * blk] = make_double2(re, dneg(im));
@@ -398,7 +391,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_oz_transform(const __grid_con
           for (int j = 0; j < 16; ++j) {
             const int n = n0 + j;
             if (n >= g.n_cols) break;
-            dst[(long long)(g.out_slice0 + n) * blk] = make_double2(i2d_scaled(S[j], ea + eB_s[n] - 52), 0.0);
+            dst[(long long)(g.out_slice0 + n) * blk] = make_double2(tf_i2d(S[j], ea + eB_s[n] - 52), 0.0);
           }
         }
       }
