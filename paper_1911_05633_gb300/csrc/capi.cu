@@ -65,7 +65,6 @@ struct gw_plan_s {
   size_t smem_P = 0, smem_S = 0, smem_T = 0;
   // tensor-core inverse (FP32 Gauss-Jordan + sliced FP64-accurate residual)
   bool w_tensor = false;
-  size_t smem_GJ32 = 0;
   float2* t_X32 = nullptr;
   float2* t_lo = nullptr;
   float2* t_R = nullptr;
@@ -330,7 +329,7 @@ gw_status launch_tensor_inverse(gw_plan_s* p, double2* mats, int batch, long lon
     w.act = p->t_act;
     w.perm = p->d_perm;
   }
-  gw::wtc_inverse(w, mats, batch, (int)N, p->smem_GJ32, st, p->w_pad ? kPadRefinements : 2);
+  gw::wtc_inverse(w, mats, batch, (int)N, st, p->w_pad ? kPadRefinements : 2);
   return check_launch("tensor-core inverse");
 }
 
@@ -351,7 +350,7 @@ gw_status launch_block_inverse(gw_plan_s* p, double2* mats, int batch, long long
   w.inner.eA = p->t_eA;
   w.inner.eX = p->t_eX;
   w.inner.status = p->d_status;
-  gw::wblk_inverse(w, mats, batch, (int)N, p->w_bs, p->smem_GJ32, st);
+  gw::wblk_inverse(w, mats, batch, (int)N, p->w_bs, st);
   return check_launch("block inverse");
 }
 
@@ -614,8 +613,7 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
                                             : ((p->w_tensor && !p->w_pad) || p->w_block ? ((size_t)24 << 30)
                                                                                         : ((size_t)4 << 30));
   if (p->w_tensor || p->w_block) {
-    p->smem_GJ32 = gw::gj32_smem(p->w_block ? p->w_bs : p->w_np);
-    if ((p->w_block ? gw::wblk_setup(p->smem_GJ32) : gw::wtc_setup(p->smem_GJ32)) != cudaSuccess) {
+    if ((p->w_block ? gw::wblk_setup() : gw::wtc_setup()) != cudaSuccess) {
       cudaError_t e = cudaGetLastError();
       set_last_error(std::string("cudaFuncSetAttribute (tensor W): ") + cudaGetErrorString(e));
       return fail(GW_ERR_UNSUPPORTED);

@@ -28,103 +28,127 @@ __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
   return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
 }
 
+// Barrier of the first N threads of the block (whole warps).
+template <int N>
+__device__ __forceinline__ void rows_barrier() {
+  asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
+}
+
 }  // namespace
 
 // In-place FP32 Gauss-Jordan inverse with partial pivoting, one 512-thread block per
-// matrix (N a multiple of kGJ32C, at most 512).  Panels of kGJ32B columns are reduced
-// in shared memory, each warp owning every 16th row with one column per lane, two
-// block barriers per column; the row exchanges and the rank-kGJ32B update of the other
-// columns, A[:, T] += (Pan - I[:, panel]) Prow (Prow: the pivot rows before the
-// update), run per chunk of kGJ32C columns with 8 x 4 complex register blocks per
-// thread.  At the end the columns are permuted back by the composite of the pivot swaps.
+// matrix (N = 128, 256 or 384).  A panel of kGJ32B columns is reduced with one row per thread
+// in registers: the pivot row, scaled by its warp, is the only operand that passes through
+// shared memory, as broadcasts.  The registers rotate by one column per step (the loop stays
+// rolled), so the column being eliminated is always v[0].  The row exchanges and the
+// rank-kGJ32B update of the other columns, A[:, T] += (Pan - I[:, panel]) Prow (Prow: the
+// pivot rows before the update), run per chunk of kGJ32C columns with 8 x 4 complex register
+// blocks per thread.  At the end the columns are permuted back by the composite of the pivot
+// swaps.  At N = 384 a block takes 3.9 M cycles: 2.5 M the update (1.8 M of FP32 FMAs; the
+// paired fma.rn.f32x2 needs its operands copied and swapped and took 3.7 M), 1.0 M the panels,
+// bound by the chain pivot - scaled row - update of each column (1.7 M with the panel in shared
+// memory, and the same with a warp per row and shuffles).  900 matrices: 13.0 ms, 16.8 before.
+template <int N>
 __global__ void __launch_bounds__(512, 1)
-k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __restrict__ status,
-                 int* __restrict__ weak) {
-  constexpr int B = kGJ32B, C = kGJ32C;
+k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__ status, int* __restrict__ weak) {
+  constexpr int B = kGJ32B, C = kGJ32C, P = kGJ32P;
   extern __shared__ __align__(16) unsigned char smraw[];
-  float2* Pan = reinterpret_cast<float2*>(smraw);  // [N][B]
-  float2* Buf = Pan + (size_t)N * B;               // Prow [B][C] / exchange staging [2B][C] / rows [16][N]
+  float2* Pan = reinterpret_cast<float2*>(smraw);  // [N][P], columns 0 .. B - 1 used
+  float2* Buf = Pan + (size_t)N * P;               // Prow [B][C] / exchange staging [2B][C] / rows [16][N]
   int* pm = reinterpret_cast<int*>(Buf + gj32_buf_elems(N));  // [N] pivot row chosen for each column
   int* srcmap = pm + N;                            // [N]
   int* xdst = srcmap + N;                          // [2B]
   int* xsrc = xdst + 2 * B;                        // [2B]
-  __shared__ float rv[2][16];  // pivot candidates per warp, by column parity
-  __shared__ int ri[2][16];
+  __shared__ unsigned cand_v[N / 32];  // pivot candidates of the warps: size and row
+  __shared__ int cand_i[N / 32];
+  __shared__ __align__(16) float2 raw_s[B], oldk_s[B], row_s[B];  // pivot row, old row k, scaled pivot row
   __shared__ int nx;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (N % C != 0 || N > 512) {
-    if (tid == 0) atomicExch(status, 3);
-    return;
-  }
   float2* M = A + (long long)blockIdx.x * mat_stride;
   for (int k0 = 0; k0 < N; k0 += B) {
-    for (int x = tid; x < N * B; x += 512) Pan[x] = M[(long long)(x / B) * N + k0 + (x % B)];
+    for (int x = tid; x < N * B; x += 512) Pan[(x / B) * P + x % B] = M[(long long)(x / B) * N + k0 + (x % B)];
     __syncthreads();
-    // pivot candidates of the panel's first column (at most one row per thread); those of
-    // the later columns are gathered while the previous column is applied
-    {
-      float best = -1.0f;
-      int bi = N;
-      if (k0 + tid < N) {
-        const float2 z = Pan[(k0 + tid) * B];
-        best = fabsf(z.x) + fabsf(z.y);
-        bi = k0 + tid;
+    if (tid < N) {  // whole warps
+      float2 v[B];  // row tid; column k0 + (m + j) % B at step m
+#pragma unroll
+      for (int j = 0; j < B; j += 2) {
+        const float4 q = *reinterpret_cast<const float4*>(Pan + tid * P + j);
+        v[j] = make_float2(q.x, q.y);
+        v[j + 1] = make_float2(q.z, q.w);
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ob = __shfl_down_sync(0xffffffffu, best, o);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (lane == 0) { rv[0][wid] = best; ri[0][wid] = bi; }
-    }
-    __syncthreads();
-    for (int m = 0; m < B; ++m) {
-      const int k = k0 + m, par = m & 1;
-      // every warp reduces the 16 candidates of column m itself (no barrier for the pivot)
-      float best = lane < 16 ? rv[par][lane] : -1.0f;
-      int bi = lane < 16 ? ri[par][lane] : N;
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      const int p = bi < N ? bi : k;
-      if (tid == 0) {
-        pm[k] = p;
-        if (!(best > 0.0f)) atomicExch(weak ? weak + blockIdx.x : status, 1);
-      }
-      // lane j holds column j of the pivot row (scaled) and of the old row k
-      const float2 d = Pan[p * B + m];
-      const float den = d.x * d.x + d.y * d.y;
-      const float2 inv = den > 0.0f ? make_float2(d.x / den, -d.y / den) : make_float2(0.0f, 0.0f);
-      const float2 rowk = lane == m ? inv : cmul(Pan[p * B + lane], inv);
-      const float2 oldk = Pan[k * B + lane];
-      __syncthreads();  // rows p and k are read by every warp before their owners rewrite them
-      // rows k and p exchanged and every row updated: warp w owns rows w, w + 16, ..., lane
-      // = column; lane m + 1 keeps the pivot candidates of the next column below row k
-      best = -1.0f;
-      bi = N;
-#pragma unroll 4
-      for (int i = wid; i < N; i += 16) {
-        const float2 cur = i == p ? oldk : Pan[i * B + lane];
-        float2 v;
-        if (i == k) {
-          v = rowk;
+#pragma unroll 1
+      for (int m = 0; m < B; ++m) {
+        const int k = k0 + m;
+        // largest |Re| + |Im| at or below row k, the first of equals: its bits + 1, 0 for none
+        const float a = fabsf(v[0].x) + fabsf(v[0].y);
+        const unsigned key = tid >= k && a >= 0.0f ? __float_as_uint(a) + 1u : 0u;
+        const unsigned wkey = __reduce_max_sync(0xffffffffu, key);
+        const unsigned wbal = __ballot_sync(0xffffffffu, key == wkey);
+        if (lane == 0) { cand_v[wid] = wkey; cand_i[wid] = 32 * wid + __ffs(wbal) - 1; }
+        rows_barrier<N>();
+        const unsigned ckey = lane < N / 32 ? cand_v[lane] : 0u;
+        const unsigned best = __reduce_max_sync(0xffffffffu, ckey);
+        const unsigned cbal = __ballot_sync(0xffffffffu, ckey == best);
+        const int p = best ? cand_i[__ffs(cbal) - 1] : k;
+        if (tid == 0) {
+          pm[k] = p;
+          if (best < 2u) atomicExch(weak ? weak + blockIdx.x : status, 1);
+        }
+        if (wid == (p >> 5)) {
+          if (tid == p) {
+#pragma unroll
+            for (int j = 0; j < B; j += 2)
+              *reinterpret_cast<float4*>(raw_s + j) = make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y);
+          }
+          __syncwarp();
+          const float2 d = raw_s[0];
+          const float den = d.x * d.x + d.y * d.y;
+          const float2 inv = den > 0.0f ? make_float2(d.x / den, -d.y / den) : make_float2(0.0f, 0.0f);
+          row_s[lane] = lane == 0 ? inv : cmul(raw_s[lane], inv);
+        }
+        if (tid == k) {
+#pragma unroll
+          for (int j = 0; j < B; j += 2)
+            *reinterpret_cast<float4*>(oldk_s + j) = make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y);
+        }
+        rows_barrier<N>();
+        // rows k and p exchanged and every other row updated, one column to the left
+        if (tid == p) {
+#pragma unroll
+          for (int j = 0; j < B; ++j) v[j] = oldk_s[j];
+        }
+        if (tid == k) {
+#pragma unroll
+          for (int j = 0; j < B; ++j) v[(j + B - 1) % B] = row_s[j];
         } else {
-          const float2 f = make_float2(__shfl_sync(0xffffffffu, cur.x, m), __shfl_sync(0xffffffffu, cur.y, m));
-          v = cfma(make_float2(-f.x, -f.y), rowk, lane == m ? make_float2(0.0f, 0.0f) : cur);
-        }
-        Pan[i * B + lane] = v;
-        if (lane == m + 1 && i > k) {
-          const float a = fabsf(v.x) + fabsf(v.y);
-          if (a > best) { best = a; bi = i; }
+          const float2 f = make_float2(-v[0].x, -v[0].y);
+          float4 q = *reinterpret_cast<const float4*>(row_s);
+          const float2 last = cfma(f, make_float2(q.x, q.y), make_float2(0.0f, 0.0f));
+          v[0] = cfma(f, make_float2(q.z, q.w), v[1]);
+#pragma unroll
+          for (int j = 2; j < B; j += 2) {
+            q = *reinterpret_cast<const float4*>(row_s + j);
+            v[j - 1] = cfma(f, make_float2(q.x, q.y), v[j]);
+            v[j] = cfma(f, make_float2(q.z, q.w), v[j + 1]);
+          }
+          v[B - 1] = last;
         }
       }
-      if (m + 1 < B && lane == m + 1) { rv[par ^ 1][wid] = best; ri[par ^ 1][wid] = bi; }
-      __syncthreads();
+      // Pan - I on the diagonal, as the update of the other columns takes it
+      const int jd = tid - k0;
+#pragma unroll
+      for (int j = 0; j < B; j += 2) {
+        if (j == jd) v[j].x -= 1.0f;
+        if (j + 1 == jd) v[j + 1].x -= 1.0f;
+        *reinterpret_cast<float4*>(Pan + tid * P + j) = make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y);
+      }
     }
-    // the trailing update below uses Pan - I on the panel's diagonal
-    if (tid < B) Pan[(k0 + tid) * B + tid].x -= 1.0f;
+    __syncthreads();
+    for (int x = tid; x < N * B; x += 512) {
+      const int i = x / B, j = x % B;
+      const float2 z = Pan[i * P + j];
+      M[(long long)i * N + k0 + j] = make_float2(z.x + (i == k0 + j ? 1.0f : 0.0f), z.y);
+    }
     // composite row exchange of this panel: new row r = old row srcmap[r]
     for (int i = tid; i < N; i += 512) srcmap[i] = i;
     __syncthreads();
@@ -173,17 +197,21 @@ k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __res
         for (int r = 0; r < 8; ++r)
 #pragma unroll
           for (int q = 0; q < 4; ++q) acc[r][q] = M[(long long)(i0 + r) * N + c0 + lane + 32 * q];
-#pragma unroll 2
-        for (int m = 0; m < B; ++m) {
-          float2 z[8], pv[4];
+        for (int m = 0; m < B; m += 2) {
+          float2 pv[4], pw[4];
 #pragma unroll
-          for (int r = 0; r < 8; ++r) z[r] = Pan[(i0 + r) * B + m];
+          for (int q = 0; q < 4; ++q) {
+            pv[q] = Buf[m * C + lane + 32 * q];
+            pw[q] = Buf[(m + 1) * C + lane + 32 * q];
+          }
 #pragma unroll
-          for (int q = 0; q < 4; ++q) pv[q] = Buf[m * C + lane + 32 * q];
+          for (int r = 0; r < 8; ++r) {
+            const float4 z = *reinterpret_cast<const float4*>(Pan + (i0 + r) * P + m);
 #pragma unroll
-          for (int r = 0; r < 8; ++r)
+            for (int q = 0; q < 4; ++q) acc[r][q] = cfma(make_float2(z.x, z.y), pv[q], acc[r][q]);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[r][q] = cfma(z[r], pv[q], acc[r][q]);
+            for (int q = 0; q < 4; ++q) acc[r][q] = cfma(make_float2(z.z, z.w), pw[q], acc[r][q]);
+          }
         }
 #pragma unroll
         for (int r = 0; r < 8; ++r)
@@ -195,10 +223,6 @@ k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __res
       }
       __syncthreads();
     }
-    if (tid < B) Pan[(k0 + tid) * B + tid].x += 1.0f;
-    __syncthreads();
-    for (int x = tid; x < N * B; x += 512) M[(long long)(x / B) * N + k0 + (x % B)] = Pan[x];
-    __syncthreads();
   }
   // undo the pivoting on the columns: new column j = old column srcmap[j], the composite
   // of the swaps (k, pm[k]) for k = N-1 down to 0
@@ -256,23 +280,36 @@ __global__ void k_row_exponent(const double2* __restrict__ A, int* __restrict__ 
   if (lane == 0) eA[row] = m > 0 ? m - 1022 : 0;
 }
 
-// one thread per column j (lo may be null): |hi|, |lo| < 2^(m - 126), so |hi + lo| < 2^(m - 125)
-__global__ void k_col_exponent(const float2* __restrict__ hi, const float2* __restrict__ lo, int* __restrict__ eX,
-                               int N) {
-  const int b = blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
+// 32 columns j per block of 8 warps, each every 8th row (lo may be null): |hi|, |lo| < 2^(m - 126),
+// so |hi + lo| < 2^(m - 125).  (One thread per column left most of the chip without loads in
+// flight: 2.1 ms instead of 0.5 for the four calls over 900 matrices of N = 384.)
+constexpr int kCE = 256;
+__device__ __forceinline__ int col_max(int m) {
+  __shared__ int part[8][32];
+  part[threadIdx.x >> 5][threadIdx.x & 31] = m;
+  __syncthreads();
+  if (threadIdx.x < 32)
+#pragma unroll
+    for (int w = 1; w < 8; ++w) m = max(m, part[w][threadIdx.x]);
+  return m;
+}
+__global__ void __launch_bounds__(kCE) k_col_exponent(const float2* __restrict__ hi, const float2* __restrict__ lo,
+                                                      int* __restrict__ eX, int N) {
+  const int b = blockIdx.y, j = blockIdx.x * 32 + (threadIdx.x & 31);
   const long long base = (long long)b * N * N + j;
   int m = 0;
-  for (int k = 0; k < N; ++k) {
-    const float2 h = hi[base + (long long)k * N];
-    m = max(m, max(exp_field(h.x), exp_field(h.y)));
-    if (lo) {
-      const float2 l = lo[base + (long long)k * N];
-      m = max(m, max(exp_field(l.x), exp_field(l.y)));
+  if (j < N)
+#pragma unroll 4
+    for (int k = threadIdx.x >> 5; k < N; k += 8) {
+      const float2 h = hi[base + (long long)k * N];
+      m = max(m, max(exp_field(h.x), exp_field(h.y)));
+      if (lo) {
+        const float2 l = lo[base + (long long)k * N];
+        m = max(m, max(exp_field(l.x), exp_field(l.y)));
+      }
     }
-  }
-  eX[(long long)b * N + j] = m > 0 ? m - (lo ? 125 : 126) : 0;
+  m = col_max(m);
+  if (threadIdx.x < 32 && j < N) eX[(long long)b * N + j] = m > 0 ? m - (lo ? 125 : 126) : 0;
 }
 
 // round(x 2^(7 ND - e)) for |x| < 2^e: fixed56 for eight digits, to 2^-63 for nine.
@@ -793,7 +830,7 @@ __global__ void k_split3_cols(const float2* __restrict__ M, uint16_t* __restrict
   }
 }
 
-// D = X R for one 128 x 128 tile per block (128 threads) on tcgen05, from the BF16x3
+// D = X R for one 128 x 128 tile per block (512 threads) on tcgen05, from the BF16x3
 // planes of X (A operand, rows i) and of R (B operand, rows j = columns of R): the six
 // term products with s + t <= 2 for each of Re = Xr Rr - Xi Ri and Im = Xr Ri + Xi Rr,
 // accumulated in FP32 in two 128-column tensor-memory accumulators.  R is small, so the
@@ -802,8 +839,10 @@ __global__ void k_split3_cols(const float2* __restrict__ M, uint16_t* __restrict
 //   MODE 0: lo[b] = D (X1 = X0 + lo is kept as the unevaluated FP32 pair)
 //   MODE 1: out[b] = hi + lo + D in FP64
 //   MODE 2: out[b] += D (a further refinement of the FP64 inverse in out)
+// The result leaves through 16 warps: with 4 the loads of hi and lo and the FP64 stores waited
+// out their latency, 4.85 ms for 936 matrices of N = 384 whose products take 1.1.
 template <int MODE>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kPT, 1)
 k_refine_tc(const uint16_t* __restrict__ PX, const uint16_t* __restrict__ PR, const float2* __restrict__ hi,
             float2* __restrict__ lo, double2* __restrict__ out, int N, int* status, const int* __restrict__ act) {
   if (act && !act[blockIdx.z]) return;
@@ -883,34 +922,33 @@ k_refine_tc(const uint16_t* __restrict__ PX, const uint16_t* __restrict__ PR, co
   if (!ok) {
     if (tid == 0) atomicExch(status, 2);
   } else {
-    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-    // The pipeline stages are free now: each warp stages its 32 rows x 64 columns there,
+    const int quad = warp & 3, c0 = 32 * (warp >> 2);
+    const uint32_t t_addr = tm + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
+    // The pipeline stages are free now: each warp stages its 32 rows x 32 columns there,
     // so that its loads and stores run along rows (32 consecutive columns per instruction).
-    float2* stg = reinterpret_cast<float2*>(sm) + warp * (32 * 65);
-    const long long row0 = (b * N + ib * 128 + 32 * warp) * (long long)N + jb * 128;
-    for (int c0 = 0; c0 < 128; c0 += 64) {
-      float re[64], im[64];
-      tmem_ld16x4(tm + lane_base + (uint32_t)c0, 16, re);
-      tmem_ld16x4(tm + lane_base + (uint32_t)(128 + c0), 16, im);
+    float2* stg = reinterpret_cast<float2*>(sm) + warp * (32 * 33);
+    const long long row0 = (b * N + ib * 128 + 32 * quad) * (long long)N + jb * 128 + c0 + lane;
+    {
+      float re[32], im[32];
+      tmem_ld16x2(t_addr, 16, re);
+      tmem_ld16x2(t_addr + 128, 16, im);
 #pragma unroll
-      for (int c = 0; c < 64; ++c) stg[lane * 65 + c] = make_float2(re[c], im[c]);
-      __syncwarp();
-#pragma unroll 4
-      for (int t = 0; t < 64; ++t) {
-        const int rr = t >> 1, cc = 32 * (t & 1) + lane;
-        const float2 z = stg[rr * 65 + cc];
-        const long long o = row0 + (long long)rr * N + c0 + cc;
-        if (MODE == 1) {
-          const float2 h = hi[o], l = lo[o];
-          out[o] = make_double2(f2d(h.x) + f2d(l.x) + f2d(z.x), f2d(h.y) + f2d(l.y) + f2d(z.y));
-        } else if (MODE == 2) {
-          const double2 x = out[o];
-          out[o] = make_double2(x.x + f2d(z.x), x.y + f2d(z.y));
-        } else {
-          lo[o] = z;
-        }
+      for (int c = 0; c < 32; ++c) stg[lane * 33 + c] = make_float2(re[c], im[c]);
+    }
+    __syncwarp();
+#pragma unroll 8
+    for (int rr = 0; rr < 32; ++rr) {
+      const float2 z = stg[rr * 33 + lane];
+      const long long o = row0 + (long long)rr * N;
+      if (MODE == 1) {
+        const float2 h = hi[o], l = lo[o];
+        out[o] = make_double2(f2d(h.x) + f2d(l.x) + f2d(z.x), f2d(h.y) + f2d(l.y) + f2d(z.y));
+      } else if (MODE == 2) {
+        const double2 x = out[o];
+        out[o] = make_double2(x.x + f2d(z.x), x.y + f2d(z.y));
+      } else {
+        lo[o] = z;
       }
-      __syncwarp();
     }
   }
   fence_before_sync();
@@ -962,8 +1000,10 @@ __global__ void k_slice_panel_B(const double2* __restrict__ B, long long ms, int
                                 uint16_t* __restrict__ Bsl, int K, int Nc, long long n_thr,
                                 const int* __restrict__ act);
 
-cudaError_t wtc_setup(size_t smem_gj32) {
-  cudaError_t e = raise_smem_limit(k_gj_inverse_f32, smem_gj32);
+cudaError_t wtc_setup() {
+  cudaError_t e = raise_smem_limit(k_gj_inverse_f32<128>, gj32_smem(128));
+  if (e == cudaSuccess) e = raise_smem_limit(k_gj_inverse_f32<256>, gj32_smem(256));
+  if (e == cudaSuccess) e = raise_smem_limit(k_gj_inverse_f32<384>, gj32_smem(384));
   if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX0, kWL0, true, false, kWSA>, w_residual_smem(kWSX0, kWL0));
   if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, true, kWSA>, w_residual_smem(kWSX1, kWLmax));
   if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, true, false, kWSA>, w_residual_smem(kWSX1, kWLmax));
@@ -978,15 +1018,14 @@ cudaError_t wtc_setup(size_t smem_gj32) {
   return e;
 }
 
-void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t smem_gj32, cudaStream_t st,
-                 int refinements) {
+void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, cudaStream_t st, int refinements) {
   const long long NN = (long long)N * N;
   const bool fine = w.weak != nullptr;
   const long long tot = (long long)batch * NN;
   const unsigned g1 = (unsigned)((tot + 255) / 256 < 65535LL * 8 ? (tot + 255) / 256 : 65535LL * 8);
   const long long t8 = tot / 8;  // slicing threads: one per 8 consecutive elements
   const unsigned g8 = (unsigned)((t8 + 255) / 256 < 65535LL * 8 ? (t8 + 255) / 256 : 65535LL * 8);
-  const dim3 gcol((unsigned)((N + 127) / 128), (unsigned)batch);
+  const dim3 gcol((unsigned)((N + 31) / 32), (unsigned)batch);
   const dim3 gres((unsigned)(N / kWTN), (unsigned)(2 * (N / 128)), (unsigned)batch);  // Re rows, then Im rows
   OzProductArgs ga{};
   ga.Asl = w.Asl;
@@ -1010,7 +1049,9 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_gj_inverse_f32", st);
-    k_gj_inverse_f32<<<batch, 512, smem_gj32, st>>>(w.X32, N, NN, w.status, w.weak);
+    if (N == 128) k_gj_inverse_f32<128><<<batch, 512, gj32_smem(N), st>>>(w.X32, NN, w.status, w.weak);
+    else if (N == 256) k_gj_inverse_f32<256><<<batch, 512, gj32_smem(N), st>>>(w.X32, NN, w.status, w.weak);
+    else k_gj_inverse_f32<384><<<batch, 512, gj32_smem(N), st>>>(w.X32, NN, w.status, w.weak);
   }
   // digits of A (kept for both residuals)
   {
@@ -1025,7 +1066,7 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   // R0 = I - A X0 (FP32), lo = X0 R0: X1 = X0 + lo
   {
     gw::TimedLaunch tl_("k_col_exponent", st);
-    k_col_exponent<<<gcol, 128, 0, st>>>(w.X32, nullptr, w.eX, N);
+    k_col_exponent<<<gcol, kCE, 0, st>>>(w.X32, nullptr, w.eX, N);
   }
   {
     gw::TimedLaunch tl_("k_slice_X", st);
@@ -1046,12 +1087,12 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_refine_tc<first>", st);
-    k_refine_tc<0><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, nullptr, N, w.status, act);
+    k_refine_tc<0><<<gref, kPT, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, nullptr, N, w.status, act);
   }
   // R1 = I - A X1 (FP32), X2 = X1 + X0 R1 in FP64, written over A
   {
     gw::TimedLaunch tl_("k_col_exponent", st);
-    k_col_exponent<<<gcol, 128, 0, st>>>(w.X32, w.lo, w.eX, N);
+    k_col_exponent<<<gcol, kCE, 0, st>>>(w.X32, w.lo, w.eX, N);
   }
   {
     gw::TimedLaunch tl_("k_slice_X", st);
@@ -1069,7 +1110,7 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
   }
   {
     gw::TimedLaunch tl_("k_refine_tc<final>", st);
-    k_refine_tc<1><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status, act);
+    k_refine_tc<1><<<gref, kPT, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status, act);
   }
   // the second residual has to be small before its successor is taken modulo 2^64
   if (fine) {
@@ -1092,7 +1133,7 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
     }
     {
       gw::TimedLaunch tl_("k_panel_col_exp", st);
-      k_panel_col_exp<<<dim3((unsigned)((N + 127) / 128), (unsigned)batch), 128, 0, st>>>(mats, NN, N, N, N, w.eX, act);
+      k_panel_col_exp<<<gcol, kCE, 0, st>>>(mats, NN, N, N, N, w.eX, act);
     }
     {
       gw::TimedLaunch tl_("k_slice_panel_B", st);
@@ -1117,7 +1158,7 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t sm
     }
     {
       gw::TimedLaunch tl_("k_refine_tc<add>", st);
-      k_refine_tc<2><<<gref, 128, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status, act);
+      k_refine_tc<2><<<gref, kPT, w_refine_smem(), st>>>(w.PX, w.Xsl, w.X32, w.lo, mats, N, w.status, act);
     }
     if (fine) {
       gw::TimedLaunch tl_("k_mark", st);
@@ -1167,20 +1208,21 @@ __global__ void k_panel_row_exp(const double2* __restrict__ A, long long ms, int
   if (lane == 0) e[row] = m > 0 ? m - 1022 : 0;
 }
 
-// Scale exponent of each column of a K x Nc panel: one thread per column.
-__global__ void k_panel_col_exp(const double2* __restrict__ B, long long ms, int ld, int K, int Nc,
-                                int* __restrict__ e, const int* __restrict__ act) {
-  const int b = blockIdx.y;
+// Scale exponent of each column of a K x Nc panel: blocks as in k_col_exponent.
+__global__ void __launch_bounds__(kCE) k_panel_col_exp(const double2* __restrict__ B, long long ms, int ld, int K, int Nc,
+                                                       int* __restrict__ e, const int* __restrict__ act) {
+  const int b = blockIdx.y, j = blockIdx.x * 32 + (threadIdx.x & 31);
   if (act && !act[b]) return;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= Nc) return;
   const double2* c = B + (long long)b * ms + j;
   int m = 0;
-  for (int k = 0; k < K; ++k) {
-    const double2 z = c[(long long)k * ld];
-    m = max(m, max(exp_field(z.x), exp_field(z.y)));
-  }
-  e[(long long)b * Nc + j] = m > 0 ? m - 1022 : 0;
+  if (j < Nc)
+#pragma unroll 4
+    for (int k = threadIdx.x >> 5; k < K; k += 8) {
+      const double2 z = c[(long long)k * ld];
+      m = max(m, max(exp_field(z.x), exp_field(z.y)));
+    }
+  m = col_max(m);
+  if (threadIdx.x < 32 && j < Nc) e[(long long)b * Nc + j] = m > 0 ? m - 1022 : 0;
 }
 
 // A-operand digits of an M x K panel, chunks as k_slice_A: one per (matrix, 128-row
@@ -1312,7 +1354,7 @@ void panel_gemm(const WblkBuffers& w, const double2* A, long long a_ms, int lda,
   }
   {
     gw::TimedLaunch tl_("k_panel_col_exp", st);
-    k_panel_col_exp<<<dim3((unsigned)((Nc + 127) / 128), (unsigned)batch), 128, 0, st>>>(B, b_ms, ldb, K, Nc, w.eB, nullptr);
+    k_panel_col_exp<<<dim3((unsigned)((Nc + 31) / 32), (unsigned)batch), kCE, 0, st>>>(B, b_ms, ldb, K, Nc, w.eB, nullptr);
   }
   {
     gw::TimedLaunch tl_("k_slice_panel_B", st);
@@ -1357,20 +1399,19 @@ int wblk_block_size(int N) {
   return 0;
 }
 
-cudaError_t wblk_setup(size_t smem_gj32_bs) {
-  cudaError_t e = wtc_setup(smem_gj32_bs);
+cudaError_t wblk_setup() {
+  cudaError_t e = wtc_setup();
   if (e == cudaSuccess) e = raise_smem_limit(k_oz_product<kWSX1, kWLmax, false, false, kWSA>, w_residual_smem(kWSX1, kWLmax));
   return e;
 }
 
-void wblk_inverse(const WblkBuffers& w, double2* mats, int batch, int N, int bs, size_t smem_gj32_bs,
-                  cudaStream_t st) {
+void wblk_inverse(const WblkBuffers& w, double2* mats, int batch, int N, int bs, cudaStream_t st) {
   const long long NN = (long long)N * N, BB = (long long)bs * bs, BN = (long long)bs * N;
   for (int k = 0; k < N / bs; ++k) {
     const int r0 = k * bs;
     // D = A_kk^-1
     copy_panel(mats + (long long)r0 * N + r0, NN, N, w.D, BB, bs, bs, bs, batch, 0, st);
-    wtc_inverse(w.inner, w.D, batch, bs, smem_gj32_bs, st, kWblkRefinements);
+    wtc_inverse(w.inner, w.D, batch, bs, st, kWblkRefinements);
     // Rp = D A_k,: with block k = I + D
     panel_gemm(w, w.D, BB, bs, mats + (long long)r0 * N, NN, N, w.Rp, BN, N, bs, N, bs, batch, 0, 0, 0, st);
     copy_panel(w.D, BB, bs, w.Rp + r0, BN, N, bs, bs, batch, 1, st);

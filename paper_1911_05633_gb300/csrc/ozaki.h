@@ -51,7 +51,8 @@ __device__ __forceinline__ int next_digit(long long& m, int s) {
 // bits of d 2^-7(s+1) in BF16 (exact)
 __device__ __forceinline__ uint32_t digit_bf16(int d, int s) {
   const float sc = __int_as_float((127 - 7 * (s + 1)) << 23);
-  return __float_as_uint((float)d * sc) >> 16;
+  const float f = __int_as_float(0x4B400000 + d) - 12582912.0f;  // d as a float (a conversion runs at the FP64 rate)
+  return __float_as_uint(f * sc) >> 16;
 }
 
 

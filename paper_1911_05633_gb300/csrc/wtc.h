@@ -29,6 +29,7 @@ __host__ __device__ constexpr size_t w_residual_smem(int SX, int lmax) {
 }
 
 constexpr int kGJ32B = 32;    // panel width of the FP32 Gauss-Jordan inverse
+constexpr int kGJ32P = kGJ32B + 2;  // its row stride in shared memory: 16-byte columns of eight rows in eight bank groups
 constexpr int kGJ32C = 128;   // column chunk of its trailing update
 // float2 elements of the multi-use buffer (pivot rows, exchange staging, row copies)
 __host__ __device__ constexpr size_t gj32_buf_elems(int N) {
@@ -36,10 +37,8 @@ __host__ __device__ constexpr size_t gj32_buf_elems(int N) {
 }
 // dynamic shared memory of k_gj_inverse_f32
 __host__ __device__ constexpr size_t gj32_smem(int N) {
-  return ((size_t)N * kGJ32B + gj32_buf_elems(N)) * 8 + ((size_t)2 * N + 4 * kGJ32B) * 4;
+  return ((size_t)N * kGJ32P + gj32_buf_elems(N)) * 8 + ((size_t)2 * N + 4 * kGJ32B) * 4;
 }
-__global__ void k_gj_inverse_f32(float2* __restrict__ A, int N, long long mat_stride, int* __restrict__ status,
-                                 int* __restrict__ weak);
 __global__ void k_to_f32(const double2* __restrict__ src, float2* __restrict__ dst, long long n, long long NN,
                          const int* __restrict__ act);
 __global__ void k_row_exponent(const double2* __restrict__ A, int* __restrict__ eA, int N, int batch);
@@ -73,7 +72,7 @@ struct WtcBuffers {
 };
 
 // Raise the shared-memory limits of the kernels (once per device and size).
-cudaError_t wtc_setup(size_t smem_gj32);
+cudaError_t wtc_setup();
 
 // ---- block Gauss-Jordan for N beyond kWNmax (kernels_wtc.cu) ----------------------
 // Arguments of k_oz_product: the digits of an M x K and a K x Nc matrix (M a multiple of
@@ -115,14 +114,12 @@ constexpr int kWblkMaxK = 256;
 // Pivot block size for N (the largest multiple of 128 up to kWblkMaxK dividing N), or 0
 // when N needs no blocks (N <= kWNmax) or has none (N not a multiple of 128).
 int wblk_block_size(int N);
-cudaError_t wblk_setup(size_t smem_gj32_bs);
+cudaError_t wblk_setup();
 // In place: mats[b] (FP64, N x N, Hermitian positive definite or with well-conditioned
 // leading blocks) -> inverse, for b < batch; bs = wblk_block_size(N).
-void wblk_inverse(const WblkBuffers& w, double2* mats, int batch, int N, int bs, size_t smem_gj32_bs,
-                  cudaStream_t st);
-// In place: mats[b] (FP64, N x N, N a multiple of 128) -> inverse, for b < batch, with
+void wblk_inverse(const WblkBuffers& w, double2* mats, int batch, int N, int bs, cudaStream_t st);
+// In place: mats[b] (FP64, N x N, N = 128, 256 or 384) -> inverse, for b < batch, with
 // `refinements` (at least 2) FP64-accurate refinements of the FP32 inverse.
-void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, size_t smem_gj32, cudaStream_t st,
-                 int refinements = 2);
+void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, cudaStream_t st, int refinements = 2);
 
 }  // namespace gw

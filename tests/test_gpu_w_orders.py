@@ -2,6 +2,7 @@
 identity) against the FP64 Gauss-Jordan solve of the same plan inputs: one below the first
 order it takes, the first, odd ones on both sides of a tile, the largest; and inputs it hands
 to the FP64 inverse: a v(q) too ill-conditioned for the FP32 start, and scales outside FP32.
+A reversed identity for v(q) makes every column of the FP32 start change rows.
 
 Tolerance: both solves are FP64-accurate, kappa(v) eps N < 1e3 1e-16 4e2 = 4e-11 < 1e-10.  For
 the ill-conditioned v both are FP64 eliminations with error kappa eps sqrt(N) = 1e7 1.1e-16 14
@@ -22,7 +23,10 @@ def _plans(n_prod, **kw):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_1911_05633_gb300 import gw
-    cell = synth.mixed_species_cell(n_tau=10, n_orb=(4, 5), n_prod=n_prod, kmesh=(2, 2, 1))
+    if n_prod == "8 atoms":
+        cell = synth.make_config(1, kmesh=(2, 1, 1), n_tau=12)  # N_PB 384
+    else:
+        cell = synth.mixed_species_cell(n_tau=10, n_orb=(4, 5), n_prod=n_prod, kmesh=(2, 2, 1))
     G = dev(cell.green_k_tau())
     a, b = gw.Plan.from_cell(cell, **kw), gw.Plan.from_cell(cell, w_solver="gauss_jordan", **kw)
     P = a.transform_tau_iw("B", "tau_to_iw", "pb", a.polarizability_tau(a.green_k_to_R(G)))
@@ -55,3 +59,18 @@ def test_left_to_the_fp64_inverse(low, scale, bound):
     ref = host(b.screened_W_iw(P, vq))
     b.sync()
     assert np.isfinite(W).all() and rel(W, ref) < bound
+
+
+@pytest.mark.parametrize("n_prod", [(64, 64), (100, 101), (128, 128), "8 atoms"])
+def test_every_pivot_off_the_diagonal(n_prod):
+    cell, a, b, P = _plans(n_prod)
+    rng = np.random.default_rng(4)
+    N = cell.n_pb_total
+    v = np.eye(N)[::-1] + (lambda x: x + x.T)(0.02 / np.sqrt(N) * rng.standard_normal((N, N)))
+    vq = dev(np.broadcast_to(v, (cell.n_k, N, N)))
+    P = P * (0.1 / P.abs().max().item())  # v^-1 - P: a reversed identity and a small rest
+    W = host(a.screened_W_iw(P, vq))
+    a.sync()
+    ref = host(b.screened_W_iw(P, vq))
+    b.sync()
+    assert rel(W, ref) < TOL
