@@ -185,81 +185,112 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_oz_transform(const __grid_con
   if (warp < kTfSlicerWarps) {
     // ---- slicers: row r of the tile, K half h of every 16-wide step ----
     const int r = 16 * warp + (lane & 15), h = lane >> 4;
-    int step = 0;
-    bool ok = true;
-    for (int i = 0; i < my_tiles && ok; ++i) {
-      const int t = (int)blockIdx.x + i * (int)gridDim.x;
+    struct Row {          // this thread's row of a tile
+      const double2* src;  // its slice 0
+      long long blk;       // elements from one slice to the next
+      bool valid;
+    };
+    auto row_of = [&](int i) {
       DevEntry E;
       long long blk, base;
       int r0, ct;
-      entry_of(t, E, blk, base, r0, ct);
-      const long long x = r0 + r;
-      const bool valid = x < blk;
-      if (warp == 0 && lane == 0 && i + 1 < my_tiles) {
-        // the next tile's input, into L2 while this one is cut
-        DevEntry En;
-        long long bn, basen;
-        int rn, ctn;
-        entry_of(t + (int)gridDim.x, En, bn, basen, rn, ctn);
-        const uint32_t bytes = (uint32_t)(min(128ll, bn - rn) * 16);
-        const int ns = g.real_in ? g.K : (g.K + 1) / 2;
-        for (int k = 0; k < ns; ++k) prefetch_l2(g.in + basen * g.n_in + k * bn + rn, bytes);
-      }
-      const double2* src = g.in + base * g.n_in + x;
-      // the 8 values of this thread in K step ks
-      auto load8 = [&](int ks, double* w) {
-        if (g.real_in) {
+      entry_of((int)blockIdx.x + i * (int)gridDim.x, E, blk, base, r0, ct);
+      return Row{g.in + base * g.n_in + r0 + r, blk, r0 + r < blk};
+    };
+    // the 8 values of this thread in K step ks
+    auto load8 = [&](const Row& R, int ks, double* w) {
+      if (g.real_in) {
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int k = ks * 16 + 8 * h + u;
-            w[u] = (valid && k < g.K) ? reinterpret_cast<const double*>(src + k * blk)[0] : 0.0;
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int sl = ks * 8 + 4 * h + j;  // values 2 sl, 2 sl + 1
-            double2 p = make_double2(0.0, 0.0);
-            if (valid && 2 * sl < g.K) p = src[sl * blk];
-            w[2 * j] = p.x;
-            w[2 * j + 1] = p.y;
-          }
+        for (int u = 0; u < 8; ++u) {
+          const int k = ks * 16 + 8 * h + u;
+          w[u] = (R.valid && k < g.K) ? reinterpret_cast<const double*>(R.src + k * R.blk)[0] : 0.0;
         }
-      };
-      // one K step cut into its stage: the digit planes of 8 values of this thread
-      auto cut = [&](const double* w, int e, int st) {
-        unsigned char* A = As + st * kTfAStage + kmajor_offset(128, r, 8 * h);
-        long long M[8];
+      } else {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) M[u] = fixed56(w[u], e);
-        tf_cut8(M, A);
-        fence_smem_to_async();
-        mbar_arrive(&a_full[st]);
-      };
-      // the scale pass, one K step at a time; the cut reads the values again (from L2)
-      int mx = 0;
+        for (int j = 0; j < 4; ++j) {
+          const int sl = ks * 8 + 4 * h + j;  // values 2 sl, 2 sl + 1
+          double2 p = make_double2(0.0, 0.0);
+          if (R.valid && 2 * sl < g.K) p = R.src[sl * R.blk];
+          w[2 * j] = p.x;
+          w[2 * j + 1] = p.y;
+        }
+      }
+    };
+    // their high words, for the row's scale
+    auto load8_hi = [&](const Row& R, int ks, int* w) {
+      if (g.real_in) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int k = ks * 16 + 8 * h + u;
+          w[u] = (R.valid && k < g.K) ? reinterpret_cast<const int*>(R.src + k * R.blk)[1] : 0;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int sl = ks * 8 + 4 * h + j;
+          const bool in = R.valid && 2 * sl < g.K;
+          w[2 * j] = in ? reinterpret_cast<const int*>(R.src + sl * R.blk)[1] : 0;
+          w[2 * j + 1] = in ? reinterpret_cast<const int*>(R.src + sl * R.blk)[3] : 0;
+        }
+      }
+    };
+    auto max8 = [&](const int* w, int mx) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) mx = max(mx, (w[u] >> 20) & 0x7ff);
+      return mx;
+    };
+    // one K step cut into its stage: the digit planes of 8 values of this thread
+    auto cut = [&](const double* w, int e, int st) {
+      unsigned char* A = As + st * kTfAStage + kmajor_offset(128, r, 8 * h);
+      long long M[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) M[u] = fixed56(w[u], e);
+      tf_cut8(M, A);
+      fence_smem_to_async();
+      mbar_arrive(&a_full[st]);
+    };
+    int step = 0, mx = 0;
+    bool ok = true;
+    Row R{};
+    if (my_tiles > 0) {
+      R = row_of(0);
 #pragma unroll 1
       for (int ks = 0; ks < KS; ++ks) {
-        double w[8];
-        load8(ks, w);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) mx = max(mx, exp_field(w[u]));
+        int w[8];
+        load8_hi(R, ks, w);
+        mx = max8(w, mx);
       }
+    }
+    for (int i = 0; i < my_tiles && ok; ++i) {
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
       const int e = mx > 0 ? mx - 1022 : 0;
+      Row Rn = R;
+      Rn.valid = false;
+      if (i + 1 < my_tiles) Rn = row_of(i + 1);
       const int b = i & 1;
       ok = mbar_wait(&e_empty[b], (uint32_t)((i >> 1) & 1) ^ 1u, kTfWaitNs, g.status);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       if (h == 0) eA_s[b][r] = e;
       mbar_arrive(&e_full[b]);
+      // The tile is cut while the next one's scales are taken, so that its loads, from DRAM, have
+      // the whole step to come in and the cut's own find the tile in L2.  (With the scale pass of
+      // its own, fed by bulk prefetches that one lane issued for its whole warp, three transforms
+      // of the 16-atom cell took 4.20 ms; prefetches spread over the warps 3.52, this 3.31; with
+      // prefetches two tiles ahead as well 3.48, with the cut's loads a step ahead 3.44.)
+      mx = 0;
 #pragma unroll 1
       for (int ks = 0; ks < KS; ++ks, ++step) {
         double w[8];
-        load8(ks, w);
+        int wn[8];
+        load8(R, ks, w);
+        load8_hi(Rn, ks, wn);
         const int st = step % kTfStages;
         ok = mbar_wait(&a_empty[st], (uint32_t)((step / kTfStages) & 1) ^ 1u, kTfWaitNs, g.status);
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         cut(w, e, st);
+        mx = max8(wn, mx);
       }
+      R = Rn;
     }
     if (!ok) atomicExch(g.status, 2);
   } else if (warp == kTfMmaWarp) {
