@@ -168,11 +168,13 @@ def contraction_flops(cell, entries, kdims) -> float:
     return f * cell.n_tau
 
 
-def kernel_work(name: str, cell, info, entries, kdims):
+def kernel_work(name: str, cell, info, entries, kdims, chain=False):
     """Algorithmic work of one sweep for the kernels that can dominate it: (bound,
     work, kind, units) with flops for "alu"/"tensor" (real flops) and bytes for "hbm",
     and `units` the matrices (W solve) or pair entries the sweep processes; None for
-    the others.  Per launch = this / launches per sweep."""
+    the others.  Per launch = this / launches per sweep.  chain: the FP64 contractions ran
+    over symmetric orbital pairs (k_chain), which leaves n_a^2 n_b^2 complex multiply-adds
+    per (entry, node) in FP64 arithmetic."""
     N = cell.n_pb_total
     nq = info["n_q_solved"]
     nnu = int((cell.nu_idx >= 0).sum()) if info["w_symmetric"] else cell.nu_idx.size
@@ -189,6 +191,10 @@ def kernel_work(name: str, cell, info, entries, kdims):
         return "tensor", 4 * 20 * 2.0 * N ** 3 * n_inv, "bf16", n_inv
     if name == "k_ozaki_residual<second>":  # 36 slice pairs
         return "tensor", 4 * 36 * 2.0 * N ** 3 * n_inv, "bf16", n_inv
+    if chain and name in ("k_polarizability_fp64", "k_self_energy_fp64"):
+        slices = (nt + 1) // 2 if name == "k_polarizability_fp64" else nt + 1  # Sigma: and the exchange's one
+        pairs = sum((cell.n_orb_of(int(a)) * cell.n_orb_of(int(b))) ** 2 for a, b in entries[:, :2])
+        return "alu", 8.0 * pairs * slices, "fp64", len(entries)
     if name == "k_polarizability_fp64":  # stages 1 and 2 only when stage 3 runs on the tensor cores
         f = stage_bc_flops(cell, entries, kdims) if info["p_tensor"] else contraction_flops(cell, entries, kdims)
         return "alu", f / (2 if info["c_symmetric"] else 1), "fp64", len(entries)
@@ -520,9 +526,10 @@ def dominant_contraction_roofline(kt, steps, cell, plan, peaks, fp32_peak, fp64_
     if mixed:
         work = row_work(cell, ent, kd, row, inf["c_symmetric"])
     else:  # the FP64 kernel does the small stages; its dense stage runs as digit GEMMs
-        w = kernel_work(k, cell, inf, ent, kd)
+        w = kernel_work(k, cell, inf, ent, kd, chain="k_chain" in kt)
         fl = w[1]
-        byt = row_work(cell, ent, kd, row, inf["c_symmetric"])[1]
+        # over orbital pairs the rows' DRAM traffic is the other kernels', k_chain's above all
+        byt = 0.0 if "k_chain" in kt else row_work(cell, ent, kd, row, inf["c_symmetric"])[1]
         work = (fl, byt, 0.0, fl)
     ms, nl = cands[k]
     roof = contraction_roofline(k, ms / steps, nl / steps, work, peaks, fp32_peak, fp64_peak, mixed)
@@ -785,7 +792,7 @@ def dominant_kernel_roofline(kt, steps, cell, plan, peaks, fp32_peak, fp64_peak)
         return None
     dom_k = max(kt, key=lambda k: kt[k][0])
     ms_tot, nl = kt[dom_k]
-    w = kernel_work(dom_k, cell, plan.info, plan.entries, pb_dims(plan))
+    w = kernel_work(dom_k, cell, plan.info, plan.entries, pb_dims(plan), chain="k_chain" in kt)
     if w is None:
         return {"kernel": dom_k, "bound": None}
     bound, work, kind, units = w
