@@ -139,8 +139,8 @@ struct DeviceGuard {
 // Orders N_PB that the tensor-core inverse takes beside an identity, and the refinements there:
 // the third and, where it is needed, the fourth have residuals to nine digits, for the error
 // of an FP64 elimination or less.  The line: 196 matrices in two batches, W solve of N = 80 2.34 ms
-// against 1.82 by the FP64 inverse in shared memory, N = 96 2.39 against 3.18, 120 2.55 against
-// 9.33, 136 (in 256) 8.34 against 13.2, 200 8.79 against 34.2, 288 (in 384) 21.8 against 83.7.
+// against 1.82 by the FP64 inverse in shared memory, N = 96 1.81 against 3.18, 120 2.13 against
+// 9.33, 136 (in 256) 5.92 against 13.2, 200 7.03 against 34.2, 288 (in 384) 16.9 against 83.8.
 constexpr int kPadMinN = 88;
 constexpr int kPadRefinements = 4;
 // Scratch of the tensor-core inverse per matrix element: three FP32 arrays, the digit planes
@@ -329,7 +329,7 @@ gw_status launch_tensor_inverse(gw_plan_s* p, double2* mats, int batch, long lon
     w.act = p->t_act;
     w.perm = p->d_perm;
   }
-  gw::wtc_inverse(w, mats, batch, (int)N, st, p->w_pad ? kPadRefinements : 2);
+  gw::wtc_inverse(w, mats, batch, (int)N, st, p->w_pad ? kPadRefinements : 2, (int)p->h.n_pb_total());
   return check_launch("tensor-core inverse");
 }
 

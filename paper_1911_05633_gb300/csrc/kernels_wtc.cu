@@ -28,16 +28,14 @@ __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
   return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
 }
 
-// Barrier of the first N threads of the block (whole warps).
-template <int N>
-__device__ __forceinline__ void rows_barrier() {
-  asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
-}
+// Barrier of the first n threads of the block (whole warps).
+__device__ __forceinline__ void rows_barrier(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 
 }  // namespace
 
 // In-place FP32 Gauss-Jordan inverse with partial pivoting, one 512-thread block per
-// matrix (N = 128, 256 or 384).  A panel of kGJ32B columns is reduced with one row per thread
+// matrix (N = 128, 256 or 384; from row and column Na, a multiple of kGJ32B, on the matrix is an
+// identity and is left alone).  A panel of kGJ32B columns is reduced with one row per thread
 // in registers: the pivot row, scaled by its warp, is the only operand that passes through
 // shared memory, as broadcasts.  The registers rotate by one column per step (the loop stays
 // rolled), so the column being eliminated is always v[0].  The row exchanges and the
@@ -48,9 +46,11 @@ __device__ __forceinline__ void rows_barrier() {
 // paired fma.rn.f32x2 needs its operands copied and swapped and took 3.7 M), 1.0 M the panels,
 // bound by the chain pivot - scaled row - update of each column (1.7 M with the panel in shared
 // memory, and the same with a warp per row and shuffles).  900 matrices: 13.0 ms, 16.8 before.
+// 196 matrices of order 288 in 384: 3.4 ms, 5.5 with the identity eliminated too.
 template <int N>
 __global__ void __launch_bounds__(512, 1)
-k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__ status, int* __restrict__ weak) {
+k_gj_inverse_f32(float2* __restrict__ A, int Na, long long mat_stride, int* __restrict__ status,
+                 int* __restrict__ weak) {
   constexpr int B = kGJ32B, C = kGJ32C, P = kGJ32P;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* Pan = reinterpret_cast<float2*>(smraw);  // [N][P], columns 0 .. B - 1 used
@@ -65,10 +65,10 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
   __shared__ int nx;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   float2* M = A + (long long)blockIdx.x * mat_stride;
-  for (int k0 = 0; k0 < N; k0 += B) {
-    for (int x = tid; x < N * B; x += 512) Pan[(x / B) * P + x % B] = M[(long long)(x / B) * N + k0 + (x % B)];
+  for (int k0 = 0; k0 < Na; k0 += B) {
+    for (int x = tid; x < Na * B; x += 512) Pan[(x / B) * P + x % B] = M[(long long)(x / B) * N + k0 + (x % B)];
     __syncthreads();
-    if (tid < N) {  // whole warps
+    if (tid < Na) {  // whole warps
       float2 v[B];  // row tid; column k0 + (m + j) % B at step m
 #pragma unroll
       for (int j = 0; j < B; j += 2) {
@@ -85,8 +85,8 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
         const unsigned wkey = __reduce_max_sync(0xffffffffu, key);
         const unsigned wbal = __ballot_sync(0xffffffffu, key == wkey);
         if (lane == 0) { cand_v[wid] = wkey; cand_i[wid] = 32 * wid + __ffs(wbal) - 1; }
-        rows_barrier<N>();
-        const unsigned ckey = lane < N / 32 ? cand_v[lane] : 0u;
+        rows_barrier(Na);
+        const unsigned ckey = lane < Na / 32 ? cand_v[lane] : 0u;
         const unsigned best = __reduce_max_sync(0xffffffffu, ckey);
         const unsigned cbal = __ballot_sync(0xffffffffu, ckey == best);
         const int p = best ? cand_i[__ffs(cbal) - 1] : k;
@@ -111,7 +111,7 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
           for (int j = 0; j < B; j += 2)
             *reinterpret_cast<float4*>(oldk_s + j) = make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y);
         }
-        rows_barrier<N>();
+        rows_barrier(Na);
         // rows k and p exchanged and every other row updated, one column to the left
         if (tid == p) {
 #pragma unroll
@@ -144,13 +144,13 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
       }
     }
     __syncthreads();
-    for (int x = tid; x < N * B; x += 512) {
+    for (int x = tid; x < Na * B; x += 512) {
       const int i = x / B, j = x % B;
       const float2 z = Pan[i * P + j];
       M[(long long)i * N + k0 + j] = make_float2(z.x + (i == k0 + j ? 1.0f : 0.0f), z.y);
     }
     // composite row exchange of this panel: new row r = old row srcmap[r]
-    for (int i = tid; i < N; i += 512) srcmap[i] = i;
+    for (int i = tid; i < Na; i += 512) srcmap[i] = i;
     __syncthreads();
     if (wid == 0) {
       if (lane == 0)
@@ -161,9 +161,9 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
       __syncwarp();
       // the moved rows (at most 2B), compacted in row order
       int n = 0;
-      for (int r0 = k0; r0 < N; r0 += 32) {
+      for (int r0 = k0; r0 < Na; r0 += 32) {
         const int r = r0 + lane;
-        const bool mv = r < N && srcmap[r] != r;
+        const bool mv = srcmap[r] != r;
         const unsigned bal = __ballot_sync(0xffffffffu, mv);
         const int pos = n + __popc(bal & ((1u << lane) - 1u));
         if (mv && pos < 2 * B) { xdst[pos] = r; xsrc[pos] = srcmap[r]; }
@@ -173,7 +173,7 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
     }
     __syncthreads();
     const int n = nx;
-    for (int c0 = 0; c0 < N; c0 += C) {
+    for (int c0 = 0; c0 < Na; c0 += C) {  // (whole chunks: N is a multiple of C)
       const bool has_panel = k0 >= c0 && k0 < c0 + C;
       // (a) the row exchange on this chunk's other columns, staged through shared memory
       for (int x = tid; x < n * C; x += 512) {
@@ -191,7 +191,7 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
       __syncthreads();
       // (c) rows i0 .. i0 + 7, columns c0 + lane + 32 q: 32 independent loads in flight per
       // thread, then 8 x 4 complex FMAs per pair of shared-memory vectors (z, pv)
-      for (int i0 = 8 * wid; i0 < N; i0 += 8 * 16) {
+      for (int i0 = 8 * wid; i0 < Na; i0 += 8 * 16) {
         float2 acc[8][4];
 #pragma unroll
         for (int r = 0; r < 8; ++r)
@@ -226,20 +226,20 @@ k_gj_inverse_f32(float2* __restrict__ A, long long mat_stride, int* __restrict__
   }
   // undo the pivoting on the columns: new column j = old column srcmap[j], the composite
   // of the swaps (k, pm[k]) for k = N-1 down to 0
-  for (int i = tid; i < N; i += 512) srcmap[i] = i;
+  for (int i = tid; i < Na; i += 512) srcmap[i] = i;
   __syncthreads();
   if (tid == 0)
-    for (int k = N - 1; k >= 0; --k) {
+    for (int k = Na - 1; k >= 0; --k) {
       const int p = pm[k];
       if (p != k) { const int t = srcmap[k]; srcmap[k] = srcmap[p]; srcmap[p] = t; }
     }
   __syncthreads();
   float2* rb = Buf + (size_t)wid * N;
-  for (int i = wid; i < N; i += 16) {
+  for (int i = wid; i < Na; i += 16) {
     float2* Mi = M + (long long)i * N;
-    for (int j = lane; j < N; j += 32) rb[j] = Mi[j];
+    for (int j = lane; j < Na; j += 32) rb[j] = Mi[j];
     __syncwarp();
-    for (int j = lane; j < N; j += 32) Mi[j] = rb[srcmap[j]];
+    for (int j = lane; j < Na; j += 32) Mi[j] = rb[srcmap[j]];
     __syncwarp();
   }
 }
@@ -1018,8 +1018,9 @@ cudaError_t wtc_setup() {
   return e;
 }
 
-void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, cudaStream_t st, int refinements) {
+void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, cudaStream_t st, int refinements, int n) {
   const long long NN = (long long)N * N;
+  const int Na = n > 0 ? (n + kGJ32B - 1) / kGJ32B * kGJ32B : N;
   const bool fine = w.weak != nullptr;
   const long long tot = (long long)batch * NN;
   const unsigned g1 = (unsigned)((tot + 255) / 256 < 65535LL * 8 ? (tot + 255) / 256 : 65535LL * 8);
@@ -1049,9 +1050,9 @@ void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, cudaStrea
   }
   {
     gw::TimedLaunch tl_("k_gj_inverse_f32", st);
-    if (N == 128) k_gj_inverse_f32<128><<<batch, 512, gj32_smem(N), st>>>(w.X32, NN, w.status, w.weak);
-    else if (N == 256) k_gj_inverse_f32<256><<<batch, 512, gj32_smem(N), st>>>(w.X32, NN, w.status, w.weak);
-    else k_gj_inverse_f32<384><<<batch, 512, gj32_smem(N), st>>>(w.X32, NN, w.status, w.weak);
+    if (N == 128) k_gj_inverse_f32<128><<<batch, 512, gj32_smem(N), st>>>(w.X32, Na, NN, w.status, w.weak);
+    else if (N == 256) k_gj_inverse_f32<256><<<batch, 512, gj32_smem(N), st>>>(w.X32, Na, NN, w.status, w.weak);
+    else k_gj_inverse_f32<384><<<batch, 512, gj32_smem(N), st>>>(w.X32, Na, NN, w.status, w.weak);
   }
   // digits of A (kept for both residuals)
   {

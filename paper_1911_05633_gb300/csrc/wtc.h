@@ -120,6 +120,8 @@ cudaError_t wblk_setup();
 void wblk_inverse(const WblkBuffers& w, double2* mats, int batch, int N, int bs, cudaStream_t st);
 // In place: mats[b] (FP64, N x N, N = 128, 256 or 384) -> inverse, for b < batch, with
 // `refinements` (at least 2) FP64-accurate refinements of the FP32 inverse.
-void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, cudaStream_t st, int refinements = 2);
+// n: order of the matrices within an identity of order N (0: N).
+void wtc_inverse(const WtcBuffers& w, double2* mats, int batch, int N, cudaStream_t st, int refinements = 2,
+                 int n = 0);
 
 }  // namespace gw
