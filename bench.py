@@ -44,8 +44,8 @@ UNIT = "sweep/s"
 # in this launch.
 TRAFFIC = {
     # bench.py --small captures (56 matrices of N_PB = 384 per launch): DRAM read + write / 56
-    "k_gj_inverse_f32": {"file": "kernels_wtc.cu", "src_sha": "818f6fc1dcc6cb59",
-                         "bytes_per_unit": (66.10e6 + 254.12e6) / 56},
+    "k_gj_inverse_f32": {"file": "kernels_wtc.cu", "src_sha": "f6d43d35fd0a1278",
+                         "bytes_per_unit": (66.11e6 + 264.68e6) / 56},
     # bench.py --atoms 8 captures (profiles/k_contract_diamond8_small.md): 352 entries of the
     # same species as the 72-atom cell; units are (entry, node) pairs: 352 x 64 for Sigma,
     # 352 x 32 computed nodes for P (each writing its node and the mirrored one)

@@ -138,9 +138,9 @@ struct DeviceGuard {
 
 // Orders N_PB that the tensor-core inverse takes beside an identity, and the refinements there:
 // the third and, where it is needed, the fourth have residuals to nine digits, for the error
-// of an FP64 elimination or less.  The line: 196 matrices in two batches, W solve of N = 80 2.34 ms
-// against 1.82 by the FP64 inverse in shared memory, N = 96 1.81 against 3.18, 120 2.13 against
-// 9.33, 136 (in 256) 5.92 against 13.2, 200 7.03 against 34.2, 288 (in 384) 16.9 against 83.8.
+// of an FP64 elimination or less.  The line: 196 matrices in two batches, W solve of N = 64 2.19 ms
+// against 1.64 by the FP64 inverse in shared memory, N = 80 1.77 against 1.82, N = 96 1.81 against
+// 3.18, 120 2.13 against 9.33, 136 (in 256) 5.92 against 13.2, 200 7.03 against 34.2, 288 (in 384) 16.9 against 83.8.
 constexpr int kPadMinN = 88;
 constexpr int kPadRefinements = 4;
 // Scratch of the tensor-core inverse per matrix element: three FP32 arrays, the digit planes

@@ -46,7 +46,7 @@ __device__ __forceinline__ void rows_barrier(int n) { asm volatile("bar.sync 1, 
 // paired fma.rn.f32x2 needs its operands copied and swapped and took 3.7 M), 1.0 M the panels,
 // bound by the chain pivot - scaled row - update of each column (1.7 M with the panel in shared
 // memory, and the same with a warp per row and shuffles).  900 matrices: 13.0 ms, 16.8 before.
-// 196 matrices of order 288 in 384: 3.4 ms, 5.5 with the identity eliminated too.
+// 196 matrices of order 288 in 384: 3.5 ms, 5.5 with the identity eliminated too.
 template <int N>
 __global__ void __launch_bounds__(512, 1)
 k_gj_inverse_f32(float2* __restrict__ A, int Na, long long mat_stride, int* __restrict__ status,
