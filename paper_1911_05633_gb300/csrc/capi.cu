@@ -770,7 +770,7 @@ gw_status gw_fourier_k_to_R(gw_plan_t p, gw_block kind, int n_slices, const void
   gw::ActiveTimer timing(&p->timer);
   if (lattice_takes(p, kind, n_slices))
     return gw::lattice_run(p->lattice, p->h, p->d_ent, kind == GW_BLOCK_PB ? p->d_pb_off : p->d_orb_off,
-                           kind == GW_BLOCK_PB, n_slices, false, (double2*)const_cast<void*>(F_k), (double2*)F_R,
+                           p->d_phase, kind == GW_BLOCK_PB, n_slices, false, (double2*)const_cast<void*>(F_k), (double2*)F_R,
                            p->d_status, S(stream));
   const long long N = dense_n(p, kind);
   return launch_gather(p, kind, n_slices, (const double2*)F_k, (long long)n_slices * N * N, N * N, nullptr, 0, 0,
@@ -790,7 +790,7 @@ gw_status gw_fourier_R_to_k(gw_plan_t p, gw_block kind, int n_slices, const void
   gw::ActiveTimer timing(&p->timer);
   if (lattice_takes(p, kind, n_slices))
     return gw::lattice_run(p->lattice, p->h, p->d_ent, kind == GW_BLOCK_PB ? p->d_pb_off : p->d_orb_off,
-                           kind == GW_BLOCK_PB, n_slices, true, (double2*)F_k, (double2*)const_cast<void*>(F_R),
+                           p->d_phase, kind == GW_BLOCK_PB, n_slices, true, (double2*)F_k, (double2*)const_cast<void*>(F_R),
                            p->d_status, S(stream));
   const long long N = dense_n(p, kind);
   return launch_scatter(p, kind, n_slices, (const double2*)F_R, n_slices, 0, (double2*)F_k,

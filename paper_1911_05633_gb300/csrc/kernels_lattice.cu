@@ -33,6 +33,13 @@ constexpr int kLtWarps = 8;                           // slicer warps, and as ma
 constexpr int kLtThreads = 32 * (2 * kLtWarps + 1);   // and one that issues the products
 constexpr int kLtStages = 3;
 constexpr uint32_t kLtStep = kOzDigits * kTfPlane;    // 32 KB: digits of 128 rows, one K step
+// Rows that the digits hold: the largest exponent field of a row within these.  A sum is a
+// multiple of 2^(e - 61) for the row's scale 2^e (2^-56 of it times the smallest column scale,
+// 2^-5 at 32 points) and below 2^(e + 7), so that these keep it a normal double, and what the
+// digits drop of such a row, its subnormal values, is below 2^-62 of it.  Any other row that
+// is not all zero (G(tau) far from both ends at low temperature) is summed in FP64.
+constexpr int kLtLow = 64, kLtHigh = 2032;
+constexpr int kLtDirect = 1 << 20;                    // in place of such a row's scale exponent
 
 struct LatArgs {
   const DevEntry* ent;
@@ -45,6 +52,7 @@ struct LatArgs {
   const uint16_t* B;       // static operands
   const long long* B_off;  // [n_active] offset of a pair's operand (uint16 units)
   const int* eB;           // [n_active][64]
+  const double2* phase;    // [E][n_k] e^{+i k.R}
   int tiles_per_block;
   int* status;
 };
@@ -150,10 +158,20 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
         for (int u = 0; u < 8; ++u) mx = max(mx, exp_field(w[ks][u]));
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
       const int e = mx > 0 ? mx - 1022 : 0;
+      bool direct = mx > kLtHigh && mx < 2047;
+      if (__any_sync(0xffffffffu, mx < kLtLow)) {
+        unsigned long long any = 0;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+          for (int u = 0; u < 8; ++u) any |= (unsigned long long)__double_as_longlong(w[ks][u]) << 1;
+        const unsigned with = __ballot_sync(0xffffffffu, any != 0);  // lanes r and r + 16 hold a row's halves
+        if (mx < kLtLow && ((with >> (lane & 15)) & 0x10001u)) direct = true;
+      }
       const int it = t - t0, b = it & 1;
       ok = mbar_wait(&e_empty[b], (uint32_t)((it >> 1) & 1) ^ 1u, kLtWaitNs, g.status);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      if (h == 0) eA_s[b][r] = e;
+      if (h == 0) eA_s[b][r] = direct ? kLtDirect : e;
       mbar_arrive(&e_full[b]);
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
@@ -249,6 +267,24 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
           mbar_arrive(&t_empty[bf]);
         }
         if (!valid) continue;
+        if (ea == kLtDirect) {
+          for (int m = 8 * c; m < min(8 * c + 8, n_out); ++m) {
+            if (!SCATTER && !(i < re_s[m] && j < ce_s[m])) continue;
+            double2 a = make_double2(0.0, 0.0);
+            for (int q2 = 0; q2 < n_in; ++q2) {
+              if (SCATTER && !(i < re_s[q2] && j < ce_s[q2])) continue;
+              const double2 v = SCATTER ? g.entries[off_s[q2] + (long long)s * re_s[q2] * ce_s[q2] + i * ce_s[q2] + j]
+                                        : g.dense[q2 * g.k_stride + dense_at(s, i, j)];
+              const double2 p = g.phase[(long long)(e0 + (SCATTER ? q2 : m)) * g.n_k + (SCATTER ? m : q2)];
+              const double py = SCATTER ? p.y : -p.y;
+              a = make_double2(fma(p.x, v.x, fma(-py, v.y, a.x)), fma(p.x, v.y, fma(py, v.x, a.y)));
+            }
+            if (SCATTER) g.dense[m * g.k_stride + dense_at(s, i, j)] = a;
+            else g.entries[off_s[m] + (long long)s * re_s[m] * ce_s[m] + i * ce_s[m] + j] =
+                     make_double2(a.x * (1.0 / g.n_k), a.y * (1.0 / g.n_k));
+          }
+          continue;
+        }
 #pragma unroll
         for (int k = 0; k < 16; k += 2) {
           const int n = 16 * c + k, m = n >> 1;
@@ -378,8 +414,9 @@ void lattice_free(LatticePlan& l) {
   l = LatticePlan{};
 }
 
-gw_status lattice_run(const LatticePlan& l, const HostPlan& h, const DevEntry* d_ent, const int* d_row_off, bool pb,
-                      int n_slices, bool to_k, double2* dense, double2* entries, int* d_status, cudaStream_t st) {
+gw_status lattice_run(const LatticePlan& l, const HostPlan& h, const DevEntry* d_ent, const int* d_row_off,
+                      const double2* d_phase, bool pb, int n_slices, bool to_k, double2* dense, double2* entries,
+                      int* d_status, cudaStream_t st) {
   const std::vector<int>& ro = pb ? h.pb_off : h.orb_off;
   const long long N = ro.back();
   int band = 0;
@@ -400,6 +437,7 @@ gw_status lattice_run(const LatticePlan& l, const HostPlan& h, const DevEntry* d
   a.B = l.d_B[to_k];
   a.B_off = l.d_off[to_k];
   a.eB = l.d_e[to_k];
+  a.phase = d_phase;
   a.status = d_status;
   // about six blocks per SM over the whole launch, at least four tiles each
   const long long want = std::max<long long>(1, 6LL * l.n_sm / l.n_active);

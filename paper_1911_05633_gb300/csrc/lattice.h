@@ -26,7 +26,8 @@ struct LatticePlan {
 gw_status lattice_init(LatticePlan& l, const HostPlan& h);
 void lattice_free(LatticePlan& l);
 // dense [n_k][n_slices][N][N] <-> the entry layout with n_slices slices.
-gw_status lattice_run(const LatticePlan& l, const HostPlan& h, const DevEntry* d_ent, const int* d_row_off, bool pb,
-                      int n_slices, bool to_k, double2* dense, double2* entries, int* d_status, cudaStream_t st);
+gw_status lattice_run(const LatticePlan& l, const HostPlan& h, const DevEntry* d_ent, const int* d_row_off,
+                      const double2* d_phase, bool pb, int n_slices, bool to_k, double2* dense, double2* entries,
+                      int* d_status, cudaStream_t st);
 
 }  // namespace gw

@@ -48,3 +48,63 @@ def test_against_fp64_kernels(kmesh, cutoff, n_orb, n_prod, far, chained):
     a.sync()
     b.sync()
     assert ("k_lattice_tc" in a.timing_read()) == chained
+
+
+def _rows(plan, cell, kind, to_k, values):
+    """Inputs of one transform, one slice per entry of `values`: a function of the slice's random
+    numbers [.., elements]; flat, in the layout of the direction's input."""
+    rng = np.random.default_rng(12)
+    N, ns = plan.dense_n(kind), len(values)
+    if to_k:
+        out = np.zeros(plan.len(kind, ns), np.complex128)
+        off = plan.offsets(kind)
+        for e in range(len(off) - 1):
+            n = int(off[e + 1] - off[e])
+            for s, f in enumerate(values):
+                out[ns * off[e] + s * n: ns * off[e] + (s + 1) * n] = f(rng.standard_normal(n) + 1j * rng.standard_normal(n))
+        return out
+    out = np.zeros((cell.n_k, ns, N * N), np.complex128)
+    for s, f in enumerate(values):
+        out[:, s] = f(rng.standard_normal((cell.n_k, N * N)) + 1j * rng.standard_normal((cell.n_k, N * N)))
+    return out.reshape(-1)
+
+
+def _slices(plan, cell, kind, to_k, x, ns):
+    """The output of a transform as one array per slice."""
+    N = plan.dense_n(kind)
+    if to_k:
+        return [y.reshape(-1) for y in x.reshape(cell.n_k, ns, N * N).transpose(1, 0, 2)]
+    off = plan.offsets(kind)
+    parts = [x[ns * off[e]: ns * off[e + 1]].reshape(ns, -1) for e in range(len(off) - 1)]
+    return [np.concatenate([p[s] for p in parts]) for s in range(ns)]
+
+
+SIZES = [1.0, 1e-280, 1e-291, 1e-295, 1e-300, 1e-305, 1e-308, 1e-318, 1e300, 1e305, 0.0]
+
+
+@pytest.mark.parametrize("to_k", [False, True])
+@pytest.mark.parametrize("same", [False, True])
+def test_values_near_the_ends_of_the_range(to_k, same):
+    """One size per slice, random over the mesh (or the classes) or one value that cancels in the
+    sums.  Per slice: 2e-14 of its largest value as above, and half a unit of the subnormal numbers
+    in each of the four products of a term, 64 terms: 128 x 2^-1074."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1911_05633_gb300 import gw
+    cell = synth.mixed_species_cell(n_tau=9, n_orb=(4, 5), n_prod=(30, 35), kmesh=(3, 3, 3))
+    a, b = gw.Plan.from_cell(cell), gw.Plan.from_cell(cell, fp64_products="fp64")
+
+    def of(size):
+        return lambda x: size * (np.full_like(x, -1.23) if same else x)
+
+    F = dev(_rows(a, cell, "pb", to_k, [of(s) for s in SIZES]))
+    run = (lambda p: p.fourier_R_to_k("pb", len(SIZES), F)) if to_k else (lambda p: p.fourier_k_to_R("pb", len(SIZES), F))
+    a.timing_enable(True)
+    got, ref = host(run(a)), host(run(b))
+    a.sync()
+    assert "k_lattice_tc" in a.timing_read()
+    for size, x, y in zip(SIZES, *(_slices(a, cell, "pb", to_k, z, len(SIZES)) for z in (got, ref))):
+        assert np.isfinite(y).all()
+        tol = 2e-14 * size * (27 if to_k else 1) + 128 * 2.0 ** -1074
+        assert max(np.abs(x.real - y.real).max(), np.abs(x.imag - y.imag).max()) <= tol, size
