@@ -37,7 +37,8 @@ constexpr uint32_t kLtStep = kOzDigits * kTfPlane;    // 32 KB: digits of 128 ro
 // multiple of 2^(e - 61) for the row's scale 2^e (2^-56 of it times the smallest column scale,
 // 2^-5 at 32 points) and below 2^(e + 7), so that these keep it a normal double, and what the
 // digits drop of such a row, its subnormal values, is below 2^-62 of it.  Any other row that
-// is not all zero (G(tau) far from both ends at low temperature) is summed in FP64.
+// is not all zero (G(tau) far from both ends at low temperature; a NaN or an infinity, which
+// the digits would lose) is summed in FP64.
 constexpr int kLtLow = 64, kLtHigh = 2032;
 constexpr int kLtDirect = 1 << 20;                    // in place of such a row's scale exponent
 
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
         for (int u = 0; u < 8; ++u) mx = max(mx, exp_field(w[ks][u]));
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
       const int e = mx > 0 ? mx - 1022 : 0;
-      bool direct = mx > kLtHigh && mx < 2047;
+      bool direct = mx > kLtHigh;
       if (__any_sync(0xffffffffu, mx < kLtLow)) {
         unsigned long long any = 0;
 #pragma unroll

@@ -108,3 +108,29 @@ def test_values_near_the_ends_of_the_range(to_k, same):
         assert np.isfinite(y).all()
         tol = 2e-14 * size * (27 if to_k else 1) + 128 * 2.0 ** -1074
         assert max(np.abs(x.real - y.real).max(), np.abs(x.imag - y.imag).max()) <= tol, size
+
+
+@pytest.mark.parametrize("to_k", [False, True])
+def test_nan_and_infinities_pass_through(to_k):
+    """One element of each kind among finite ones: the outputs that read it get what FP64
+    arithmetic gives them, every other output its value (2e-14 as above, of sums of 27 terms)."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1911_05633_gb300 import gw
+    cell = synth.mixed_species_cell(n_tau=9, n_orb=(4, 5), n_prod=(30, 35), kmesh=(3, 3, 3))
+    a, b = gw.Plan.from_cell(cell), gw.Plan.from_cell(cell, fp64_products="fp64")
+    x = _rows(a, cell, "pb", to_k, [lambda z: z] * 3)
+    for i, bad in enumerate([np.nan, np.inf, -np.inf * 1j, complex(1.0, np.nan), complex(np.inf, np.inf)]):
+        x[(2 * i + 1) * x.size // 11] = bad
+    F = dev(x)
+    run = (lambda p: p.fourier_R_to_k("pb", 3, F)) if to_k else (lambda p: p.fourier_k_to_R("pb", 3, F))
+    a.timing_enable(True)
+    got, ref = host(run(a)), host(run(b))
+    a.sync()
+    assert "k_lattice_tc" in a.timing_read()
+    bad = ~np.isfinite(ref)
+    assert 5 * 27 <= bad.sum() <= 5 * 27 * 3
+    for g, r in ((got.real, ref.real), (got.imag, ref.imag)):
+        assert np.array_equal(np.isnan(g), np.isnan(r)) and np.array_equal(g[np.isinf(r)], r[np.isinf(r)])
+    assert np.abs(got[~bad] - ref[~bad]).max() <= 2e-14 * 27 * np.abs(x[np.isfinite(x)]).max()
