@@ -14,6 +14,7 @@ constexpr int kChainMax = 64;  // product functions per atom and orbital pairs n
 // A static column operand per species: digits [KS][kOzDigits][NT x 16] and exponents [NT].
 struct ChainTable {
   int KS = 0, NT = 0;
+  int e_min = 0, e_max = 0;  // of the exponents
   uint16_t* d_B = nullptr;  // [n_species] operands, back to back
   int* d_e = nullptr;       // [n_species][NT]
 };

@@ -197,6 +197,7 @@ struct ChainArgs {
   const int* eA;
   const uint16_t* B;     // static operands of all species: that of b in the first product, of a in the second
   const int* eB;
+  int eB_min, eB_max;
   // P: out[e][s0 + slice][n2 .. ] = -s value at row K = column of the second product, K' = its row
   double2* P;
   int n_tau, s0, ms_shift;
@@ -368,12 +369,21 @@ __global__ void __launch_bounds__(ch_threads(NT), 1) k_chain(const __grid_consta
     if (tid == 0 && u + (int)gridDim.x < g.n_units) load_a(u + gridDim.x);
     ch_sums<W>(t_addr, NT, S);
     fence_before_sync();  // ordered before the next unit's products by the barrier below
+    // every result of the warp zero or a normal number (|S| < 2^62)?
+    const bool normal = __all_sync(0xffffffffu, er <= -100000 || (er + g.eB_min - 56 >= -1022 && er + g.eB_max + 8 <= 1023));
+    auto slow = [&](long long s, int e) { return er > -100000 ? tf_i2d_any(s, e) : 0.0; };
     if (SIGMA) {
       // lanes on consecutive doubles of one n2
       double* d = g.D + (long long)u * g.ld_d * 128 + row;
+      if (normal) {
 #pragma unroll
-      for (int j = 0; j < W; ++j)
-        if (n0 + j < g.ld_d) d[(n0 + j) * 128] = er > -100000 ? tf_i2d(S[j], er + eB2[n0 + j] - 56) : 0.0;
+        for (int j = 0; j < W; ++j)
+          if (n0 + j < g.ld_d) d[(n0 + j) * 128] = tf_i2d(S[j], er + eB2[n0 + j] - 56);
+      } else {
+#pragma unroll
+        for (int j = 0; j < W; ++j)
+          if (n0 + j < g.ld_d) d[(n0 + j) * 128] = slow(S[j], er + eB2[n0 + j] - 56);
+      }
     } else {
       const int grp = warp >> 2, tg = tid & 127;
       double* stg = reinterpret_cast<double*>(B2 + BB) + grp * (8 * 64 * 2);
@@ -383,10 +393,16 @@ __global__ void __launch_bounds__(ch_threads(NT), 1) k_chain(const __grid_consta
 #pragma unroll
       for (int h = 0; h < W / 8; ++h) {
         if (h > 0) asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
+        // -s (s = 1 or 2) folded into the integer and the exponent
+        if (normal) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)  // -s (s = 1 or 2) folded into the integer and the exponent
-          stg[(2 * j + c) * 64 + r] =
-              er > -100000 ? tf_i2d(-S[8 * h + j], er + eB2[n0 + 8 * h + j] - 56 + g.ms_shift) : 0.0;
+          for (int j = 0; j < 8; ++j)
+            stg[(2 * j + c) * 64 + r] = tf_i2d(-S[8 * h + j], er + eB2[n0 + 8 * h + j] - 56 + g.ms_shift);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            stg[(2 * j + c) * 64 + r] = slow(-S[8 * h + j], er + eB2[n0 + 8 * h + j] - 56 + g.ms_shift);
+        }
         asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
         const int Kp = tg & 63;
 #pragma unroll
@@ -583,6 +599,8 @@ gw_status chain_init(ChainPlan& c, const HostPlan& h) {
         for (int k = 0; k < red; ++k) mx = std::max(mx, host_exp_field(value(r, k)));
         const int e = mx > 0 ? mx - 1022 : 0;
         ex[(size_t)s * t.NT + r] = e;
+        t.e_min = std::min(t.e_min, e);
+        t.e_max = std::max(t.e_max, e);
         for (int k = 0; k < red; ++k) {
           uint16_t d[kOzDigits];
           host_tf_digits(host_fixed56(value(r, k), e), d);
@@ -663,6 +681,8 @@ gw_status chain_polarizability(ChainPlan& c, const HostPlan& h, const DevEntry* 
     a.eA = c.d_eP;
     a.B = c.kp.d_B;
     a.eB = c.kp.d_e;
+    a.eB_min = c.kp.e_min;
+    a.eB_max = c.kp.e_max;
     a.P = P;
     a.n_tau = h.n_tau;
     a.s0 = s0;
@@ -693,6 +713,8 @@ gw_status chain_self_energy(ChainPlan& c, const HostPlan& h, const DevEntry* d_e
     a.eA = c.d_eS;
     a.B = c.pk.d_B;
     a.eB = c.pk.d_e;
+    a.eB_min = c.pk.e_min;
+    a.eB_max = c.pk.e_max;
     a.D = c.d_D;
     a.ld_d = c.max_pairs;
     a.status = d_status;

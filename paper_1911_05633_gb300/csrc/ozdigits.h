@@ -84,6 +84,9 @@ __device__ __forceinline__ double tf_i2d(long long S, int e) {
   return __hiloint2double(S ? hi + (e << 20) : 0, __double2loint(d));
 }
 
+// tf_i2d for any exponent: subnormal, zero or infinite where the result is.
+__device__ __forceinline__ double tf_i2d_any(long long S, int e) { return scalbn(__ll2double_rn(S), e); }
+
 // The digit products of one K step for columns NT wide, as a schedule fixed at compile
 // time: digit s of the rows against digits t .. t + cnt - 1 of the columns (consecutive
 // planes, one MMA cnt NT wide) into accumulators slot .. slot + cnt - 1; `init`: the MMA

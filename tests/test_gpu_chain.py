@@ -48,3 +48,56 @@ def test_pairs_against_fp64_kernels(n_orb, n_prod, n_tau, far, chained):
     assert rel(host(S), host(S2)) < 1e-13
     assert rel(host(X), host(X2)) < 1e-13
     b.sync()
+
+
+def _plans(n_tau):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1911_05633_gb300 import gw
+    cell = _cell((5, 9), (33, 48), n_tau)
+    a, b = gw.Plan.from_cell(cell), gw.Plan.from_cell(cell, fp64_products="fp64")
+    a.timing_enable(True)
+    return cell, a, b
+
+
+def _slices(p, kind, n, x):
+    """A flat buffer in the entry layout as views [slice][elements] per entry."""
+    off = p.offsets(kind)
+    return [x[n * off[e]: n * off[e + 1]].reshape(n, -1) for e in range(len(off) - 1)]
+
+
+def _agree(plan, kind, n, got, ref, floor):
+    """Per node: 1e-13 in the Frobenius norm (as above) beside `floor` per element."""
+    for i in range(n):
+        g, r = (np.concatenate([q[i] for q in _slices(plan, kind, n, x)]) for x in (got, ref))
+        size = max(np.abs(r).max(), 2.0 ** -1022)  # the squares stay in the range
+        assert np.isfinite(r).all()
+        assert np.linalg.norm((g - r) / size) <= 1e-13 * np.linalg.norm(r / size) + np.sqrt(r.size) * floor / size, i
+
+
+def test_values_near_the_ends_of_the_range():
+    """P, Sigma and Sigma_x of inputs of one size per node against the FP64-only kernels.  The
+    digits take subnormal elements of M, W~ and v for zero: less than 2^-1022 each, in a sum with
+    the coefficients of both atoms (and G for Sigma)."""
+    sizes = [1.0, 1e-140, 1e-145, 1e-148, 1e-152, 1e-160, 1e150]
+    nt = 2 * len(sizes) - 1
+    cell, a, b = _plans(nt)
+    rng = np.random.default_rng(8)
+    z = lambda n: rng.standard_normal(n) + 1j * rng.standard_normal(n)
+    G, W, G1 = z(a.len("orb", nt)), z(a.len("pb", nt)), z(a.len("orb", nt))
+    node = np.array(sizes + sizes[-2::-1])  # G(tau) and G(beta - tau) of one size
+    for x, kind, sc in ((G, "orb", node), (W, "pb", node ** 2)):
+        for y in _slices(a, kind, nt, x):
+            y *= sc[:, None]
+    c_k = max(np.abs(s.C).sum(axis=(1, 2)).max() for s in cell.species)  # sum over (L, L'') of |C[K][L][L'']|
+    c = max(np.abs(s.C).sum() for s in cell.species)
+    _agree(a, "pb", nt, host(a.polarizability_tau(dev(G))), host(b.polarizability_tau(dev(G))), 8 * c_k ** 2 * 2.0 ** -1022)
+    for size in (1.0, 1e-300, 1e300):
+        v = dev(z(a.len("pb", 1)) * size)
+        S, X = a.self_energy_tau(dev(G1), dev(W), v_R=v)
+        S2, X2 = b.self_energy_tau(dev(G1), dev(W), v_R=v)
+        for n, got, ref in ((nt, S, S2), (1, X, X2)):
+            _agree(a, "orb", n, host(got), host(ref), 4 * c ** 2 * np.abs(G1).max() * 2.0 ** -1022)
+    a.sync()
+    assert "k_chain" in a.timing_read()
