@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(256) k_polarizability_pairs(const DevEntry* __
     mr = __reduce_max_sync(0xffffffffu, mr);
     mi = __reduce_max_sync(0xffffffffu, mi);
     if (lane == 0) {
-      e_s[p] = mr > 0 ? mr - 1022 : 0;
-      e_s[64 + p] = mi > 0 ? mi - 1022 : 0;
+      e_s[p] = tf_row_scale(mr);
+      e_s[64 + p] = tf_row_scale(mi);
     }
   }
   __syncthreads();
@@ -150,8 +150,8 @@ __global__ void __launch_bounds__(256) k_slice_w_units(const DevEntry* __restric
     mr = __reduce_max_sync(0xffffffffu, mr);
     mi = __reduce_max_sync(0xffffffffu, mi);
     if (lane == 0) {
-      e_s[K] = mr > 0 ? mr - 1022 : 0;
-      e_s[64 + K] = mi > 0 ? mi - 1022 : 0;
+      e_s[K] = tf_row_scale(mr);
+      e_s[64 + K] = tf_row_scale(mi);
     }
   }
   __syncthreads();
@@ -324,10 +324,11 @@ __global__ void __launch_bounds__(ch_threads(NT), 1) k_chain(const __grid_consta
     ch_sums<W>(t_addr, NT, S);
     // the scale of each row (c, n) of the second operand: the largest value over r
     int mine = -100000;
+    const int none = ea > kOzNaN / 2 ? ea : -100000;  // of a zero sum
 #pragma unroll
     for (int j = 0; j < W; ++j) {
       const long long a = S[j] ^ (S[j] >> 63);  // |S| <= a + 1
-      const int ex = S[j] ? 64 - __clzll(a) + ea + eB1[n0 + j] - 56 : -100000;
+      const int ex = S[j] ? 64 - __clzll(a) + ea + eB1[n0 + j] - 56 : none;
       const int m = __reduce_max_sync(0xffffffffu, ex);
       if (lane == j) mine = m;
     }

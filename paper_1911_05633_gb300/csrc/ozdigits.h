@@ -84,8 +84,14 @@ __device__ __forceinline__ double tf_i2d(long long S, int e) {
   return __hiloint2double(S ? hi + (e << 20) : 0, __double2loint(d));
 }
 
+// Scale exponent of a row that holds an infinity or a NaN (its digits are zero): what is
+// computed from it is NaN.
+constexpr int kOzNaN = 1 << 20;
+__device__ __forceinline__ int tf_row_scale(int m) { return m == 2047 ? kOzNaN : m > 0 ? m - 1022 : 0; }
 // tf_i2d for any exponent: subnormal, zero or infinite where the result is.
-__device__ __forceinline__ double tf_i2d_any(long long S, int e) { return scalbn(__ll2double_rn(S), e); }
+__device__ __forceinline__ double tf_i2d_any(long long S, int e) {
+  return e > kOzNaN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(__ll2double_rn(S), e);
+}
 
 // The digit products of one K step for columns NT wide, as a schedule fixed at compile
 // time: digit s of the rows against digits t .. t + cnt - 1 of the columns (consecutive

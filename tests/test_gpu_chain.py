@@ -101,3 +101,25 @@ def test_values_near_the_ends_of_the_range():
             _agree(a, "orb", n, host(got), host(ref), 4 * c ** 2 * np.abs(G1).max() * 2.0 ** -1022)
     a.sync()
     assert "k_chain" in a.timing_read()
+
+
+def test_nan_and_infinities_pass_through():
+    """One element that is no number in G, W~ and v: the outputs that take it are no numbers, as in
+    FP64 arithmetic, the others keep their values (1e-13 as above)."""
+    nt = 9
+    cell, a, b = _plans(nt)
+    rng = np.random.default_rng(9)
+    z = lambda n: rng.standard_normal(n) + 1j * rng.standard_normal(n)
+    G, W, v, G1 = z(a.len("orb", nt)), z(a.len("pb", nt)), z(a.len("pb", 1)), z(a.len("orb", nt))
+    bad = [np.nan, np.inf, complex(1.0, np.nan), complex(2.0, -np.inf)]
+    for x in (G, W, v):
+        x[[(2 * i + 1) * x.size // 9 for i in range(4)]] = bad
+    S, X = a.self_energy_tau(dev(G1), dev(W), v_R=dev(v))
+    S2, X2 = b.self_energy_tau(dev(G1), dev(W), v_R=dev(v))
+    pairs = [(S, S2), (X, X2), (a.polarizability_tau(dev(G)), b.polarizability_tau(dev(G)))]
+    a.sync()
+    assert "k_chain" in a.timing_read()
+    for got, ref in ((host(x), host(y)) for x, y in pairs):
+        ok = np.isfinite(ref)
+        assert np.array_equal(np.isfinite(got), ok) and 0 < ok.sum() < ok.size
+        assert rel(got[ok], ref[ok]) < 1e-13
