@@ -444,23 +444,26 @@ static gw_status alloc_w_scratch(gw_plan_s* p) {
   return GW_OK;
 }
 
-// The FP64 digit-GEMM scratch of the Sigma stage W~ C^b and of the P stage Y C^b.
+// The FP64 digit scratch of Sigma and of P: of both products over symmetric pairs or, where
+// that does not fit the device's memory, of the stages W~ C^b and Y C^b, which need less.  A
+// call whose scratch cannot be allocated fails, the next one runs the FP64 kernels without any.
 static gw_status alloc_oz_sigma(gw_plan_s* p) {
-  if (p->chain.ok) {
+  if (p->chain.ok && gw::chain_alloc_s(p->chain, p->h, (size_t)4 << 30) == GW_OK) {
     p->oz_pending = false;
-    return gw::chain_alloc_s(p->chain, p->h, (size_t)4 << 30);
+    return GW_OK;
   }
   const gw_status st = gw::oz_sigma_init(p->oz, p->h, (size_t)4 << 30);
   p->oz_pending = false;
+  if (st != GW_OK) p->sigma_tensor = false;
   if (st != GW_OK) return st;
   if (gw::uploads_landed() != cudaSuccess) return GW_ERR_CUDA;
   p->sigma_tensor = p->oz.ready;
   return GW_OK;
 }
 static gw_status alloc_oz_pol(gw_plan_s* p) {
-  if (p->chain.ok) {
+  if (p->chain.ok && gw::chain_alloc_p(p->chain, p->h, (size_t)4 << 30) == GW_OK) {
     p->ozp_pending = false;
-    return gw::chain_alloc_p(p->chain, p->h, (size_t)4 << 30);
+    return GW_OK;
   }
   const gw_status st = gw::oz_pol_init(p->ozp, p->h, (size_t)4 << 30);
   p->ozp_pending = false;
@@ -658,8 +661,8 @@ gw_status gw_plan_create(const gw_cell* cell, const gw_basis* basis, const int k
     gw::set_last_error("");
   }
   if (!(opt && opt->fp64_products == 1)) {
-    if ((st = gw::chain_init(p->chain, h)) != GW_OK) return fail(st);
-    if ((st = gw::lattice_init(p->lattice, h)) != GW_OK) return fail(st);
+    gw::chain_init(p->chain, h);
+    gw::lattice_init(p->lattice, h);
   }
   if (p->sigma_tensor) {
     if (defer) p->oz_pending = true;

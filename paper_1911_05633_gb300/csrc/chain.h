@@ -39,9 +39,10 @@ struct ChainPlan {
   int tau_s = 0;
 };
 
-// Whether the plan's contractions fit; uploads the tables when they do (ok).
-gw_status chain_init(ChainPlan& c, const HostPlan& h);
-// Scratch of one contraction within `cap` bytes.
+// Whether the plan's contractions fit; uploads the tables when they do (ok: false as well when
+// there is no memory for them).
+void chain_init(ChainPlan& c, const HostPlan& h);
+// Scratch of one contraction within `cap` bytes (p_ready, s_ready).
 gw_status chain_alloc_p(ChainPlan& c, const HostPlan& h, size_t cap);
 gw_status chain_alloc_s(ChainPlan& c, const HostPlan& h, size_t cap);
 void chain_free(ChainPlan& c);

@@ -522,8 +522,8 @@ size_t sigma_smem(int max_np) { return std::max((size_t)max_np * max_np, (size_t
 
 bool up(void** dst, const void* src, size_t bytes) {
   if (cudaMalloc(dst, bytes ? bytes : 16) != cudaSuccess) {
+    *dst = nullptr;
     cudaGetLastError();
-    set_last_error("device allocation for the FP64 contractions failed");
     return false;
   }
   return !src || cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
@@ -547,17 +547,17 @@ gw_status launch_status(const char* what) {
 // 398, K = 32 333 / 372 and 681 / 894; n = 5 K = 16 267 / 267 and 559 / 598; n = 9 K = 8 529 /
 // 521 and 1257 / 1046, K = 16 541 / 977 and 1284 / 2057, K = 64 907 / 4122 and 1880 / 9605.
 constexpr int kChainMinK = 12, kChainMinKnn = 400;
-gw_status chain_init(ChainPlan& c, const HostPlan& h) {
+void chain_init(ChainPlan& c, const HostPlan& h) {
   c = ChainPlan{};
-  if (!h.c_symmetric) return GW_OK;
+  if (!h.c_symmetric) return;
   int max_k = 0, max_np = 0, max_n = 0;
   for (int s = 0; s < h.n_species; ++s) {
     max_n = std::max(max_n, h.n_orb[s]);
     max_k = std::max(max_k, h.n_prod[s]);
   }
   max_np = max_n * (max_n + 1) / 2;
-  if (max_k > kChainMax || max_np > kChainMax) return GW_OK;
-  if (max_k < kChainMinK || max_k * max_n * max_n < kChainMinKnn) return GW_OK;
+  if (max_k > kChainMax || max_np > kChainMax) return;
+  if (max_k < kChainMinK || max_k * max_n * max_n < kChainMinKnn) return;
   c.max_pairs = max_np;
   c.kp.NT = (max_k + 15) / 16 * 16;
   c.kp.KS = (max_np + 15) / 16;
@@ -568,7 +568,7 @@ gw_status chain_init(ChainPlan& c, const HostPlan& h) {
   cudaDeviceGetAttribute(&c.n_sm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const size_t lim = (size_t)std::max(smem_max, 0) - 2048;  // the kernel's static shared memory
-  if (chain_smem<false>(c.kp) > lim || chain_smem<true>(c.pk) > lim || pairs_smem(max_n) > lim) return GW_OK;
+  if (chain_smem<false>(c.kp) > lim || chain_smem<true>(c.pk) > lim || pairs_smem(max_n) > lim) return;
   std::vector<unsigned char> pr((size_t)h.n_species * 2 * kChainMax, 0), pi((size_t)h.n_species * 256, 0);
   for (int s = 0; s < h.n_species; ++s) {
     const int n = h.n_orb[s];
@@ -617,17 +617,16 @@ gw_status chain_init(ChainPlan& c, const HostPlan& h) {
       !up((void**)&c.d_pidx, pi.data(), pi.size()) ||
       !up((void**)&c.d_species, h.species.data(), h.species.size() * sizeof(int))) {
     chain_free(c);
-    return GW_ERR_OOM;
+    return;
   }
   if (chain_raise<false>(c.kp) != cudaSuccess || chain_raise<true>(c.pk) != cudaSuccess ||
       raise_smem_limit(k_polarizability_pairs, pairs_smem(max_n)) != cudaSuccess ||
       raise_smem_limit(k_sigma_pairs, sigma_smem(max_np)) != cudaSuccess) {
-    set_last_error("cudaFuncSetAttribute (FP64 contractions)");
+    cudaGetLastError();
     chain_free(c);
-    return GW_ERR_UNSUPPORTED;
+    return;
   }
   c.ok = true;
-  return GW_OK;
 }
 
 void chain_free(ChainPlan& c) {
@@ -642,8 +641,11 @@ gw_status chain_alloc_p(ChainPlan& c, const HostPlan& h, size_t cap) {
   const size_t E = (size_t)h.n_entries(), per = c.kp.KS * kChStep + 128 * sizeof(int);
   c.tau_p = (int)std::max<size_t>(1, std::min<size_t>((size_t)(h.n_tau + 1) / 2, cap / std::max<size_t>(1, E * per)));
   const size_t n = E * c.tau_p;
-  if (!up((void**)&c.d_AP, nullptr, n * c.kp.KS * kChStep) || !up((void**)&c.d_eP, nullptr, n * 128 * sizeof(int)))
+  if (!up((void**)&c.d_AP, nullptr, n * c.kp.KS * kChStep) || !up((void**)&c.d_eP, nullptr, n * 128 * sizeof(int))) {
+    cudaFree(c.d_AP);
+    c.d_AP = nullptr;
     return GW_ERR_OOM;
+  }
   c.p_ready = true;
   return GW_OK;
 }
@@ -654,8 +656,13 @@ gw_status chain_alloc_s(ChainPlan& c, const HostPlan& h, size_t cap) {
   c.tau_s = (int)std::max<size_t>(1, std::min<size_t>((size_t)h.n_tau, cap / std::max<size_t>(1, E * per)));
   const size_t n = E * c.tau_s;
   if (!up((void**)&c.d_AS, nullptr, n * c.pk.KS * kChStep) || !up((void**)&c.d_eS, nullptr, n * 128 * sizeof(int)) ||
-      !up((void**)&c.d_D, nullptr, n * c.max_pairs * 128 * sizeof(double)))
+      !up((void**)&c.d_D, nullptr, n * c.max_pairs * 128 * sizeof(double))) {
+    cudaFree(c.d_AS);
+    cudaFree(c.d_eS);
+    c.d_AS = nullptr;
+    c.d_eS = nullptr;
     return GW_ERR_OOM;
+  }
   c.s_ready = true;
   return GW_OK;
 }

@@ -333,14 +333,14 @@ void lat_launch(int KS, dim3 grid, size_t smem, const LatArgs& a, cudaStream_t s
 // Taken on meshes of at most 32 points with some phase that is no quarter turn (quarter turns
 // cost two additions per term and stay with the FP64 kernels), while the pairs' operands are
 // small beside the data.
-gw_status lattice_init(LatticePlan& l, const HostPlan& h) {
+void lattice_init(LatticePlan& l, const HostPlan& h) {
   l = LatticePlan{};
   std::vector<int> first;
   for (size_t q = 0; q + 1 < h.pair_start.size(); ++q)
     if (h.pair_start[q + 1] > h.pair_start[q]) first.push_back(h.pair_start[q]);
   const int n_act = (int)first.size();
   first.push_back(h.n_entries());
-  if (!h.phase_code.empty() || h.n_k > kLatMaxK || n_act == 0) return GW_OK;
+  if (!h.phase_code.empty() || h.n_k > kLatMaxK || n_act == 0) return;
   for (int p = 0; p < n_act; ++p) l.max_cls = std::max(l.max_cls, first[p + 1] - first[p]);
   l.n_active = n_act;
   l.all_pairs = n_act == h.n_atoms * h.n_atoms;
@@ -355,7 +355,7 @@ gw_status lattice_init(LatticePlan& l, const HostPlan& h) {
     }
     if (tot * sizeof(uint16_t) > kLatMaxBytes) {
       lattice_free(l);
-      return GW_OK;
+      return;
     }
     std::vector<uint16_t> dig(tot, 0);
     for (int p = 0; p < n_act; ++p) {
@@ -388,21 +388,19 @@ gw_status lattice_init(LatticePlan& l, const HostPlan& h) {
         !up((void**)&l.d_e[d], ex.data(), ex.size() * sizeof(int)) ||
         (d == 0 && !up((void**)&l.d_first, first.data(), first.size() * sizeof(int)))) {
       cudaGetLastError();
-      lattice_free(l);
-      set_last_error("device allocation for the lattice transforms failed");
-      return GW_ERR_OOM;
+      lattice_free(l);  // the FP64 kernels, which need no operands
+      return;
     }
   }
   if (lat_raise<false>() != cudaSuccess || lat_raise<true>() != cudaSuccess) {
     cudaGetLastError();
     lattice_free(l);
-    return GW_OK;
+    return;
   }
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&l.n_sm, cudaDevAttrMultiProcessorCount, dev);
   l.ok = true;
-  return GW_OK;
 }
 
 void lattice_free(LatticePlan& l) {

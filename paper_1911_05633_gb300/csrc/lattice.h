@@ -23,7 +23,8 @@ struct LatticePlan {
   int* d_e[2] = {nullptr, nullptr};
 };
 
-gw_status lattice_init(LatticePlan& l, const HostPlan& h);
+// ok where the plan's transforms fit and their operands are on the device.
+void lattice_init(LatticePlan& l, const HostPlan& h);
 void lattice_free(LatticePlan& l);
 // dense [n_k][n_slices][N][N] <-> the entry layout with n_slices slices.
 gw_status lattice_run(const LatticePlan& l, const HostPlan& h, const DevEntry* d_ent, const int* d_row_off,
