@@ -224,13 +224,6 @@ unsigned band_splits(const gw_plan_s* p, gw_block kind, int n_slices) {
   return (unsigned)std::max<long long>(1, std::min<long long>({want, (el + 255) / 256, 65535}));
 }
 
-// Whether a transform of n_slices slices goes to the tensor cores (lattice.h): from about
-// 8 million FP64 multiply-adds on, 15 us of the chip; below that either way is launch latency.
-bool lattice_takes(const gw_plan_s* p, gw_block kind, int n_slices) {
-  const double len = (double)(kind == GW_BLOCK_PB ? p->h.off_pb : p->h.off_orb).back();
-  return p->lattice.ok && len * n_slices * p->h.n_k * 4.0 >= 8e6;
-}
-
 gw_status launch_gather(gw_plan_s* p, gw_block kind, int n_slices, const double2* F_k, long long k_stride,
                         long long s_stride, const double2* F_sub, long long sub_k_stride, long long sub_s_stride,
                         double2* F_R, int out_n_slices, int out_slice0, double scale, cudaStream_t st,
@@ -771,7 +764,7 @@ gw_status gw_fourier_k_to_R(gw_plan_t p, gw_block kind, int n_slices, const void
   if (!F_k || !F_R || n_slices <= 0) { set_last_error("bad argument"); return GW_ERR_ARG; }
   DeviceGuard guard(p->device);
   gw::ActiveTimer timing(&p->timer);
-  if (lattice_takes(p, kind, n_slices))
+  if (gw::lattice_takes(p->lattice, p->h, kind == GW_BLOCK_PB, n_slices, false))
     return gw::lattice_run(p->lattice, p->h, p->d_ent, kind == GW_BLOCK_PB ? p->d_pb_off : p->d_orb_off,
                            p->d_phase, kind == GW_BLOCK_PB, n_slices, false, (double2*)const_cast<void*>(F_k), (double2*)F_R,
                            p->d_status, S(stream));
@@ -791,7 +784,7 @@ gw_status gw_fourier_R_to_k(gw_plan_t p, gw_block kind, int n_slices, const void
   if (!F_k || !F_R || n_slices <= 0) { set_last_error("bad argument"); return GW_ERR_ARG; }
   DeviceGuard guard(p->device);
   gw::ActiveTimer timing(&p->timer);
-  if (lattice_takes(p, kind, n_slices))
+  if (gw::lattice_takes(p->lattice, p->h, kind == GW_BLOCK_PB, n_slices, true))
     return gw::lattice_run(p->lattice, p->h, p->d_ent, kind == GW_BLOCK_PB ? p->d_pb_off : p->d_orb_off,
                            p->d_phase, kind == GW_BLOCK_PB, n_slices, true, (double2*)F_k, (double2*)const_cast<void*>(F_R),
                            p->d_status, S(stream));

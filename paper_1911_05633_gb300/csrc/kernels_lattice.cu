@@ -328,6 +328,31 @@ void lat_launch(int KS, dim3 grid, size_t smem, const LatArgs& a, cudaStream_t s
   }
 }
 
+// Elements (lane, class) that the warps of k_gather_k_to_R and k_scatter_R_to_k go through for
+// one slice, per element of the pairs with entries: a warp takes 32 consecutive elements of a
+// row atom's band, and all its lanes wait for the one with the most classes.
+double lat_sweep(const HostPlan& h, const std::vector<int>& ro) {
+  const int n = h.n_atoms, N = ro[n];
+  std::vector<int> cls(N);  // of the pair that each column belongs to
+  double steps = 0.0, el = 0.0;
+  for (int a = 0; a < n; ++a) {
+    for (int b = 0; b < n; ++b)
+      for (int i = ro[b]; i < ro[b + 1]; ++i) cls[i] = h.pair_start[a * n + b + 1] - h.pair_start[a * n + b];
+    const long long band = (long long)(ro[a + 1] - ro[a]) * N;
+    int col = 0;
+    for (long long x = 0; x < band; x += 32) {
+      int most = 0;
+      for (long long y = x; y < std::min(band, x + 32); ++y) {
+        most = std::max(most, cls[col]);
+        el += cls[col] > 0;
+        if (++col == N) col = 0;
+      }
+      steps += 32.0 * most;
+    }
+  }
+  return el > 0.0 ? steps / el : 0.0;
+}
+
 }  // namespace
 
 // Taken on meshes of at most 32 points with some phase that is no quarter turn (quarter turns
@@ -344,6 +369,10 @@ void lattice_init(LatticePlan& l, const HostPlan& h) {
   for (int p = 0; p < n_act; ++p) l.max_cls = std::max(l.max_cls, first[p + 1] - first[p]);
   l.n_active = n_act;
   l.all_pairs = n_act == h.n_atoms * h.n_atoms;
+  if (h.n_k <= kLatHeld) {
+    l.sweep[0] = lat_sweep(h, h.orb_off);
+    l.sweep[1] = lat_sweep(h, h.pb_off);
+  }
   for (int d = 0; d < 2; ++d) {  // 0: k -> R, 1: R -> k
     std::vector<long long> off(n_act);
     std::vector<int> ex((size_t)n_act * 64, 0);
@@ -401,6 +430,20 @@ void lattice_init(LatticePlan& l, const HostPlan& h) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&l.n_sm, cudaDevAttrMultiProcessorCount, dev);
   l.ok = true;
+}
+
+// From about 8 million FP64 multiply-adds on, 15 us of the chip; below that either way is launch
+// latency.  On up to kLatHeld points the FP64 kernels read an element once for all its classes,
+// so that their time is that of the steps their warps take (60 ns per thousand either way),
+// while a tile costs this kernel the same for any mesh and class count up to 8 (about 120 ns
+// per thousand elements): the line is at 2.2 steps per element k -> R and 1.4 R -> k, where
+// the FP64 sum over k of an element is longer.  On 8 atoms, in us FP64 / here: 7x1x1 with 1.25
+// classes per pair (1.7 steps) 103 / 184 and 147 / 165, 3x2x1 with 2.6 (2.9) 116 / 103 and
+// 113 / 103; 24 atoms with n = 2, 1x3x1, 1.3 classes (3.9) 161 / 82 and 168 / 79.
+bool lattice_takes(const LatticePlan& l, const HostPlan& h, bool pb, int n_slices, bool to_k) {
+  const double len = (double)(pb ? h.off_pb : h.off_orb).back();
+  if (!l.ok || len * n_slices * h.n_k * 4.0 < 8e6) return false;
+  return h.n_k > kLatHeld || l.sweep[pb ? 1 : 0] >= (to_k ? 1.4 : 2.2);
 }
 
 void lattice_free(LatticePlan& l) {

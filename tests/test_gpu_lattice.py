@@ -134,3 +134,23 @@ def test_nan_and_infinities_pass_through(to_k):
     for g, r in ((got.real, ref.real), (got.imag, ref.imag)):
         assert np.array_equal(np.isnan(g), np.isnan(r)) and np.array_equal(g[np.isinf(r)], r[np.isinf(r)])
     assert np.abs(got[~bad] - ref[~bad]).max() <= 2e-14 * 27 * np.abs(x[np.isfinite(x)]).max()
+
+
+def test_few_classes_on_a_small_mesh_stay_with_the_fp64_kernels():
+    """One class per pair on three points, in blocks as wide as two warps: one step of the FP64
+    kernels' warps per element; with every class kept, three."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1911_05633_gb300 import gw
+    for cutoff, want in ((6.5, {"k_gather_k_to_R", "k_scatter_R_to_k"}), (0.0, {"k_lattice_tc"})):
+        cell = synth.SynthCell("line", np.diag([30.0, 8.0, 8.0]), np.array([[i / 5, 0, 0] for i in range(5)]),
+                               np.zeros(5, np.int32), [synth.Species("s", 3, 64, None)], (3, 1, 1), 20.0, 9, cutoff,
+                               seed=5).build()
+        p = gw.Plan.from_cell(cell)
+        ns = 1 + 8_000_000 // (4 * cell.n_k * p.len("pb", 1))
+        p.timing_enable(True)
+        F = torch.ones(cell.n_k * ns * p.dense_n("pb") ** 2, dtype=torch.complex128, device="cuda")
+        p.fourier_R_to_k("pb", ns, p.fourier_k_to_R("pb", ns, F))
+        p.sync()
+        assert set(p.timing_read()) == want
