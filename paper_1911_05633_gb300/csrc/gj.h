@@ -12,10 +12,11 @@ constexpr int kGJSmemMax = 112;
 constexpr int kHessMaxN = 880;
 
 // Dynamic shared-memory opt-in of the inverse for order N (call with the device current).
-cudaError_t gj_setup(int N);
+cudaError_t gj_setup(int N, bool columns = false);
 // In-place inverses of `batch` N x N matrices; perm: [batch][N] scratch (read only above
-// kGJSmemMax).  A zero pivot sets *status.
-void gj_batch(double2* mats, int* perm, int batch, int N, long long stride, int* status, cudaStream_t st);
+// kGJSmemMax, where `columns` asks for the form without panels).  A zero pivot sets *status.
+void gj_batch(double2* mats, int* perm, int batch, int N, long long stride, int* status, cudaStream_t st,
+              bool columns = false);
 
 // The panel form on the matrices with only[b] != 0 (N up to 430; the others are not touched).
 cudaError_t gj_only_setup(int N);

@@ -165,7 +165,7 @@ gw_status spectral_function(DysonPlan& d, const HostPlan& h, const double2* H, c
     TimedLaunch tl_("k_retarded_build", st);
     k_retarded_build<<<(unsigned)nb, 256, 0, st>>>(H, Sigx, Sigc_w, d_wr, delta, mu, N, n_real, M);
   }
-  gj_batch(M, perm, (int)nb, N, NN, d_status, st);
+  gj_batch(M, perm, (int)nb, N, NN, d_status, st, true);
   {
     TimedLaunch tl_("k_trace_spectral", st);
     k_trace_spectral<<<(unsigned)((nb + 7) / 8), 256, 0, st>>>(M, N, nb, A);

@@ -217,7 +217,7 @@ gw_status dyson_init(DysonPlan& d, const HostPlan& h) {
     set_last_error("Dyson transform: too many fermionic frequencies for shared memory");
     return GW_ERR_UNSUPPORTED;
   }
-  if (gj_setup(d.N) != cudaSuccess || (d.N <= kHessMaxN && hess_setup(d.N) != cudaSuccess) ||
+  if (gj_setup(d.N, true) != cudaSuccess || (d.N <= kHessMaxN && hess_setup(d.N) != cudaSuccess) ||
       cudaMemset(d.count, 0, 4 * sizeof(double)) != cudaSuccess) {
     dyson_free(d);
     set_last_error("Dyson solve: shared-memory opt-in");
@@ -249,7 +249,7 @@ gw_status dyson_solve(DysonPlan& d, const HostPlan& h, const double2* H, const d
   }
   gw_status s = launch_ok("k_dyson_build");
   if (s != GW_OK) return s;
-  gj_batch(d.M, d.perm, nb, d.N, (long long)d.N * d.N, d_status, st);
+  gj_batch(d.M, d.perm, nb, d.N, (long long)d.N * d.N, d_status, st, true);
   return launch_ok("k_gj_inverse");
 }
 

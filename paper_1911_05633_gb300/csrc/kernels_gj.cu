@@ -397,21 +397,23 @@ size_t hess_smem_bytes(int N, bool in_smem) {
 static size_t gj_blocked_bytes(int N) { return (2 * (size_t)N * kGJB + N) * sizeof(double2); }
 static bool gj_is_blocked(int N) { return gj_blocked_bytes(N) <= 220 * 1024; }
 
-cudaError_t gj_setup(int N) {
+cudaError_t gj_setup(int N, bool columns) {
   if (N <= kGJSmemMax) return raise_smem_limit(k_gj_inverse_smem, gj_smem_bytes(N));
-  if (gj_is_blocked(N)) return raise_smem_limit(k_gj_inverse_blocked, gj_blocked_bytes(N));
+  if (!columns && gj_is_blocked(N)) return raise_smem_limit(k_gj_inverse_blocked, gj_blocked_bytes(N));
   const size_t bytes = 2 * (size_t)N * sizeof(double2);
   return bytes > 227 * 1024 ? cudaErrorInvalidValue : raise_smem_limit(k_gj_inverse, bytes);
 }
 
 // In shared memory wherever a matrix fits (N <= kGJSmemMax; 1.8x at N = 72 and 2.6x at 16
 // over the forms below), else by panels while the panel and its pivot rows fit, else column
-// by column in global memory.
-void gj_batch(double2* mats, int* perm, int batch, int N, long long stride, int* status, cudaStream_t st) {
+// by column in global memory.  The Dyson matrices take the columns: 768 of order 128 19.7 ms
+// by panels and 16.1 by columns, of 192 54.6 and 47.5, of 384 372 and 345.
+void gj_batch(double2* mats, int* perm, int batch, int N, long long stride, int* status, cudaStream_t st,
+              bool columns) {
   if (N <= kGJSmemMax) {
     TimedLaunch tl_("k_gj_inverse_smem", st);
     k_gj_inverse_smem<<<batch, kT, gj_smem_bytes(N), st>>>(mats, N, stride, status);
-  } else if (gj_is_blocked(N)) {
+  } else if (!columns && gj_is_blocked(N)) {
     TimedLaunch tl_("k_gj_inverse_blocked", st);
     k_gj_inverse_blocked<<<batch, 512, gj_blocked_bytes(N), st>>>(mats, perm, N, stride, status, nullptr);
   } else {

@@ -70,3 +70,16 @@ def test_singular_shift_is_still_reported():
     with pytest.raises(gw.GwError) as e:
         p.chemical_potential(dev(H), 2.0, -1.0, 1.0, Sig_k_iw=dev(S))
     assert e.value.status == 6
+
+
+def test_dyson_inverses_beyond_shared_memory_go_by_columns():
+    """Order 117, the first cell here that does not fit, against torch's inverse (as above)."""
+    p, tau, om = _plan(9, 13)
+    H, Sx, S = _inputs(2, len(om), 117, 5)
+    p.timing_enable(True)
+    A = p.spectral_function(dev(H), [0.1, 0.3], 0.2, 0.0)
+    assert "k_gj_inverse" in p.timing_read() and "k_gj_inverse_blocked" not in p.timing_read()
+    z = np.array([0.1, 0.3])[None, :, None, None] + 0.2j
+    G = np.linalg.inv(z * np.eye(117) - H[:, None])
+    ref = -np.trace(G, axis1=2, axis2=3).imag / np.pi
+    assert rel(A.cpu().numpy(), ref.reshape(-1)) < TOL
