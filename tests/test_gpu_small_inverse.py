@@ -83,3 +83,16 @@ def test_dyson_inverses_beyond_shared_memory_go_by_columns():
     G = np.linalg.inv(z * np.eye(117) - H[:, None])
     ref = -np.trace(G, axis1=2, axis2=3).imag / np.pi
     assert rel(A.cpu().numpy(), ref.reshape(-1)) < TOL
+
+
+def test_short_search_goes_without_the_forms():
+    """One evaluation of N(mu) takes one solve, a longer search the Hessenberg forms; N agrees."""
+    p, tau, om = _plan(3, 4)
+    H, Sx, S = _inputs(2, len(om), 12, 5)
+    a = dict(Sigx_k=dev(Sx), Sig_k_iw=dev(S))
+    p.timing_enable(True)
+    mu, n = p.chemical_potential(dev(H), 12.0, -0.5, 0.5, tol=1.0, **a)
+    assert mu == 0.0 and "k_gj_inverse_smem" in p.timing_read() and "k_hessenberg" not in p.timing_read()
+    mu2, n2 = p.chemical_potential(dev(H), n, -1e-9, 1e-9, tol=1e-10, **a)
+    assert "k_hessenberg" in p.timing_read()
+    assert abs(n2 - n) < 1e-7 and abs(mu2) < 1e-9
