@@ -1224,7 +1224,8 @@ gw_status gw_chemical_potential(gw_plan_t p, const void* H_k, const void* Sigx_k
   };
   // The same from the Hessenberg forms, reduced once; a mu at which one of the matrices is
   // singular to rounding goes to the solve, whose pivots decide, and the forms (in the same
-  // buffer) are made again.  Forms cost about two solves (64 k x 48 frequencies of order 72:
+  // buffer) are made again; so does a failure that an earlier call left, which the solve
+  // reports.  Forms cost about two solves (64 k x 48 frequencies of order 72:
   // 18.3 ms against 8.9; 2 x 48 of order 144: 7.9 against 4.3), so a search of one or two
   // evaluations goes without them.
   int evals = 1;
@@ -1237,7 +1238,7 @@ gw_status gw_chemical_potential(gw_plan_t p, const void* H_k, const void* Sigx_k
     if (e != GW_OK) return e;
     reduced = true;
     bool weak = false;
-    if ((e = gw::dyson_search_count(p->dyson, h, mu, Tlast, n, &weak, s)) != GW_OK || !weak) return e;
+    if ((e = gw::dyson_search_count(p->dyson, h, mu, Tlast, p->d_status, n, &weak, s)) != GW_OK || !weak) return e;
     reduced = false;
     return solve_count(mu, n);
   };

@@ -46,13 +46,13 @@ gw_status dyson_density(DysonPlan& d, const HostPlan& h, const double2* H, const
 // The search for mu evaluates N(mu) many times on the same H and Sigma: dyson_search_begin
 // leaves the Hessenberg forms of M(k, n) = i w_n - H - Sigma_x - Sigma_c in d.M, and each
 // dyson_search_count takes N(mu) from tr (mu + M)^{-1}, O(N^2) per matrix (synchronous on
-// st).  *weak: some mu + M is singular to the trace's rounding.  N <= kHessMaxN.
+// st).  *weak: some mu + M is singular to the trace's rounding, or *status is set.  N <= kHessMaxN.
 // 64 k x 48 frequencies of order 72, 43 evaluations: before, one inverse per evaluation,
 // 17 ms each.
 gw_status dyson_search_begin(DysonPlan& d, const HostPlan& h, const double2* H, const double2* Sigx,
                              const double2* Sigc, cudaStream_t st);
-gw_status dyson_search_count(DysonPlan& d, const HostPlan& h, double mu, const double2* Tlast, double* n, bool* weak,
-                             cudaStream_t st);
+gw_status dyson_search_count(DysonPlan& d, const HostPlan& h, double mu, const double2* Tlast, const int* status,
+                             double* n, bool* weak, cudaStream_t st);
 
 // Linearised quasiparticle energies E [n_k][N] ascending (kernels_qp.cu): Sigma_c from
 // the sampled frequencies n = 0 and n = 1.  N <= kQpMaxN.

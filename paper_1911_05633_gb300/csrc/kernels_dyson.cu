@@ -141,14 +141,14 @@ __global__ void __launch_bounds__(32) k_trace_m1(const double2* __restrict__ H, 
 }
 
 // out[0] = (s / N_k) sum_k Re Tr[-G(k, beta-)] from the traces tr[k n_w + n] of G(k, i w_n)
-// (the sum that k_density_trace takes element by element), out[1] = *flag, which is
-// cleared.  One block: n_k n_w terms of a few FP64 operations.
+// (the sum that k_density_trace takes element by element), out[1] != 0 with *flag, which is
+// cleared, or *status.  One block: n_k n_w terms of a few FP64 operations.
 __global__ void __launch_bounds__(512) k_density_of_traces(const double2* __restrict__ tr,
                                                            const double2* __restrict__ m1,
                                                            const double* __restrict__ w,
                                                            const double2* __restrict__ Tlast, double beta, double mu,
                                                            int N, int n_w, int n_k, double spin, int* flag,
-                                                           double* __restrict__ out) {
+                                                           const int* status, double* __restrict__ out) {
   __shared__ double red[16];
   double acc = 0.0;
   for (int b = threadIdx.x; b < n_k * n_w; b += blockDim.x) {
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(512) k_density_of_traces(const double2* __rest
     double s = 0.0;
     for (int i = 0; i < 16; ++i) s += red[i];
     out[0] = -spin * s / n_k;
-    out[1] = (double)*flag;
+    out[1] = *flag || *status ? 1.0 : 0.0;
     *flag = 0;
   }
 }
@@ -285,13 +285,13 @@ gw_status dyson_search_begin(DysonPlan& d, const HostPlan& h, const double2* H, 
   return launch_ok("k_hessenberg");
 }
 
-gw_status dyson_search_count(DysonPlan& d, const HostPlan& h, double mu, const double2* Tlast, double* n, bool* weak,
-                             cudaStream_t st) {
+gw_status dyson_search_count(DysonPlan& d, const HostPlan& h, double mu, const double2* Tlast, const int* status,
+                             double* n, bool* weak, cudaStream_t st) {
   hess_trace(d.M, d.scale, mu, d.N, (long long)h.n_k * d.n_w, d.tr, reinterpret_cast<int*>(d.count + 2), st);
   {
     TimedLaunch tl_("k_density_of_traces", st);
     k_density_of_traces<<<1, 512, 0, st>>>(d.tr, d.m1, d.w, Tlast, h.beta, mu, d.N, d.n_w, d.n_k, h.spin,
-                                           reinterpret_cast<int*>(d.count + 2), d.count);
+                                           reinterpret_cast<int*>(d.count + 2), status, d.count);
   }
   gw_status s = launch_ok("k_hess_trace");
   if (s != GW_OK) return s;

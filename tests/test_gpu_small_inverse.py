@@ -96,3 +96,21 @@ def test_short_search_goes_without_the_forms():
     mu2, n2 = p.chemical_potential(dev(H), n, -1e-9, 1e-9, tol=1e-10, **a)
     assert "k_hessenberg" in p.timing_read()
     assert abs(n2 - n) < 1e-7 and abs(mu2) < 1e-9
+
+
+def test_failure_of_an_earlier_call_is_reported():
+    """A Dyson step with an exactly singular matrix leaves its status; the search that follows
+    reports it (as it does a zero pivot of its own), and the next one is clean."""
+    from paper_1911_05633_gb300 import gw
+    p, tau, om = _plan(1, 2)
+    w = (2 * om + 1) * np.pi / 20.0
+    S = np.zeros((2, len(om), 2, 2), np.complex128)
+    S[:] = (1j * w)[None, :, None, None] * np.eye(2)
+    p.dyson_green_tau(dev(np.zeros((2, 2, 2))), 0.0, Sig_k_iw=dev(S))
+    H, Sx, S = _inputs(2, len(om), 2, 9)
+    a = dict(Sigx_k=dev(Sx), Sig_k_iw=dev(S))
+    with pytest.raises(gw.GwError) as e:
+        p.chemical_potential(dev(H), 2.0, -4.0, 4.0, **a)
+    assert e.value.status == 6
+    p.chemical_potential(dev(H), 2.0, -4.0, 4.0, **a)
+    p.sync()
