@@ -30,8 +30,16 @@ __device__ __forceinline__ double2 herm_el(const double2* __restrict__ M, long l
 // Leading dimension in shared memory: odd, so that the words of a column fall on different banks.
 __host__ __device__ inline int qp_ld(int N) { return N | 1; }
 constexpr int kQT = 256;     // threads per block
-constexpr int kQPoints = 3;  // interior points per eigenvalue and section
-static_assert(kQpMaxN * kQPoints <= kQT, "one thread per section point");
+// Sections of an eigenvalue's interval per step, 2^bits: as many (up to 64) as four warps have
+// lanes for, four at least.  A step is a chain of N divisions, which four warps of an SM take in
+// the latency of one and eight do not: N = 2 46 us with four sections, 28 with 64; N = 16 327 with
+// four, 311 with 16; N = 32 709 with four, 757 with eight.
+__host__ __device__ constexpr int qp_bits(int N) {
+  int bits = 2;
+  while (bits < 6 && N * ((2 << bits) - 1) <= 128) ++bits;
+  return bits;
+}
+static_assert(kQpMaxN * ((1 << qp_bits(kQpMaxN)) - 1) <= kQT, "one thread per section point");
 
 // f(i, j) over the rows and columns r0 .. N - 1, flattened over the block (every lane busy:
 // the FP64 pipe issues two multiply-adds per clock and SM, so idle lanes are what costs).
@@ -50,8 +58,8 @@ __device__ __forceinline__ void each(int rows, int cols, F f) {
 // One block per momentum k.  The energies are the eigenvalues of X c = (E - mu) B c with
 // X = H^h + Sigma_x^h + S0^h - mu and B = I - S1^h, the same as those of A^{-1} X A^{-1},
 // A = B^{1/2}: B = L L^H by Cholesky, Z = L^{-1} X L^{-H}, Z to a real tridiagonal by
-// Householder reflections, its eigenvalues by sections on Sturm counts (all at once, three
-// interior points per eigenvalue and step).  About 13 N^3 FP64 operations per momentum; the
+// Householder reflections, its eigenvalues by sections on Sturm counts (all at once, one
+// thread per eigenvalue and interior point).  About 13 N^3 FP64 operations per momentum; the
 // cyclic Jacobi iterations this replaces took about 270 N^3: 2.96 ms for 64 momenta of N = 72, against 34.3.
 __global__ void __launch_bounds__(kQT) k_qp_energies(const double2* __restrict__ H, const double2* __restrict__ Sx,
                                                      const double2* __restrict__ Sc, int n_w, int i0, int i1,
@@ -68,7 +76,7 @@ __global__ void __launch_bounds__(kQT) k_qp_energies(const double2* __restrict__
   __shared__ double s_beta, s_lo, s_hi, s_min;
   __shared__ int s_on;
   __shared__ double lo[kQpMaxN], hi[kQpMaxN];
-  __shared__ unsigned char cnt[kQT];
+  __shared__ int above[kQpMaxN];  // first interior point with more than that many eigenvalues below it
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const long long k = blockIdx.x;
   const long long NN = (long long)N * N;
@@ -231,19 +239,22 @@ __global__ void __launch_bounds__(kQT) k_qp_energies(const double2* __restrict__
     }
   }
   __syncthreads();
-  const int ev = t / kQPoints, pt = t - ev * kQPoints;
+  const int bits = qp_bits(N), points = (1 << bits) - 1;
+  const double part = 1.0 / (1 << bits);
+  const int ev = t / points, pt = t - ev * points;
   if (pt == 0 && ev < N) {
     lo[ev] = s_lo;
     hi[ev] = s_hi;
+    above[ev] = points;
   }
   bool nan = false;
   for (int i = 0; i < N; ++i) nan = nan || !(fabs(d[i]) < 1e300) || !(e2[i] < 1e300);
   const double pmin = s_min;
   __syncthreads();
-  // 4^28 = 2^56 sections: below the last bit of the largest eigenvalue
-  for (int it = 0; it < 28; ++it) {
+  // 2^56 sections: below the last bit of the largest eigenvalue
+  for (int it = 0; it < 56; it += bits) {
     if (ev < N) {
-      const double x = lo[ev] + (hi[ev] - lo[ev]) * (0.25 * (pt + 1));
+      const double x = lo[ev] + (hi[ev] - lo[ev]) * (part * (pt + 1));
       int n = 0;  // eigenvalues below x: negative pivots of T - x
       double q = d[0] - x;
       if (fabs(q) < pmin) q = -pmin;
@@ -253,16 +264,16 @@ __global__ void __launch_bounds__(kQT) k_qp_energies(const double2* __restrict__
         if (fabs(q) < pmin) q = -pmin;
         n += q < 0.0;
       }
-      cnt[t] = (unsigned char)n;
+      if (n > ev) atomicMin(&above[ev], pt);
     }
     __syncthreads();
     if (ev < N && pt == 0) {
       // the section whose lower end has at most ev eigenvalues below it and whose upper end more
-      int s = 0;
-      while (s < kQPoints && cnt[t + s] <= ev) ++s;
+      const int s = above[ev];
       const double a = lo[ev], w = hi[ev] - lo[ev];
-      lo[ev] = s > 0 ? a + w * (0.25 * s) : a;
-      if (s < kQPoints) hi[ev] = a + w * (0.25 * (s + 1));
+      lo[ev] = s > 0 ? a + w * (part * s) : a;
+      if (s < points) hi[ev] = a + w * (part * (s + 1));
+      above[ev] = points;
     }
     __syncthreads();
   }
