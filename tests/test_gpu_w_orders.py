@@ -74,3 +74,14 @@ def test_every_pivot_off_the_diagonal(n_prod):
     ref = host(b.screened_W_iw(P, vq))
     b.sync()
     assert rel(W, ref) < TOL
+
+
+def test_route():
+    """The tensor-core inverse from order 88 on, while one frequency's matrices fit the caller's cap."""
+    for n_prod, kw, tensor in (((43, 44), {}, False), ((44, 44), {}, True), ((44, 44), {"workspace_bytes": 1 << 20}, False),
+                               ((128, 127), {}, True), ((128, 127), {"workspace_bytes": 8 << 20}, False)):
+        cell, a, b, P = _plans(n_prod, **kw)
+        a.timing_enable(True)
+        a.screened_W_iw(P, dev(cell.coulomb()[0]))
+        a.sync()
+        assert ("k_gj_inverse_f32" in a.timing_read()) == tensor, (n_prod, kw)
