@@ -38,7 +38,9 @@ constexpr uint32_t kLtStep = kOzDigits * kTfPlane;    // 32 KB: digits of 128 ro
 // 2^-5 at 32 points) and below 2^(e + 7), so that these keep it a normal double, and what the
 // digits drop of such a row, its subnormal values, is below 2^-62 of it.  Any other row that
 // is not all zero (G(tau) far from both ends at low temperature; a NaN or an infinity, which
-// the digits would lose) is summed in FP64.
+// the digits would lose) is summed in FP64 once its block's tiles are done: taken within the
+// read-out, or told from zero rows by the slicers, such rows cost transforms without any 1.4 %
+// in the middle and up to 6 % (launches of 20 to 45 us).
 constexpr int kLtLow = 64, kLtHigh = 2032;
 constexpr int kLtDirect = 1 << 20;                    // in place of such a row's scale exponent
 
@@ -54,12 +56,43 @@ struct LatArgs {
   const long long* B_off;  // [n_active] offset of a pair's operand (uint16 units)
   const int* eB;           // [n_active][64]
   const double2* phase;    // [E][n_k] e^{+i k.R}
+  double scale;            // 1 / N_k
   int tiles_per_block;
   int* status;
 };
 
 // Columns of a pair's operand, padded to the MMA's multiple of 16.
 __host__ __device__ inline int lat_nt(int cols) { return (cols + 15) & ~15; }
+
+// A pair's classes in shared memory, its first entry and the sizes of its transform.
+struct LatPair {
+  const long long* off;
+  const int* re;
+  const int* ce;
+  int e0, n_in, n_out;
+};
+
+// Outputs m0 .. m0 + 7 of one row as k_gather_k_to_R and k_scatter_R_to_k take them.
+template <bool SCATTER>
+__device__ __forceinline__ void lat_direct(const LatArgs& g, const LatPair p, long long el, int s, int i, int j, int m0) {
+#pragma unroll 1
+  for (int m = m0; m < min(m0 + 8, p.n_out); ++m) {
+    if (!SCATTER && !(i < p.re[m] && j < p.ce[m])) continue;
+    double2 a = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int q = 0; q < p.n_in; ++q) {
+      if (SCATTER && !(i < p.re[q] && j < p.ce[q])) continue;
+      const double2 v = SCATTER ? g.entries[p.off[q] + (long long)s * p.re[q] * p.ce[q] + i * p.ce[q] + j]
+                                : g.dense[q * g.k_stride + el];
+      const double2 f = g.phase[(long long)(p.e0 + (SCATTER ? q : m)) * g.n_k + (SCATTER ? m : q)];
+      const double fy = SCATTER ? f.y : -f.y;
+      a = make_double2(fma(f.x, v.x, fma(-fy, v.y, a.x)), fma(f.x, v.y, fma(fy, v.x, a.y)));
+    }
+    if (SCATTER) g.dense[m * g.k_stride + el] = a;
+    else g.entries[p.off[m] + (long long)s * p.re[m] * p.ce[m] + i * p.ce[m] + j] =
+             make_double2(a.x * g.scale, a.y * g.scale);
+  }
+}
 
 // Block (pair, chunk of its row tiles).  Slicer warps hold their row's values (all loads in
 // flight at once), take the row's scale and cut them; the epilogue reads the level sums as
@@ -125,6 +158,13 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
   auto dense_at = [&](int s, int i, int j) {
     return (long long)s * g.s_stride + (long long)(ro + i) * g.ld + co + j;
   };
+  // value m (mesh point or class) of a row
+  auto value = [&](int m, int s, int i, int j) {
+    if (!SCATTER) return __ldg(g.dense + m * g.k_stride + dense_at(s, i, j));
+    if (i < re_s[m] && j < ce_s[m])
+      return __ldg(g.entries + off_s[m] + (long long)s * re_s[m] * ce_s[m] + i * ce_s[m] + j);
+    return make_double2(0.0, 0.0);
+  };
   bool ok = true;
   if (warp < kLtWarps) {
     const int r = 16 * warp + (lane & 15), h = lane >> 4;
@@ -142,14 +182,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
         for (int q = 0; q < 4; ++q) {
           const int m = ks * 8 + 4 * h + q;  // mesh point or class
           double2 v = make_double2(0.0, 0.0);
-          if (valid && m < n_in) {
-            if (SCATTER) {
-              if (i < re_s[m] && j < ce_s[m])
-                v = __ldg(g.entries + off_s[m] + (long long)s * re_s[m] * ce_s[m] + i * ce_s[m] + j);
-            } else {
-              v = __ldg(g.dense + m * g.k_stride + dense_at(s, i, j));
-            }
-          }
+          if (valid && m < n_in) v = value(m, s, i, j);
           w[ks][2 * q] = v.x;
           w[ks][2 * q + 1] = v.y;
         }
@@ -159,20 +192,10 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
         for (int u = 0; u < 8; ++u) mx = max(mx, exp_field(w[ks][u]));
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
       const int e = mx > 0 ? mx - 1022 : 0;
-      bool direct = mx > kLtHigh;
-      if (__any_sync(0xffffffffu, mx < kLtLow)) {
-        unsigned long long any = 0;
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-          for (int u = 0; u < 8; ++u) any |= (unsigned long long)__double_as_longlong(w[ks][u]) << 1;
-        const unsigned with = __ballot_sync(0xffffffffu, any != 0);  // lanes r and r + 16 hold a row's halves
-        if (mx < kLtLow && ((with >> (lane & 15)) & 0x10001u)) direct = true;
-      }
       const int it = t - t0, b = it & 1;
       ok = mbar_wait(&e_empty[b], (uint32_t)((it >> 1) & 1) ^ 1u, kLtWaitNs, g.status);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      if (h == 0) eA_s[b][r] = direct ? kLtDirect : e;
+      if (h == 0) eA_s[b][r] = mx < kLtLow || mx > kLtHigh ? kLtDirect : e;
       mbar_arrive(&e_full[b]);
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
@@ -227,6 +250,10 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
   } else {
     const int q = warp & 3, half = (warp - kLtWarps - 1) >> 2;
     const int row = 32 * q + lane, n_chunks = NT / 16;
+    unsigned long long left = 0;  // tiles (modulo 64) where this thread's row was not for the digits
+    // rows beyond every class's block are zero
+    const int r_max = SCATTER ? __reduce_max_sync(0xffffffffu, lane < n_cls ? re_s[lane] : 0) : ra;
+    const int c_max = SCATTER ? __reduce_max_sync(0xffffffffu, lane < n_cls ? ce_s[lane] : 0) : cb;
     for (int t = t0; t < t1 && ok; ++t) {
       const int it = t - t0, b = it & 1, bf = n_buf == 2 ? it & 1 : 0, use = n_buf == 2 ? it >> 1 : it;
       const long long x = (long long)t * 128 + row;
@@ -236,6 +263,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
       ok = mbar_wait(&e_full[b], (uint32_t)((it >> 1) & 1), kLtWaitNs, g.status);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       const int ea = eA_s[b][row];
+      if (ea == kLtDirect && valid && i < r_max && j < c_max) left |= 1ull << (it & 63);
       mbar_arrive(&e_empty[b]);
       ok = mbar_wait(&t_full[bf], (uint32_t)(use & 1), kLtWaitNs, g.status);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
@@ -268,24 +296,6 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
           mbar_arrive(&t_empty[bf]);
         }
         if (!valid) continue;
-        if (ea == kLtDirect) {
-          for (int m = 8 * c; m < min(8 * c + 8, n_out); ++m) {
-            if (!SCATTER && !(i < re_s[m] && j < ce_s[m])) continue;
-            double2 a = make_double2(0.0, 0.0);
-            for (int q2 = 0; q2 < n_in; ++q2) {
-              if (SCATTER && !(i < re_s[q2] && j < ce_s[q2])) continue;
-              const double2 v = SCATTER ? g.entries[off_s[q2] + (long long)s * re_s[q2] * ce_s[q2] + i * ce_s[q2] + j]
-                                        : g.dense[q2 * g.k_stride + dense_at(s, i, j)];
-              const double2 p = g.phase[(long long)(e0 + (SCATTER ? q2 : m)) * g.n_k + (SCATTER ? m : q2)];
-              const double py = SCATTER ? p.y : -p.y;
-              a = make_double2(fma(p.x, v.x, fma(-py, v.y, a.x)), fma(p.x, v.y, fma(py, v.x, a.y)));
-            }
-            if (SCATTER) g.dense[m * g.k_stride + dense_at(s, i, j)] = a;
-            else g.entries[off_s[m] + (long long)s * re_s[m] * ce_s[m] + i * ce_s[m] + j] =
-                     make_double2(a.x * (1.0 / g.n_k), a.y * (1.0 / g.n_k));
-          }
-          continue;
-        }
 #pragma unroll
         for (int k = 0; k < 16; k += 2) {
           const int n = 16 * c + k, m = n >> 1;
@@ -298,6 +308,24 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lattice_tc(const __grid_const
       }
     }
     if (!ok) atomicExch(g.status, 2);
+    // what the digits could not hold, over what was written for it (zeros: right already)
+    for (int t = t0; left && ok && t < t1; ++t) {
+      const long long x = (long long)t * 128 + row;
+      if (x >= rows) break;
+      if (!((left >> ((t - t0) & 63)) & 1ull)) continue;
+      const int s = (int)(x / blk), ij = (int)(x - (long long)s * blk), i = ij / cb, j = ij - i * cb;
+      unsigned long long any = 0;
+      int mx = 0;
+#pragma unroll 1
+      for (int m = 0; m < n_in; ++m) {
+        const double2 v = value(m, s, i, j);
+        mx = max(mx, max(exp_field(v.x), exp_field(v.y)));
+        any |= (unsigned long long)(__double_as_longlong(v.x) | __double_as_longlong(v.y)) << 1;
+      }
+      if (any == 0 || (mx >= kLtLow && mx <= kLtHigh)) continue;
+      for (int c = half; c < n_chunks; c += 2)
+        lat_direct<SCATTER>(g, LatPair{off_s, re_s, ce_s, e0, n_in, n_out}, dense_at(s, i, j), s, i, j, 8 * c);
+    }
   }
   fence_before_sync();
   __syncthreads();
@@ -480,6 +508,7 @@ gw_status lattice_run(const LatticePlan& l, const HostPlan& h, const DevEntry* d
   a.B_off = l.d_off[to_k];
   a.eB = l.d_e[to_k];
   a.phase = d_phase;
+  a.scale = 1.0 / h.n_k;
   a.status = d_status;
   // about six blocks per SM over the whole launch, at least four tiles each
   const long long want = std::max<long long>(1, 6LL * l.n_sm / l.n_active);
