@@ -74,6 +74,7 @@ struct TfArgs {
   int NT;              // columns per tile and accumulator (multiple of 16)
   const uint16_t* Bdig;  // per column tile [KS][kOzDigits][NT x 16] in the K-major layout
   const int* eB;         // [n_ct NT] column scale exponents
+  int eB_min, eB_max;
   int* status;
 };
 
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_oz_transform(const __grid_con
     }
     for (int i = 0; i < my_tiles && ok; ++i) {
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-      const int e = mx > 0 ? mx - 1022 : 0;
+      const int e = tf_row_scale(mx);
       Row Rn = R;
       Rn.valid = false;
       if (i + 1 < my_tiles) Rn = row_of(i + 1);
@@ -359,6 +360,8 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_oz_transform(const __grid_con
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       fence_after_sync();
       double2* dst = g.out + base * g.n_out + x;
+      // every result of the warp a normal number (|S| < 2^62)?
+      const bool normal = __all_sync(0xffffffffu, ea + g.eB_min - 52 >= -1022 && ea + g.eB_max + 12 <= 1023);
       if (!STAGE && half >= n_chunks) {  // no chunk for this warp: release at once
         fence_before_sync();
         mbar_arrive(&t_empty);
@@ -404,27 +407,31 @@ __global__ void __launch_bounds__(kTfThreads, 1) k_oz_transform(const __grid_con
         }
         if (!valid) continue;
         const int n0 = ct * NT + 16 * c;  // first column of this chunk
-        if (g.out_mode != kTfOutReal) {
-          // columns 2m + c: component c of output slice m
+        auto store = [&](auto value) {
+          if (g.out_mode != kTfOutReal) {
+            // columns 2m + c: component c of output slice m
 #pragma unroll
-          for (int j = 0; j < 16; j += 2) {
-            const int n = n0 + j;
-            if (n >= g.n_cols) break;
-            const int m = n >> 1;
-            const double re = tf_i2d(S[j], ea + eB_s[n] - 52);
-            const double im = tf_i2d(S[j + 1], ea + eB_s[n + 1] - 52);
-            dst[(long long)m * blk] = make_double2(re, im);
-            if (g.out_mode == kTfOutMirror && g.n_out - 1 - m != m)
-              dst[(long long)(g.n_out - 1 - m) * blk] = make_double2(re, dneg(im));
-          }
-        } else {
+            for (int j = 0; j < 16; j += 2) {
+              const int n = n0 + j;
+              if (n >= g.n_cols) break;
+              const int m = n >> 1;
+              const double re = value(S[j], ea + eB_s[n] - 52);
+              const double im = value(S[j + 1], ea + eB_s[n + 1] - 52);
+              dst[(long long)m * blk] = make_double2(re, im);
+              if (g.out_mode == kTfOutMirror && g.n_out - 1 - m != m)
+                dst[(long long)(g.n_out - 1 - m) * blk] = make_double2(re, dneg(im));
+            }
+          } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int n = n0 + j;
-            if (n >= g.n_cols) break;
-            dst[(long long)(g.out_slice0 + n) * blk] = make_double2(tf_i2d(S[j], ea + eB_s[n] - 52), 0.0);
+            for (int j = 0; j < 16; ++j) {
+              const int n = n0 + j;
+              if (n >= g.n_cols) break;
+              dst[(long long)(g.out_slice0 + n) * blk] = make_double2(value(S[j], ea + eB_s[n] - 52), 0.0);
+            }
           }
-        }
+        };
+        if (normal) store([](long long s, int e) { return tf_i2d(s, e); });
+        else store([](long long s, int e) { return tf_i2d_any(s, e); });
       }
     }
     if (!ok) atomicExch(g.status, 2);
@@ -456,6 +463,8 @@ void tf_matrix(OzFused& f, int n_cols, int K, int NT, F value, std::vector<uint1
     for (int k = 0; k < K; ++k) mx = std::max(mx, host_exp_field(value(n, k)));
     const int e = mx > 0 ? mx - 1022 : 0;
     ex[n] = e;
+    f.e_min = std::min(f.e_min, e);
+    f.e_max = std::max(f.e_max, e);
     const int ct = n / NT, nl = n % NT;
     for (int k = 0; k < K; ++k) {
       uint16_t d[kOzDigits];
@@ -637,6 +646,8 @@ static gw_status tf_run(OzTransform& o, const OzFused& f, const DevEntry* d_ent,
   a.NT = f.NT;
   a.Bdig = f.d_B;
   a.eB = f.d_e;
+  a.eB_min = f.e_min;
+  a.eB_max = f.e_max;
   a.status = d_status;
   const int n_tiles = a.n_rt * a.n_ct;
   const unsigned grid = (unsigned)std::max(1, std::min(n_tiles, o.n_sm));

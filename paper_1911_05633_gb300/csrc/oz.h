@@ -70,6 +70,7 @@ struct OzFused {
   bool stage = false;       // the epilogue stages its sums in shared memory (KS <= 5)
   uint16_t* d_B = nullptr;  // per column tile [KS][kOzDigits][NT x 16]
   int* d_e = nullptr;       // [n_ct NT]
+  int e_min = 0, e_max = 0;  // of them
   size_t smem = 0;          // dynamic shared memory of the kernel
 };
 
