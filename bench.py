@@ -181,7 +181,7 @@ def kernel_work(name: str, cell, info, entries, kdims, chain=False):
     n_inv = nq * (nnu + 1)  # v(q) once, then every solved (q, nu)
     gj = 8.0 * N ** 3 * n_inv  # complex Gauss-Jordan inverse, or one complex N^3 product
     nt, nn, nw = info["n_tau"], info["n_nu"], info["n_omega"]
-    if name in ("k_gj_inverse_blocked", "k_gj_inverse"):
+    if name in ("k_gj_inverse_smem", "k_gj_inverse_blocked", "k_gj_inverse"):
         return "alu", gj, "fp64", n_inv
     if name == "k_gj_inverse_f32":
         return "alu", gj, "fp32", n_inv
@@ -191,8 +191,8 @@ def kernel_work(name: str, cell, info, entries, kdims, chain=False):
         return "tensor", 4 * 20 * 2.0 * N ** 3 * n_inv, "bf16", n_inv
     if name == "k_ozaki_residual<second>":  # 36 slice pairs
         return "tensor", 4 * 36 * 2.0 * N ** 3 * n_inv, "bf16", n_inv
-    if chain and name in ("k_polarizability_fp64", "k_self_energy_fp64"):
-        slices = (nt + 1) // 2 if name == "k_polarizability_fp64" else nt + 1  # Sigma: and the exchange's one
+    if name == "k_sigma_pairs" or (chain and name == "k_polarizability_fp64"):  # (k_polarizability_pairs goes by that name)
+        slices = nt + 1 if name == "k_sigma_pairs" else (nt + 1) // 2  # Sigma: and the exchange's one
         pairs = sum((cell.n_orb_of(int(a)) * cell.n_orb_of(int(b))) ** 2 for a, b in entries[:, :2])
         return "alu", 8.0 * pairs * slices, "fp64", len(entries)
     if name == "k_polarizability_fp64":  # stages 1 and 2 only when stage 3 runs on the tensor cores
@@ -511,7 +511,7 @@ CONTRACTION_KERNELS = {
     "k_polarizability_tc": ("P", True), "k_polarizability_f32": ("P", True),
     "k_self_energy_tc": ("S", True), "k_self_energy_f32": ("S", True),
     "k_contract_p_tc": ("P", True), "k_contract_s_tc": ("S", True),
-    "k_polarizability_fp64": ("P", False), "k_self_energy_fp64": ("S", False),
+    "k_polarizability_fp64": ("P", False), "k_self_energy_fp64": ("S", False), "k_sigma_pairs": ("S", False),
 }
 
 

@@ -115,9 +115,11 @@ typedef struct {
                              larger multiple of 128),
                              1: FP64 Gauss-Jordan inverse always */
   int fp64_products;      /* 0 automatic: FP64-accurate digit products on the tensor cores for
-                             the W~ C^b stage of the GW_FP64 Sigma (every K <= 384), the Y C^b
-                             stage of the GW_FP64 P (every n^2 <= 384) and the structured
-                             bosonic transforms (reduction <= 384);
+                             both products of the GW_FP64 P and Sigma with C (C symmetric, n <= 10,
+                             K <= 64) or else the W~ C^b stage of Sigma (every K <= 384) and the
+                             Y C^b stage of P (every n^2 <= 384), the structured bosonic
+                             transforms (reduction <= 384) and the lattice transforms of meshes
+                             with other than quarter-turn phases (N_k <= 32);
                              1: FP64 arithmetic only */
   double r_b;             /* radius of sphere B in bohr (Sec. 2, Fig. 2): an entry whose
                              minimum-image distance |R + t_b - t_a| exceeds r_b by more than
@@ -146,9 +148,10 @@ typedef struct {
   double cond_boson;
   int w_symmetric;            /* the W solve runs on nu >= 0 and half of the q mesh (see gw_screened_W_iw) */
   int n_q_solved;             /* momenta solved per frequency */
-  int w_tensor;               /* inverses of order N_PB by FP32 Gauss-Jordan + two tensor-core refinements */
-  int sigma_tensor;           /* GW_FP64 Sigma: stage W~ C^b by FP64-accurate tensor-core products */
-  int p_tensor;               /* GW_FP64 P: stage Y C^b by FP64-accurate tensor-core products (device plans) */
+  int w_tensor;               /* inverses of order N_PB by FP32 Gauss-Jordan + two tensor-core refinements
+                                 (0 for the orders that are solved beside an identity, see w_solver) */
+  int sigma_tensor;           /* GW_FP64 Sigma: products with C by FP64-accurate tensor-core products */
+  int p_tensor;               /* GW_FP64 P: products with C by FP64-accurate tensor-core products (device plans) */
   int transform_tensor;       /* bit 0: GW_IN_REAL bosonic i nu -> tau, bit 1: GW_IN_MIRROR bosonic
                                  tau -> i nu of the product-basis layout by FP64-accurate
                                  tensor-core products (device plans) */

@@ -675,7 +675,8 @@ gw_status chain_polarizability(ChainPlan& c, const HostPlan& h, const DevEntry* 
   for (int s0 = 0; s0 < nodes; s0 += c.tau_p) {
     const int te = std::min(c.tau_p, nodes - s0);
     {
-      TimedLaunch tl_("k_polarizability_fp64", st);  // the FP64 stage of P, as on the other path
+      // the name of the row's FP64 stage on the other path, which is what timings of the row look for
+      TimedLaunch tl_("k_polarizability_fp64", st);
       k_polarizability_pairs<<<dim3(h.n_entries(), te), 256, pairs_smem(max_n), st>>>(
           d_ent, c.d_species, c.d_pair, G, h.n_tau, s0, c.kp.KS, c.d_AP, c.d_eP);
     }
@@ -728,7 +729,7 @@ gw_status chain_self_energy(ChainPlan& c, const HostPlan& h, const DevEntry* d_e
     a.status = d_status;
     chain_launch<true>(c.pk, a, c.n_sm, st);
     {
-      TimedLaunch tl_("k_self_energy_fp64", st);  // the FP64 stage of Sigma, as on the other path
+      TimedLaunch tl_("k_sigma_pairs", st);
       k_sigma_pairs<<<dim3(h.n_entries(), te), 256, sigma_smem(c.max_pairs), st>>>(
           d_ent, c.d_species, c.d_pidx, c.d_D, c.max_pairs, G, h.n_tau, g_fixed, s0, sign, Sig, n_slices);
     }

@@ -1,6 +1,7 @@
 // W solve on the tensor cores (Eq. W_1): each inverse (v(q)^-1, then (v^-1 - P)^-1) is
-// computed in FP32 by Gauss-Jordan and refined twice, X <- X + X (I - A X), with the
-// residual I - A X evaluated to FP64 accuracy on tcgen05 from exact BF16 slices of A
+// computed in FP32 by Gauss-Jordan and refined, X <- X + X (I - A X) (twice, or four times
+// beside an identity and for the pivots of the block inverse), with the residual I - A X
+// evaluated to FP64 accuracy on tcgen05 from exact BF16 slices of A
 // and X (an Ozaki-type splitting): after a power-of-two scaling per row of A and per
 // column of X, every entry is a sum of slices a_s = alpha_s 2^-7(s+1), |alpha_s| <= 128,
 // each exact in BF16 (k_oz_product below).  Two refinements take the FP32 inverse (error
@@ -446,8 +447,11 @@ __global__ void k_slice_X(const float2* __restrict__ hi, const float2* __restric
 // at two thirds of it: their operand reads bound them).
 //
 // Exactness: the level sums over at most 512 real terms are integers in their unit
-// 2^-7(L+2) below 2^24 for L <= 5, exact in FP32 whatever rounding the tensor core applies;
-// levels 6 and 7 round far below 2^-52 of the scale.  A longer reduction (N = 384: 768 terms)
+// 2^-7(L+2) up to 2^24 for L <= 5, exact in FP32 whatever rounding the tensor core applies;
+// of eight levels 6 and 7 round far below 2^-52 of the scale.  With nine digits the sum has
+// units of 2^-59: level 6 (unit 2^-56) passes 2^24 only if almost all of its 512 x 7 products
+// have their largest size and one sign (18.9 M at worst), and then loses a unit; levels 7 and 8
+// (2^-63 and 2^-70) are rounded together.  A longer reduction (N = 384: 768 terms)
 // is taken in two halves: the accumulators are read out as exact 64-bit sums in units of
 // 2^-52 in between.  The sum of all levels is rounded once.
 constexpr int kPT = 512;          // threads: 4 warps per tensor-memory lane quadrant, 16 columns each

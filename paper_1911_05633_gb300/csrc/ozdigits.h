@@ -159,9 +159,6 @@ __device__ __forceinline__ int tf_level_int(float v, float sc) {
   return 4 * (__float_as_int(y) - 0x4C400000) + (__float_as_int((x - (y - 50331648.0f)) + 12582912.0f) - 0x4B400000);
 }
 
-// Adds the single levels l and l + 1 (two accumulators read together) to the 64-bit sums:
-// I_l 2^7 + I_{l+1} is a 32-bit integer, shifted once into units of 2^-52 (levels 6 and 7:
-// rounded, half up, at 2^-52).
 // I_l 2^7 + I_{l+1} of two single levels; the two offsets of the reads go out in one subtraction.
 template <bool WIDE>
 __device__ __forceinline__ int tf_pair_int(float v0, float s0, float v1, float s1) {
@@ -170,6 +167,9 @@ __device__ __forceinline__ int tf_pair_int(float v0, float s0, float v1, float s
                (__float_as_uint(fmaf(v1, s1, 12582912.0f)) - 129u * 0x4B400000u));
 }
 
+// Adds the single levels l and l + 1 (two accumulators read together) to the 64-bit sums:
+// I_l 2^7 + I_{l+1} is a 32-bit integer, shifted once into units of 2^-52 (levels 6 and 7:
+// rounded, half up, at 2^-52).
 template <bool WIDE>
 __device__ __forceinline__ void tf_add_pair(long long* S, const float* v, int l) {
   const float s0 = __int_as_float((127 + 7 * l) << 23), s1 = __int_as_float((127 + 7 * (l + 1)) << 23);

@@ -100,7 +100,8 @@ def test_values_near_the_ends_of_the_range():
         for n, got, ref in ((nt, S, S2), (1, X, X2)):
             _agree(a, "orb", n, host(got), host(ref), 4 * c ** 2 * np.abs(G1).max() * 2.0 ** -1022)
     a.sync()
-    assert "k_chain" in a.timing_read()
+    t = a.timing_read()
+    assert {"k_chain", "k_slice_w_units", "k_sigma_pairs"} <= set(t) and "k_self_energy_fp64" not in t
 
 
 def test_nan_and_infinities_pass_through():
