@@ -112,8 +112,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t saddr, uint32_t parity) {
 }
 
 // Wait for the mbarrier phase with the given parity.  Gives up and returns false
-// after `timeout_ns` of wall time, or as soon as *abort is non-zero (another block
-// already gave up), so that a failure costs one timeout, not one per block.
+// after `timeout_ns` of wall time, or as soon as *abort is 2 (another block already gave
+// up), so that a failure costs one timeout, not one per block.  Other values of the status
+// (1: a zero pivot, of this call or of one before it) are no reason to leave work undone.
 __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint64_t timeout_ns,
                                           const volatile int* abort) {
   const uint32_t a = smem_u32(mbar);
@@ -121,7 +122,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint6
   const uint64_t t0 = global_ns();
   for (;;) {
     if (mbar_try_wait(a, parity)) return true;
-    if (abort && *abort) return false;
+    if (abort && *abort == 2) return false;
     if (global_ns() - t0 > timeout_ns) return false;
   }
 }

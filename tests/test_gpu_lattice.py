@@ -154,3 +154,27 @@ def test_few_classes_on_a_small_mesh_stay_with_the_fp64_kernels():
         p.fourier_R_to_k("pb", ns, p.fourier_k_to_R("pb", ns, F))
         p.sync()
         assert set(p.timing_read()) == want
+
+
+def test_status_of_an_earlier_call_stops_nothing():
+    """A Dyson step with a singular matrix leaves its status for the next synchronisation; the
+    transforms launched before that do their work."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1911_05633_gb300 import gw
+    cell = synth.mixed_species_cell(n_tau=9, n_orb=(4, 5), n_prod=(30, 35), kmesh=(3, 3, 3))
+    a, b = gw.Plan.from_cell(cell), gw.Plan.from_cell(cell, fp64_products="fp64")
+    N, w = a.dense_n("orb"), (2 * cell.omega_idx + 1) * np.pi / cell.beta
+    S = np.zeros((cell.n_k, len(w), N, N), np.complex128)
+    S[:] = (1j * w)[None, :, None, None] * np.eye(N)  # i w - Sigma = 0
+    a.dyson_green_tau(dev(np.zeros((cell.n_k, N, N))), 0.0, Sig_k_iw=dev(S))
+    rng = np.random.default_rng(13)
+    F = dev(rng.standard_normal(cell.n_k * 3 * a.dense_n("pb") ** 2))
+    a.timing_enable(True)
+    got = host(a.fourier_k_to_R("pb", 3, F))
+    assert "k_lattice_tc" in a.timing_read()
+    assert rel(got, host(b.fourier_k_to_R("pb", 3, F))) < 2e-14
+    with pytest.raises(gw.GwError) as e:
+        a.sync()
+    assert e.value.status == 6

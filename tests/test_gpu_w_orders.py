@@ -85,3 +85,24 @@ def test_route():
         a.screened_W_iw(P, dev(cell.coulomb()[0]))
         a.sync()
         assert ("k_gj_inverse_f32" in a.timing_read()) == tensor, (n_prod, kw)
+
+
+@pytest.mark.parametrize("n_prod", [(43, 44), (44, 44), (100, 101), (128, 128)])
+def test_singular_v_is_reported_as_such(n_prod):
+    """A v(q) with a zero row: status 6, as by the FP64 elimination, not a wait that gave up; and
+    the plan works again after it."""
+    from paper_1911_05633_gb300 import gw
+    cell, a, b, P = _plans(n_prod)
+    N = cell.n_pb_total
+    v = cell.coulomb()[0].reshape(cell.n_k, N, N).copy()
+    ref = host(b.screened_W_iw(P, dev(v)))
+    bad = v.copy()
+    bad[1, 7] = bad[1, :, 7] = 0.0
+    for p in (a, b):
+        p.screened_W_iw(P, dev(bad))
+        with pytest.raises(gw.GwError) as e:
+            p.sync()
+        assert e.value.status == 6
+    W = host(a.screened_W_iw(P, dev(v)))
+    a.sync()
+    assert rel(W, ref) < TOL
