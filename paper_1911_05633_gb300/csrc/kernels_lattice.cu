@@ -10,7 +10,7 @@
 // 27 points and 5.4 kept classes per pair take 290 clocks per element and SM.  Cutting the 54
 // values into digits and reading the sums back is integer and FP32 work of about a tenth of
 // that, and the products are free beside it.
-// G, v and Sigma of the 16-atom cell on a 3x3x3 mesh (1392 entries, 48 slices): 0.99 ms in
+// G, v and Sigma of the 16-atom cell on a 3x3x3 mesh (1392 entries, 48 slices): 0.98 ms in
 // three launches, 4.64 ms by k_gather_k_to_R and k_scatter_R_to_k.
 #include <cuda_runtime.h>
 

@@ -33,7 +33,7 @@ constexpr int kQT = 256;     // threads per block
 // Sections of an eigenvalue's interval per step, 2^bits: as many (up to 64) as four warps have
 // lanes for, four at least.  A step is a chain of N divisions, which four warps of an SM take in
 // the latency of one and eight do not: N = 2 46 us with four sections, 28 with 64; N = 16 327 with
-// four, 311 with 16; N = 32 709 with four, 757 with eight.
+// four, 266 with eight, 311 with 16; N = 32 709 with four, 757 with eight.
 __host__ __device__ constexpr int qp_bits(int N) {
   int bits = 2;
   while (bits < 6 && N * ((2 << bits) - 1) <= 128) ++bits;
